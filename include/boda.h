@@ -91,7 +91,9 @@ typedef struct boda_plan_opts {
     int tile_id;                 /* -1: automatic; otherwise index into the variant's tile table (boda_conv_plan_describe
                                     prints the name).  BODA_VARIANT_DIRECT: 0..8 GEMM-blocked FP32 tiles direct_128x128 ..
                                     direct_32x16, 9..11 pixel-per-thread direct_pixel_k8/16/32, 12..15 the same compiled
-                                    at run time for the exact shape direct_rtc_k4/8/16/32.  K1CONV / TCONV (pixels x
+                                    at run time for the exact shape direct_rtc_k4/8/16/32, 16..17 direct_64x48 and
+                                    direct_128x48, 18..22 direct_nhwc_128x128/96/64/48/32 (over a staged NHWC copy of
+                                    the input: needs workspace).  K1CONV / TCONV (pixels x
                                     channels): 0..4 igemm_128x64/96/128/192/256 (TMA im2col tiles, cluster split),
                                     5..15 halo_128/256/512xBN (TCONV stride 1 or space-to-depth view: shared-memory
                                     reuse of the input across taps), 16..19 gconv_128x64/96/128/192 (input gathered
@@ -101,7 +103,8 @@ typedef struct boda_plan_opts {
                                     padding, windows up to 11x11: the space-to-depth view built in shared memory
                                     straight from NCHW, nothing staged).  A tile that cannot run the shape is refused
                                     with BODA_ERR_UNSUPPORTED. */
-    int split_k;                 /* 0: automatic; otherwise the number of reduction splits of a tensor-core variant */
+    int split_k;                 /* 0: automatic; otherwise the number of reduction splits (tensor-core variants and the GEMM-blocked
+                                    FP32 tiles) */
     int device;                  /* CUDA device ordinal; -1: the current device */
     int s2d;                     /* strided TCONV layers: -1 automatic, 0 never, 1 always run the stride-1
                                     "space-to-depth" view (stride t on C channels = stride 1 on C*t*t channels
@@ -148,9 +151,9 @@ int boda_conv_plan_describe(const boda_conv_plan* plan, char* buf, size_t buf_by
  * the re-laid-out input (the "input transformation" that the paper's k1conv and tconv apply, Section 5). */
 size_t boda_conv_plan_workspace_bytes(const boda_conv_plan* plan);
 
-/* Kernels one boda_conv_fwd_planned call launches when the filters are bound: 1 for DIRECT and for the tensor-core
- * kernels that read NCHW themselves (gather, NCHW 1x1, first-layer kernel), 2 for the others (input staging and the
- * main kernel). */
+/* Kernels one boda_conv_fwd_planned call launches when the filters are bound: 1 for the kernels that read NCHW themselves
+ * (DIRECT tiles 0..17, gather, NCHW 1x1, first-layer kernel), 2 for the others (input staging and the main kernel); DIRECT
+ * tiles 18..22 add a third where the sums of tiles cut between CTAs are put together. */
 int boda_conv_plan_kernels_per_call(const boda_conv_plan* plan);
 
 /*

@@ -12,6 +12,7 @@
 
 #include "boda_internal.h"
 #include "igemm_tf32.h"
+#include "simt_conv.h"
 
 namespace boda {
 
@@ -141,6 +142,8 @@ struct boda_conv_plan {
     int* d_status = nullptr;
     DirectTapEntry* d_tab = nullptr;     // DIRECT
     DirectRtc* rtc = nullptr;            // DIRECT, tiles compiled at run time
+    int split = 1;                       // DIRECT, GEMM-blocked tiles: CTAs of a cluster that share a tile's reduction
+    SimtPlan* simt = nullptr;            // DIRECT, tiles over a staged input
     IgemmPlan* ig = nullptr;             // K1CONV / TCONV
     size_t ws_bytes = 0;
     bool in_packed = false;              // chained layers: the input arrives in the staged layout
@@ -154,9 +157,10 @@ int conv_fwd_planned_ex(boda_conv_plan* p, const float* in, const float* filt, c
     if (!p || !in || !out) return BODA_ERR_INVALID_ARG;
     if (p->variant == BODA_VARIANT_DIRECT) {
         if (!filt) return BODA_ERR_INVALID_ARG;
+        if (p->simt) return simt_launch(p->simt, in, filt, bias, out, workspace, stream, after_staging);
         if (after_staging) BODA_CUDA_TRY(cudaEventRecord(after_staging, stream));
         if (p->rtc) return direct_rtc_launch(p->rtc, in, filt, bias, out, stream);
-        return direct_launch(p->d, p->tile_id, in, filt, bias, out, p->d_tab, stream);
+        return direct_launch(p->d, p->tile_id, p->split, in, filt, bias, out, p->d_tab, stream);
     }
     if (p->ws_bytes && !workspace && !p->in_packed) return BODA_ERR_NOMEM;
     return igemm_launch(p->ig, in, filt, bias, out, workspace, stream, after_staging);
@@ -226,6 +230,7 @@ int boda_conv_plan_destroy(boda_conv_plan* plan)
     (void)cudaSetDevice(plan->device);
     if (plan->d_tab) (void)cudaFree(plan->d_tab);
     if (plan->rtc) direct_rtc_destroy(plan->rtc);
+    if (plan->simt) simt_plan_destroy(plan->simt);
     if (plan->ig) igemm_plan_destroy(plan->ig);
     (void)cudaSetDevice(prev);
     delete plan;
@@ -248,7 +253,7 @@ static int plan_build(const boda_conv_shape& shape, const boda_plan_opts& o, Dev
     if (variant == BODA_VARIANT_DIRECT) {
         p->math = BODA_MATH_FP32;
         if (tile_id >= direct_num_tiles() || (tile_id >= 0 && !direct_tile_legal(p->d, tile_id))) { delete p; return BODA_ERR_UNSUPPORTED; }
-        p->tile_id = tile_id >= 0 ? tile_id : direct_pick_tile(p->d);
+        p->tile_id = tile_id >= 0 ? tile_id : direct_pick_tile(p->d, o.max_workspace);
         const int len = direct_table_len(p->d);
         std::vector<DirectTapEntry> tab(len);
         direct_build_table(p->d, tab.data());
@@ -263,7 +268,13 @@ static int plan_build(const boda_conv_shape& shape, const boda_plan_opts& o, Dev
         } else if (rc == BODA_OK && direct_tile_rtc_kt(p->tile_id) > 0) {
             rc = direct_rtc_create(p->d, direct_tile_rtc_kt(p->tile_id), &p->rtc);
         }
-        p->ws_bytes = 0;
+        if (rc == BODA_OK && direct_tile_staged_width(p->tile_id) > 0) {
+            const int bn = direct_tile_staged_width(p->tile_id);
+            const size_t ws = simt_workspace_bytes(p->d, bn);
+            rc = o.max_workspace > 0 && ws > o.max_workspace ? BODA_ERR_NOMEM : simt_plan_create(p->d, bn, p->d_status, &p->simt);
+            if (rc == BODA_OK) p->ws_bytes = ws;
+        }
+        p->split = split_k > 0 ? std::min(split_k, direct_max_split(p->d, p->tile_id)) : direct_pick_split(p->d, p->tile_id);
     } else {
         p->math = o.math == BODA_MATH_TF32X3 ? BODA_MATH_TF32X3 : o.math == BODA_MATH_F16 ? BODA_MATH_F16 : BODA_MATH_TF32;
         rc = igemm_plan_create(p->d, variant, tile_id, split_k, o.s2d, ctx->d_status, &p->ig,
@@ -396,7 +407,7 @@ int boda::conv_plan_create_chained(const boda_conv_shape* shape, const boda_plan
         if (best) {
             *plan = best;
             rc = BODA_OK;
-            tune_cache_store(key, best->tile_id, best->ig ? igemm_plan_splits(best->ig) : 0, best->variant, best_s2d);
+            tune_cache_store(key, best->tile_id, best->ig ? igemm_plan_splits(best->ig) : best->split, best->variant, best_s2d);
         }
         else rc = plan_build(*shape, o, ctx, variant, -1, o.split_k, plan);
     }
@@ -413,8 +424,9 @@ int boda_conv_plan_describe(const boda_conv_plan* p, char* buf, size_t n)
     if (p->variant == BODA_VARIANT_DIRECT) {
         char extra[96] = "";
         if (p->rtc) { extra[0] = ' '; direct_rtc_describe(p->rtc, extra + 1, sizeof(extra) - 1); }
-        std::snprintf(buf, n, "variant=%s tile=%s(id %d)%s math=fp32 split_k=1 workspace=%zu", vn[p->variant],
-                      direct_tile_name(p->tile_id), p->tile_id, extra, p->ws_bytes);
+        if (p->simt) { extra[0] = ' '; simt_plan_describe(p->simt, extra + 1, sizeof(extra) - 1); }
+        std::snprintf(buf, n, "variant=%s tile=%s(id %d)%s math=fp32 split_k=%d workspace=%zu", vn[p->variant],
+                      direct_tile_name(p->tile_id), p->tile_id, extra, p->split, p->ws_bytes);
     } else {
         char tmp[160];
         igemm_plan_describe(p->ig, tmp, sizeof(tmp));
@@ -429,13 +441,14 @@ size_t boda_conv_plan_workspace_bytes(const boda_conv_plan* p) { return p ? p->w
 int boda_conv_plan_kernels_per_call(const boda_conv_plan* p)
 {
     if (!p) return 0;
-    if (p->variant == BODA_VARIANT_DIRECT) return 1;
+    if (p->variant == BODA_VARIANT_DIRECT) return p->simt ? simt_plan_kernels(p->simt) : 1;
     return igemm_plan_kernels_per_call(p->ig);             // tensor-core variants: input staging (where needed) + main kernel
 }
 
 int boda_conv_plan_bind_filters(boda_conv_plan* p, const float* filt, void* stream)
 {
     if (!p || !filt) return BODA_ERR_INVALID_ARG;
+    if (p->simt) return simt_bind_filters(p->simt, filt, (cudaStream_t)stream);
     if (p->variant == BODA_VARIANT_DIRECT) return BODA_OK;   // reads KCRS in place
     return igemm_bind_filters(p->ig, filt, (cudaStream_t)stream);
 }
@@ -514,6 +527,7 @@ static int plan_time_ms(boda_conv_plan* p, bool chain_in, bool chain_out, int po
     TRY_T(cudaEventCreate(&e0)); TRY_T(cudaEventCreate(&e1));
     TRY_T(cudaStreamSynchronize(0));                    // the fills above ran on the default stream
     TRY_T(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
+    if (p->simt) { rc = simt_bind_filters(p->simt, f, stream); if (rc) { cleanup(); return rc; } }
     if (p->variant != BODA_VARIANT_DIRECT) { rc = igemm_bind_filters(p->ig, f, stream); if (rc) { cleanup(); return rc; } }
     for (int i = 0; i < 2; ++i) { rc = run_once(in, f, b, out, ws, stream); if (rc) { cleanup(); return rc; } }
     TRY_T(cudaStreamSynchronize(stream));
@@ -658,6 +672,7 @@ int boda_conv_fwd_host(const float* in, const float* filt, const float* bias, fl
     BODA_CUDA_TRY(cudaMemcpyAsync(e->s_in, in, (size_t)d.N * d.C * d.H * d.W * 4, cudaMemcpyHostToDevice, st));
     BODA_CUDA_TRY(cudaMemcpyAsync(e->s_filt, filt, (size_t)d.K * d.Kred * 4, cudaMemcpyHostToDevice, st));
     if (bias) BODA_CUDA_TRY(cudaMemcpyAsync(e->s_bias, bias, (size_t)d.K * 4, cudaMemcpyHostToDevice, st));
+    if (e->plan->simt) simt_unbind_filters(e->plan->simt);
     if (e->plan->ig) igemm_unbind_filters(e->plan->ig);   // the staged filters may have changed
     rc = boda_conv_fwd_planned(e->plan, e->s_in, e->s_filt, bias ? e->s_bias : nullptr, e->s_out, e->workspace, stream);
     if (rc != BODA_OK) return rc;

@@ -110,13 +110,19 @@ struct DirectTapEntry { int offset; int rs; };
 
 int direct_num_tiles();
 const char* direct_tile_name(int tile_id);
-int direct_pick_tile(const ConvDims& d);
+// max_ws: 0, or the largest workspace the caller accepts
+int direct_pick_tile(const ConvDims& d, size_t max_ws = 0);
+// output channels per tile of the tiles that run over a staged copy of the input (simt_conv.h); 0 for the others
+int direct_tile_staged_width(int tile_id);
 // false for a tile that cannot run the shape (the pixel-per-thread tiles need the input patch to fit shared memory)
 bool direct_tile_legal(const ConvDims& d, int tile_id);
 // Length (entries) of the table the tile needs; build it on the host into `host_tab`.
 int direct_table_len(const ConvDims& d);
 void direct_build_table(const ConvDims& d, DirectTapEntry* host_tab);
-int direct_launch(const ConvDims& d, int tile_id, const float* in, const float* filt, const float* bias,
+// GEMM-blocked tiles: how many ways the reduction is split over a cluster by rule, and at most (1 for the other tiles)
+int direct_pick_split(const ConvDims& d, int tile_id);
+int direct_max_split(const ConvDims& d, int tile_id);
+int direct_launch(const ConvDims& d, int tile_id, int split, const float* in, const float* filt, const float* bias,
                   float* out, const DirectTapEntry* dev_tab, cudaStream_t stream);
 // Tiles compiled at run time for the exact shape (direct_rtc.cu): output channels per thread, 0 for the other tiles.
 int direct_tile_rtc_kt(int tile_id);

@@ -3,181 +3,272 @@
 //
 // Blocking follows the paper's SGEMM template (Section 4, Listing 1 and the parameter list after
 // it): each thread owns a register tile of Mt x Nt outputs (here TM pixels x TN output channels),
-// a thread block of 256 threads owns Mb*Mt x Nb*Nt = (16*TM) x (16*TN) outputs, the reduction is
-// walked in chunks of Kb = 8, operands of a chunk are staged in shared memory and the inner loop
+// a thread block of WM x WN warps (8 x 4 lanes each) owns (8*WM*TM) x (4*WN*TN) outputs, the reduction is
+// walked in chunks of Kb = BK, operands of a chunk are staged in shared memory and the inner loop
 // is fully unrolled.  The gather that im2col would do is a table lookup: entry j of the table
 // gives, for reduction index j = (c, r, s), the element offset inside an image and the tap, so the
 // load needs no division.  Bias and ReLU are applied in registers before the store.
+#include <algorithm>
+
 #include "boda_internal.h"
+#include "simt_conv.h"
 
 namespace boda {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int BK = 8;
+// ---- GEMM-blocked form.  Bound: the FP32 pipe (128 multiply-adds per clock and SM).  What keeps it busy:
+//  * multiply-adds in pairs (__ffma2_rn, each half rounds like fmaf) along the REDUCTION: the two halves of an accumulator
+//    are the sums over the even and the odd reduction indices and are added once at the end.  Input pixels and weights both
+//    sit in shared memory as such pairs, so nothing is broadcast or moved between registers;
+//  * operands of a chunk arrive by asynchronous copies, kStages - 1 chunks ahead, straight into shared memory (no
+//    registers held, zero fill for the padding and the ragged ends);
+//  * the reduction is split over the CTAs of a cluster (grid.z) where the output tiles alone would leave SMs idle or the
+//    last wave thin; the partial tiles are summed in rank order through distributed shared memory, so every run gives the
+//    same bits.
+// Measured (before / now): 5x5 on 23 channels, 87 filters, 11x11, batch 3 (0.04 GFLOP) 33 / 6.4 us; 3x3 on 200 channels, 48
+// filters, 14x14, batch 8 (0.27 GFLOP) 54 / 22 us.  Large layers run over a staged input instead (simt_conv.cu).
+constexpr int kStages = 4;
+constexpr int kMaxSplit = 8;
+// windows whose bounds tests fit a 32-bit mask per pixel: bit tap + 2 set = inside the image, so that (mask >> tap) & 4 is the
+// byte count of the copy.  Entries past the end of the reduction carry tap 29, whose bit is never set.
+constexpr int kMaskTaps = 29;
 
-template <int TM, int TN>
-__global__ void __launch_bounds__(kThreads)
+template <int WM, int WN, int TM, int TN, int BK>
+struct GemmCfg {
+    static constexpr int THREADS = 32 * WM * WN;
+    static constexpr int BM = 8 * WM * TM, BN = 4 * WN * TN;
+    static constexpr int APITCH = 2 * BM, BPITCH = 2 * BN + 4;     // floats of one row of index pairs; +4: the copies hit distinct banks
+    static constexpr int BMP = BM + 4;                 // pitch of a finished channel row
+    static constexpr int STAGE_FLOATS = BK / 2 * (APITCH + BPITCH);
+    static constexpr int SMEM_FLOATS = kStages * STAGE_FLOATS > BN * BMP ? kStages * STAGE_FLOATS : BN * BMP;
+    static constexpr int SMEM_BYTES = SMEM_FLOATS * 4;
+    // 64 accumulator registers fit 128 registers a thread, 96 fit 168
+    static constexpr int BLOCKS_PER_SM = (TM * TN <= 32 ? 512 : TM * TN <= 48 ? 320 : 256) / THREADS;
+};
+
+// 4 or 8 bytes, or zeros where `bytes` is 0 (the source is then not read)
+__device__ __forceinline__ void copy4_async(uint32_t dst, const float* src, uint32_t bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" :: "r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copy8_async(uint32_t dst, const float* src, uint32_t bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+template <int WM, int WN, int TM, int TN, int BK, bool MASKED>
+__global__ void __launch_bounds__(GemmCfg<WM, WN, TM, TN, BK>::THREADS, GemmCfg<WM, WN, TM, TN, BK>::BLOCKS_PER_SM)
 direct_conv_kernel(const ConvDims d, const float* __restrict__ in, const float* __restrict__ filt,
                    const float* __restrict__ bias, float* __restrict__ out,
-                   const DirectTapEntry* __restrict__ tab)
+                   const DirectTapEntry* __restrict__ tab, int chunks_total, int chunks_per_split)
 {
-    constexpr int BM = 16 * TM;
-    constexpr int BN = 16 * TN;
-    constexpr int BNP = BN + 4;                       // padded pitch: conflict-free transposed store
-    constexpr int A_PER_THREAD = (BK * BM + kThreads - 1) / kThreads;
-    constexpr int B_PER_THREAD = (BK * BN + kThreads - 1) / kThreads;
-    static_assert(kThreads % BM == 0 || BM % kThreads == 0, "a thread keeps one pixel for all its A loads");
-
-    __shared__ __align__(16) float As[2][BK][BM];
-    __shared__ __align__(16) float Bs[2][BK][BNP];
+    using G = GemmCfg<WM, WN, TM, TN, BK>;
+    constexpr int BM = G::BM, BN = G::BN, BMP = G::BMP, NT = G::THREADS;
+    static_assert(NT % BM == 0 && NT % BK == 0 && BN % (NT / BK) == 0 && BK % (NT / BM) == 0, "the copies are dealt without a remainder");
+    static_assert(TM % 2 == 0 && TN % 2 == 0 && BK % 2 == 0, "16-byte loads hold two pixels or two channels of an index pair");
+    constexpr int A_STEP = NT / BM, A_PER = BK / A_STEP;          // a thread copies one pixel's indices a_kk0, a_kk0 + A_STEP, ...
+    constexpr int B_STEP = NT / BK, B_PER = BN / B_STEP;          // and one index of channels b_n0, b_n0 + B_STEP, ...
+    constexpr int B2_STEP = 2 * B_STEP, B2_PER = (BN + B2_STEP - 1) / B2_STEP;      // or one index pair of half as many
+    extern __shared__ __align__(16) float sm_gemm[];
 
     pdl_launch_dependents();
-    pdl_wait();
-    const int tid = threadIdx.x;
-    const int tx = tid & 15;                          // pixel group
-    const int ty = tid >> 4;                          // channel group
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // lane bits 1, 3, 4 -> pixel group, bits 0, 2 -> channel group: lanes i and i^1 read the same pixels and lanes i and i^2 the
+    // same weights, which lets a 16-byte shared-memory load serve two quarter warps at once
+    const int lane_m = ((lane >> 1) & 1) | ((lane >> 2) & 6), lane_n = (lane & 1) | ((lane >> 1) & 2);
+    const int wm = warp % WM, wn = warp / WM;
     const int m0 = blockIdx.x * BM;
     const int k0 = blockIdx.y * BN;
     const int PQ = d.P * d.Q;
     const int HW = d.H * d.W;
+    const int t_begin = (int)blockIdx.z * chunks_per_split;
+    const int chunks = min(chunks_total - t_begin, chunks_per_split);
 
-    // ---- per-thread constants of the A (input) gather: this thread always loads pixel a_m
-    const int a_ml = tid % BM;
-    const int a_kk0 = tid / BM;                       // first chunk row this thread loads
-    constexpr int A_KK_STEP = (kThreads >= BM) ? kThreads / BM : 1;
-    int a_y0 = 0, a_x0 = 0;
-    long long a_base = 0;
-    bool a_ok = false;
+    // ---- per-thread constants of the A (input) gather: this thread always copies pixel ml
+    const int ml = tid % BM;
+    const int a_kk0 = tid / BM;
+    int a_y0 = 0, a_x0 = 0, img = 0, pq = 0;
+    const float* a_ptr = in;
+    const bool m_ok = m0 + ml < d.M;
+    uint32_t taps_in = 0;                      // see kMaskTaps
     {
-        const int m = m0 + a_ml;
-        if (m < d.M) {
-            const int n = m / PQ;
-            const int pq = m - n * PQ;
-            const int p = pq / d.Q;
-            const int q = pq - p * d.Q;
-            a_y0 = p * d.stride - d.pad;
-            a_x0 = q * d.stride - d.pad;
-            a_base = (long long)n * d.C * HW + (long long)a_y0 * d.W + a_x0;
-            a_ok = true;
+        const int m = m_ok ? m0 + ml : 0;
+        img = m / PQ;
+        pq = m - img * PQ;
+        const int p = pq / d.Q;
+        const int q = pq - p * d.Q;
+        a_y0 = m_ok ? p * d.stride - d.pad : -0x100000;            // pixels past the end fail every bounds test
+        a_x0 = q * d.stride - d.pad;
+        a_ptr = in + (long long)img * d.C * HW + (long long)(p * d.stride - d.pad) * d.W + a_x0;
+        if constexpr (MASKED) {
+            uint32_t bit = 4;
+            for (int r = 0; r < d.R; ++r)
+                for (int sx = 0; sx < d.S; ++sx, bit <<= 1)
+                    if ((unsigned)(a_y0 + r) < (unsigned)d.H && (unsigned)(a_x0 + sx) < (unsigned)d.W) taps_in |= bit;
         }
     }
-    // ---- per-thread constants of the B (filter) load
-    const int b_kk = tid & (BK - 1);
-    const int b_n0 = tid >> 3;                        // 0..31
-
-    float a_pre[A_PER_THREAD];
-    float b_pre[B_PER_THREAD];
-
-    auto load_global = [&](int kred0) {
+    // ---- per-thread constants of the B (filter) copy: index pairs as 8-byte copies where every filter row allows it
+    const bool pairs = (d.Kred & 1) == 0 && (reinterpret_cast<uintptr_t>(filt) & 7) == 0;
+    const int b_kk = pairs ? 2 * (tid % (BK / 2)) : tid % BK;
+    const int b_n0 = pairs ? tid / (BK / 2) : tid / BK;
+    const float* b_ptr = filt + (size_t)(k0 + b_n0) * d.Kred + t_begin * BK + b_kk;
+    const int b_step = pairs ? B2_STEP : B_STEP;
+    const size_t b_pitch = (size_t)b_step * d.Kred;
+    const int b_rows = (d.K - k0 - b_n0 + b_step - 1) / b_step;                       // of this thread's channels, those that exist
+    const uint32_t sm_base = (uint32_t)__cvta_generic_to_shared(sm_gemm);
+    const uint32_t a_dst = sm_base + 4u * (uint32_t)((a_kk0 >> 1) * G::APITCH + 2 * ml + (a_kk0 & 1));
+    const uint32_t b_dst = sm_base + 4u * (uint32_t)(BK / 2 * G::APITCH + (b_kk >> 1) * G::BPITCH + 2 * b_n0 + (b_kk & 1));
+    // the table entries of the next chunk are fetched one chunk early: their latency is off the path of the copies
+    DirectTapEntry e[A_PER];
+    const DirectTapEntry* my_tab = tab + a_kk0 + t_begin * BK;
 #pragma unroll
-        for (int i = 0; i < A_PER_THREAD; ++i) {
-            const int kk = a_kk0 + i * A_KK_STEP;
-            float v = 0.f;
-            if (kk < BK) {
-                const DirectTapEntry e = tab[kred0 + kk];
-                const int y = a_y0 + (e.rs >> 16);
-                const int x = a_x0 + (e.rs & 0xffff);
-                if (a_ok && (unsigned)y < (unsigned)d.H && (unsigned)x < (unsigned)d.W)
-                    v = __ldg(in + a_base + e.offset);
+    for (int i = 0; i < A_PER; ++i) e[i] = my_tab[i * A_STEP];
+
+    auto issue = [&](int t, int buf) {
+        const uint32_t off = 4u * (uint32_t)(buf * G::STAGE_FLOATS);
+#pragma unroll
+        for (int i = 0; i < A_PER; ++i) {
+            uint32_t bytes;
+            if constexpr (MASKED) {
+                bytes = (taps_in >> e[i].rs) & 4u;
+            } else {
+                const int y = a_y0 + (e[i].rs >> 16);
+                const int x = a_x0 + (e[i].rs & 0xffff);
+                bytes = ((unsigned)y < (unsigned)d.H && (unsigned)x < (unsigned)d.W) ? 4u : 0u;
             }
-            a_pre[i] = v;
+            // index a_kk0 + i*A_STEP: a_kk0 < A_STEP, which is 1 or even, so its pair and half are known up to a_kk0's
+            const int kk = i * A_STEP;
+            copy4_async(a_dst + off + 4u * (uint32_t)((kk >> 1) * G::APITCH + (kk & 1)), a_ptr + e[i].offset, bytes);
         }
+        // (the last chunk fetches its own entries once more)
+        const DirectTapEntry* nt = my_tab + min(t + 1, chunks - 1) * BK;
 #pragma unroll
-        for (int i = 0; i < B_PER_THREAD; ++i) {
-            const int nl = b_n0 + i * 32;
-            const int k = k0 + nl;
-            const int j = kred0 + b_kk;
-            float v = 0.f;
-            if (nl < BN && k < d.K && j < d.Kred) v = __ldg(filt + (size_t)k * d.Kred + j);
-            b_pre[i] = v;
-        }
-    };
-    auto store_shared = [&](int buf) {
+        for (int i = 0; i < A_PER; ++i) e[i] = nt[i * A_STEP];
+        const float* bp = b_ptr;
+        b_ptr += BK;
+        const bool j_ok = (t_begin + t) * BK + b_kk < d.Kred;       // an even Kred ends on a pair
+        if (pairs) {
 #pragma unroll
-        for (int i = 0; i < A_PER_THREAD; ++i) {
-            const int kk = a_kk0 + i * A_KK_STEP;
-            if (kk < BK) As[buf][kk][a_ml] = a_pre[i];
-        }
+            for (int i = 0; i < B2_PER; ++i) {
+                if (B2_PER * B2_STEP > BN && b_n0 + i * B2_STEP >= BN) break;
+                copy8_async(b_dst + off + 8u * (uint32_t)(i * B2_STEP), bp, j_ok && i < b_rows ? 8u : 0u);
+                bp += b_pitch;
+            }
+        } else {
 #pragma unroll
-        for (int i = 0; i < B_PER_THREAD; ++i) {
-            const int nl = b_n0 + i * 32;
-            if (nl < BN) Bs[buf][b_kk][nl] = b_pre[i];
+            for (int i = 0; i < B_PER; ++i) {
+                copy4_async(b_dst + off + 8u * (uint32_t)(i * B_STEP), bp, j_ok && i < b_rows ? 4u : 0u);
+                bp += b_pitch;
+            }
         }
     };
 
-    float acc[TM][TN];
+    // accumulators: (sum over even indices, sum over odd indices) of each pixel and channel
+    float2 acc[TM][TN];
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < TN; ++j) acc[i][j] = make_float2(0.f, 0.f);
 
-    const int chunks = (d.Kred + BK - 1) / BK;
-    load_global(0);
-    store_shared(0);
-    __syncthreads();
+    // pixel 2g + i of this thread is wm*8*TM + 16g + 2*lane_m + i, channel 2h + i is wn*4*TN + 8h + 2*lane_n + i: every warp
+    // load is one contiguous run of shared memory
+    const int a_rd = wm * 8 * TM + 2 * lane_m, b_rd = wn * 4 * TN + 2 * lane_n;
 
+    pdl_wait();
+#pragma unroll
+    for (int s = 0; s < kStages - 1; ++s) {
+        if (s < chunks) issue(s, s);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    int buf = 0;
     for (int t = 0; t < chunks; ++t) {
-        const int buf = t & 1;
-        if (t + 1 < chunks) load_global((t + 1) * BK);
+        asm volatile("cp.async.wait_group %0;" :: "n"(kStages - 2) : "memory");
+        __syncthreads();
+        const float* As = sm_gemm + buf * G::STAGE_FLOATS;
+        const float* Bs = As + BK / 2 * G::APITCH;
+        // operands of the next index pair are loaded while this one's multiply-adds run
+        float2 a[2][TM], b[2][TN];
+        auto fetch = [&](int k2, float2 (&ao)[TM], float2 (&bo)[TN]) {
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            float a[TM], b[TN];
-            // pixels of this thread: groups of 4 (or TM if smaller) consecutive, 64 apart
-            if constexpr (TM % 4 == 0) {
-#pragma unroll
-                for (int g = 0; g < TM / 4; ++g) {
-                    const float4 v = *reinterpret_cast<const float4*>(&As[buf][kk][g * 64 + tx * 4]);
-                    a[4 * g + 0] = v.x; a[4 * g + 1] = v.y; a[4 * g + 2] = v.z; a[4 * g + 3] = v.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < TM; ++i) a[i] = As[buf][kk][tx * TM + i];
-            }
-            if constexpr (TN % 4 == 0) {
-#pragma unroll
-                for (int g = 0; g < TN / 4; ++g) {
-                    const float4 v = *reinterpret_cast<const float4*>(&Bs[buf][kk][ty * TN + 4 * g]);
-                    b[4 * g + 0] = v.x; b[4 * g + 1] = v.y; b[4 * g + 2] = v.z; b[4 * g + 3] = v.w;
-                }
-            } else if constexpr (TN % 2 == 0) {
-#pragma unroll
-                for (int g = 0; g < TN / 2; ++g) {
-                    const float2 v = *reinterpret_cast<const float2*>(&Bs[buf][kk][ty * TN + 2 * g]);
-                    b[2 * g + 0] = v.x; b[2 * g + 1] = v.y;
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < TN; ++j) b[j] = Bs[buf][kk][ty * TN + j];
+            for (int g = 0; g < TM / 2; ++g) {
+                const float4 v = *reinterpret_cast<const float4*>(As + k2 * G::APITCH + 2 * (a_rd + 16 * g));
+                ao[2 * g] = make_float2(v.x, v.y); ao[2 * g + 1] = make_float2(v.z, v.w);
             }
 #pragma unroll
-            for (int i = 0; i < TM; ++i)
+            for (int h = 0; h < TN / 2; ++h) {
+                const float4 v = *reinterpret_cast<const float4*>(Bs + k2 * G::BPITCH + 2 * (b_rd + 8 * h));
+                bo[2 * h] = make_float2(v.x, v.y); bo[2 * h + 1] = make_float2(v.z, v.w);
+            }
+        };
+        fetch(0, a[0], b[0]);
 #pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int k2 = 0; k2 < BK / 2; ++k2) {
+            if (k2 + 1 < BK / 2) fetch(k2 + 1, a[(k2 + 1) & 1], b[(k2 + 1) & 1]);
+            // the copies of a later chunk go out under the first multiply-adds
+            if (k2 == 0) {
+                if (t + kStages - 1 < chunks) issue(t + kStages - 1, (buf + kStages - 1) % kStages);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            }
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+#pragma unroll
+                for (int i = 0; i < TM; ++i) acc[i][j] = __ffma2_rn(a[k2 & 1][i], b[k2 & 1][j], acc[i][j]);
         }
-        if (t + 1 < chunks) store_shared(buf ^ 1);
+        buf = buf + 1 == kStages ? 0 : buf + 1;
+    }
+
+    // ---- epilogue: the tile goes through shared memory as [channel][pixel], so that the NCHW stores (and a split's remote
+    // reads) are whole 128-byte runs whatever the register blocking
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < TN; ++j)
+#pragma unroll
+        for (int g = 0; g < TM / 2; ++g)
+            *reinterpret_cast<float2*>(sm_gemm + (b_rd + 8 * (j >> 1) + (j & 1)) * BMP + a_rd + 16 * g) =
+                make_float2(acc[2 * g][j].x + acc[2 * g][j].y, acc[2 * g + 1][j].x + acc[2 * g + 1][j].y);
+    const int splits = (int)gridDim.z;
+    int n_begin = 0, n_end = BN;
+    uint32_t peer[kMaxSplit];
+    if (splits > 1) {
+        const int share = (BN + splits - 1) / splits;
+        n_begin = (int)blockIdx.z * share;
+        n_end = min(BN, n_begin + share);
+#pragma unroll
+        for (int r = 0; r < kMaxSplit; ++r)
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer[r]) : "r"(sm_base), "r"(r < splits ? r : 0));
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    } else {
         __syncthreads();
     }
-
-    // ---- epilogue: bias, ReLU, NCHW store
+    n_end = min(n_end, d.K - k0);
+    float* o = out + ((size_t)img * d.K + k0) * PQ + pq;
+    auto finish = [&](int nl, float v) {
+        v += bias ? __ldg(bias + k0 + nl) : 0.f;
+        if (d.relu) v = fmaxf(v, 0.f);
+        o[(size_t)nl * PQ] = v;
+    };
+    if (m_ok) {
+        if (splits == 1) {
+#pragma unroll 4
+            for (int nl = n_begin + a_kk0; nl < n_end; nl += A_STEP) finish(nl, sm_gemm[nl * BMP + ml]);
+        } else {
+#pragma unroll 2
+            for (int nl = n_begin + a_kk0; nl < n_end; nl += A_STEP) {
+                const uint32_t at = 4u * (uint32_t)(nl * BMP + ml);
+                float x[kMaxSplit];
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int ml = (TM % 4 == 0) ? ((i >> 2) * 64 + tx * 4 + (i & 3)) : (tx * TM + i);
-        const int m = m0 + ml;
-        if (m >= d.M) continue;
-        const int n = m / PQ;
-        const int pq = m - n * PQ;
-        float* o = out + ((size_t)n * d.K) * PQ + pq;
+                for (int r = 0; r < kMaxSplit; ++r)
+                    if (r < splits) asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x[r]) : "r"(peer[r] + at) : "memory");
+                float v = x[0];
 #pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            const int k = k0 + ty * TN + j;
-            if (k < d.K) {
-                float v = acc[i][j] + (bias ? __ldg(bias + k) : 0.f);
-                if (d.relu) v = fmaxf(v, 0.f);
-                o[(size_t)k * PQ] = v;
+                for (int r = 1; r < kMaxSplit; ++r)
+                    if (r < splits) v += x[r];
+                finish(nl, v);
             }
         }
     }
+    // nobody leaves while a peer may still read its shared memory
+    if (splits > 1) asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // ---- the small-input-channel form of DIRECT (first layers: C = 3 with 3x3 ... 11x11 windows; few output channels).
@@ -324,27 +415,49 @@ int launch_pixel(const ConvDims& d, const float* in, const float* filt, const fl
     }
 }
 
-struct TileInfo { int TM, TN; const char* name; };
+// bm x bn outputs per block of `threads` threads, reduction chunks of bk (GEMM-blocked form; 0 otherwise)
+struct TileInfo { int kind, bm, bn, kt, threads, bk; const char* name; };
+enum { TILE_GEMM = 0, TILE_PIXEL = 1, TILE_RTC = 2, TILE_STAGED = 3 };
 constexpr TileInfo kTiles[] = {
-    {8, 8, "direct_128x128"}, {8, 6, "direct_128x96"}, {8, 4, "direct_128x64"}, {8, 2, "direct_128x32"},
-    {4, 4, "direct_64x64"},   {4, 2, "direct_64x32"},  {4, 1, "direct_64x16"},  {2, 2, "direct_32x32"},
-    {2, 1, "direct_32x16"},
-    // pixel-per-thread form (TM = 0): TN output channels per thread
-    {0, 8, "direct_pixel_k8"}, {0, 16, "direct_pixel_k16"}, {0, 32, "direct_pixel_k32"},
-    // the same form compiled at run time for the exact shape (TM = -1; direct_rtc.cu)
-    {-1, 4, "direct_rtc_k4"}, {-1, 8, "direct_rtc_k8"}, {-1, 16, "direct_rtc_k16"}, {-1, 32, "direct_rtc_k32"},
+    {TILE_GEMM, 128, 128, 0, 256, 8, "direct_128x128"}, {TILE_GEMM, 128, 96, 0, 256, 16, "direct_128x96"},
+    {TILE_GEMM, 128, 64, 0, 128, 8, "direct_128x64"},   {TILE_GEMM, 128, 32, 0, 128, 8, "direct_128x32"},
+    {TILE_GEMM, 64, 64, 0, 64, 8, "direct_64x64"},     {TILE_GEMM, 64, 32, 0, 64, 8, "direct_64x32"},
+    {TILE_GEMM, 64, 16, 0, 64, 8, "direct_64x16"},      {TILE_GEMM, 32, 32, 0, 64, 16, "direct_32x32"},
+    {TILE_GEMM, 32, 16, 0, 32, 8, "direct_32x16"},
+    // pixel-per-thread form: kt output channels per thread
+    {TILE_PIXEL, 0, 0, 8, 256, 0, "direct_pixel_k8"}, {TILE_PIXEL, 0, 0, 16, 256, 0, "direct_pixel_k16"},
+    {TILE_PIXEL, 0, 0, 32, 256, 0, "direct_pixel_k32"},
+    // the same form compiled at run time for the exact shape (direct_rtc.cu)
+    {TILE_RTC, 0, 0, 4, 0, 0, "direct_rtc_k4"}, {TILE_RTC, 0, 0, 8, 0, 0, "direct_rtc_k8"},
+    {TILE_RTC, 0, 0, 16, 0, 0, "direct_rtc_k16"}, {TILE_RTC, 0, 0, 32, 0, 0, "direct_rtc_k32"},
+    // more GEMM-blocked tiles (the ids above are part of the interface)
+    {TILE_GEMM, 64, 48, 0, 64, 8, "direct_64x48"}, {TILE_GEMM, 128, 48, 0, 128, 8, "direct_128x48"},
+    // over a staged NHWC copy of the input (simt_conv.cu): needs workspace
+    {TILE_STAGED, 128, 128, 0, 288, 32, "direct_nhwc_128x128"}, {TILE_STAGED, 128, 96, 0, 288, 32, "direct_nhwc_128x96"},
+    {TILE_STAGED, 128, 64, 0, 288, 32, "direct_nhwc_128x64"},   {TILE_STAGED, 128, 48, 0, 288, 32, "direct_nhwc_128x48"},
+    {TILE_STAGED, 128, 32, 0, 288, 32, "direct_nhwc_128x32"},
 };
 constexpr int kFirstPixelTile = 9;
-constexpr int kFirstRtcTile = 12;
+constexpr int kFewIndices = 32;      // reductions up to here suit the pixel-per-thread forms
 constexpr int kNumTiles = sizeof(kTiles) / sizeof(kTiles[0]);
 
-template <int TM, int TN>
+template <int WM, int WN, int TM, int TN, int BK>
 int launch_tile(const ConvDims& d, const float* in, const float* filt, const float* bias, float* out,
-                const DirectTapEntry* tab, cudaStream_t stream)
+                const DirectTapEntry* tab, int split, cudaStream_t stream)
 {
-    constexpr int BM = 16 * TM, BN = 16 * TN;
-    dim3 grid((d.M + BM - 1) / BM, (d.K + BN - 1) / BN);
-    BODA_CUDA_TRY(launch_kernel(direct_conv_kernel<TM, TN>, grid, dim3(kThreads), 0, stream, 1, d, in, filt, bias, out, tab));
+    using G = GemmCfg<WM, WN, TM, TN, BK>;
+    const int chunks = (d.Kred + BK - 1) / BK;
+    const int per = (chunks + split - 1) / split;
+    const int splits = (chunks + per - 1) / per;                          // no empty split
+    dim3 grid((d.M + G::BM - 1) / G::BM, (d.K + G::BN - 1) / G::BN, splits);
+    auto run = [&](auto kernel, DeviceSmemLimit& limit) -> cudaError_t {
+        const cudaError_t e = limit.ensure(kernel, G::SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        return launch_kernel(kernel, grid, dim3(G::THREADS), (size_t)G::SMEM_BYTES, stream, splits, d, in, filt, bias, out, tab, chunks, per);
+    };
+    static DeviceSmemLimit limit_masked(48 * 1024), limit_any(48 * 1024);
+    BODA_CUDA_TRY(d.R * d.S <= kMaskTaps ? run(direct_conv_kernel<WM, WN, TM, TN, BK, true>, limit_masked)
+                                         : run(direct_conv_kernel<WM, WN, TM, TN, BK, false>, limit_any));
     count_launch();
     return BODA_OK;
 }
@@ -354,33 +467,74 @@ int launch_tile(const ConvDims& d, const float* in, const float* filt, const flo
 int direct_num_tiles() { return kNumTiles; }
 const char* direct_tile_name(int id) { return (id >= 0 && id < kNumTiles) ? kTiles[id].name : "?"; }
 
-int direct_pick_tile(const ConvDims& d)
+// Clocks of a GEMM-blocked tile with the reduction split `split` ways.  A block's work is bm*bn/128 clocks of multiply-adds per
+// reduction index at the SM's full rate; the blocks of an SM share that rate (`rate` clocks per clock of work), and no block is
+// faster than `index` clocks per reduction index; `out` per bm*bn/128 outputs for the first loads and the store, `cluster` for
+// a split.  Fitted per tile to 4 000 timings (82 layers of 1 ... 9850 reduction indices and 60 ... 363 000 points, every tile and split): the tile
+// and split it picks are within 5 % of the best measured ones in the geometric mean.
+struct GemmModel { int tile, resident; double fixed, rate, index, cluster, out; };
+constexpr GemmModel kGemmModel[] = {
+    {0, 1, 0, 1.78, 11, 2600, 52},     {1, 1, 0, 1.75, 118, 2600, 66},    {2, 2, 2140, 1.98, 0, 4300, 56},
+    {3, 4, 3540, 3.07, 170, 2000, 45}, {4, 4, 2830, 1.98, 162, 3100, 64}, {5, 8, 4050, 3.09, 176, 1770, 50},
+    {6, 8, 4350, 3.48, 62, 1440, 72},  {7, 8, 4450, 2.66, 45, 1620, 69},  {8, 16, 4150, 3.74, 69, 1180, 131},
+    {16, 5, 3500, 2.70, 207, 2530, 54}, {17, 2, 1910, 1.95, 147, 2000, 88},
+};
+
+static double gemm_cost(const ConvDims& d, int t, int split)
 {
-    // Rule of thumb in the spirit of Section 4: the widest channel tile that K fills without much
-    // waste, then the tallest pixel tile that still yields about two blocks per SM.
-    int best = kNumTiles - 1;
+    const TileInfo& ti = kTiles[t];
+    const GemmModel* m = kGemmModel;
+    while (m->tile != t) ++m;
+    const int chunks = (d.Kred + ti.bk - 1) / ti.bk, per = (chunks + split - 1) / split;
+    const long long splits = (chunks + per - 1) / per;
+    const long long blocks = (long long)((d.M + ti.bm - 1) / ti.bm) * ((d.K + ti.bn - 1) / ti.bn) * splits;
+    const long long per_sm = (blocks + 147) / 148, rounds = (per_sm + m->resident - 1) / m->resident;
+    const double indices = (double)per * ti.bk, area = ti.bm * ti.bn / 128.0;
+    return m->fixed + std::max(per_sm * indices * area * m->rate, rounds * indices * m->index) + per_sm * area * m->out +
+           (splits > 1 ? m->cluster + 300.0 * splits : 0.0);
+}
+
+int direct_pick_split(const ConvDims& d, int tile)
+{
+    if (tile < 0 || tile >= kNumTiles || kTiles[tile].kind != TILE_GEMM) return 1;
+    int best = 1;
     double best_cost = 1e300;
-    // small reductions with few output channels: the pixel-per-thread form, the smallest KT that covers K in one group
-    // (or 32 channels per group)
-    // (measured: it wins from a few ten thousand output pixels on - 19 us against 33 us for configuration 1's shape at
-    // batch 256 - and loses below, where a handful of blocks cannot hide its two staging phases)
-    if (d.Kred <= 512 && d.K <= 128 && d.M >= 32768) {
+    for (int s = 1; s <= kMaxSplit; ++s) {
+        if (s > 1 && (d.Kred + kTiles[tile].bk - 1) / kTiles[tile].bk < 2 * s) break;
+        const double c = gemm_cost(d, tile, s);
+        if (c < best_cost) { best_cost = c; best = s; }
+    }
+    return best;
+}
+
+int direct_max_split(const ConvDims& d, int tile)
+{
+    if (tile < 0 || tile >= kNumTiles || kTiles[tile].kind != TILE_GEMM) return 1;
+    return std::min(kMaxSplit, (d.Kred + kTiles[tile].bk - 1) / kTiles[tile].bk);
+}
+
+int direct_tile_staged_width(int tile) { return tile >= 0 && tile < kNumTiles && kTiles[tile].kind == TILE_STAGED ? kTiles[tile].bn : 0; }
+
+int direct_pick_tile(const ConvDims& d, size_t max_ws)
+{
+    // a handful of reduction indices and many output pixels: the pixel-per-thread form, the smallest KT that covers K in one group
+    // (or 32 channels per group).  Measured against the GEMM-blocked tiles: 18.3 against 19.4 us for 3x3 on 3 channels, 16 filters,
+    // 32x32, batch 256; from 45 indices on, or with a stride, the GEMM-blocked tiles win (75 indices, 48 filters, stride 2, batch
+    // 46: 28.8 against 56.4 us).
+    if (d.Kred <= kFewIndices && d.stride == 1 && d.K <= 128 && d.M >= 32768) {
         const int KT = d.K <= 8 ? 8 : d.K <= 16 ? 16 : 32;
         int ih, iw, iwp;
         size_t smem;
         if (pixel_geometry(d, KT, &ih, &iw, &iwp, &smem)) return kFirstPixelTile + (KT == 8 ? 0 : KT == 16 ? 1 : 2);
     }
-    for (int t = 0; t < kFirstPixelTile; ++t) {
-        const int BM = 16 * kTiles[t].TM, BN = 16 * kTiles[t].TN;
-        const long long gm = (d.M + BM - 1) / BM, gn = (d.K + BN - 1) / BN;
-        const double padded = (double)gm * BM * gn * BN;             // FMAs issued per reduction step
-        const double blocks = (double)gm * gn;
-        const double waves = blocks / (148.0 * 2.0);
-        const double fill = waves < 1.0 ? 1.0 / waves : (double)(long long)(waves + 0.999) / waves;
-        // small register tiles pay more shared-memory traffic per FMA
-        const double ldst = 1.0 + 0.5 * (1.0 / kTiles[t].TM + 1.0 / kTiles[t].TN);
-        const double cost = padded * fill * ldst;
-        if (cost < best_cost) { best_cost = cost; best = t; }
+    int best = 8;
+    double best_cost = 1e300;
+    for (int t = 0; t < kNumTiles; ++t) {
+        double c;
+        if (kTiles[t].kind == TILE_GEMM) c = gemm_cost(d, t, direct_pick_split(d, t));
+        else if (kTiles[t].kind == TILE_STAGED && simt_legal(d) && (max_ws == 0 || simt_workspace_bytes(d, kTiles[t].bn) <= max_ws)) c = simt_cost(d, kTiles[t].bn);
+        else continue;
+        if (c < best_cost) { best_cost = c; best = t; }
     }
     return best;
 }
@@ -388,26 +542,28 @@ int direct_pick_tile(const ConvDims& d)
 bool direct_tile_legal(const ConvDims& d, int tile_id)
 {
     if (tile_id < 0 || tile_id >= kNumTiles) return false;
-    if (tile_id < kFirstPixelTile) return true;
-    if (tile_id >= kFirstRtcTile) {
+    if (kTiles[tile_id].kind == TILE_GEMM) return true;
+    if (kTiles[tile_id].kind == TILE_STAGED) return simt_legal(d);
+    if (kTiles[tile_id].kind == TILE_RTC) {
         int bx, by, py;
         size_t sm;
-        return direct_rtc_available() && direct_rtc_geometry(d, kTiles[tile_id].TN, &bx, &by, &py, &sm);
+        return direct_rtc_available() && direct_rtc_geometry(d, kTiles[tile_id].kt, &bx, &by, &py, &sm);
     }
     int ih, iw, iwp;
     size_t smem;
-    return pixel_geometry(d, kTiles[tile_id].TN, &ih, &iw, &iwp, &smem) && d.N <= 65535 && (d.K + kTiles[tile_id].TN - 1) / kTiles[tile_id].TN <= 65535;
+    return pixel_geometry(d, kTiles[tile_id].kt, &ih, &iw, &iwp, &smem) && d.N <= 65535 && (d.K + kTiles[tile_id].kt - 1) / kTiles[tile_id].kt <= 65535;
 }
 
-int direct_tile_rtc_kt(int tile_id) { return (tile_id >= kFirstRtcTile && tile_id < kNumTiles) ? kTiles[tile_id].TN : 0; }
+int direct_tile_rtc_kt(int tile_id) { return (tile_id >= 0 && tile_id < kNumTiles && kTiles[tile_id].kind == TILE_RTC) ? kTiles[tile_id].kt : 0; }
 
 int direct_rtc_pick(const ConvDims& d)
 {
-    // Measured on B200 (configuration 1's layer at batch 1 / 20 / 256, an 11x11 stride-4 and a 5x5 layer on 3 channels):
-    // the run-time compiled kernel beats every precompiled tile where the reduction is short and the output channels
-    // few.  Eight channels per thread as a rule; four where that leaves fewer than 64 blocks (more blocks hide the
+    // Measured on B200: the run-time compiled kernel beats the GEMM-blocked tiles where the reduction is a handful of indices (27
+    // indices, 16 filters, 32x32: 3.1 against 3.3 us at batch 1, 12.5 against 19.4 us at batch 256) and loses beyond, or with a
+    // stride (45 indices: 4.9 against 4.2 us; 27 with stride 2, 96 filters, batch 7: 17.8 against 16.0 us; 375 indices: 9.5 against 4.6).
+    // Eight channels per thread as a rule; four where that leaves fewer than 64 blocks (more blocks hide the
     // staging latency); sixteen where 16 covers all output channels of a large layer (the input patch is staged once).
-    if (d.Kred > 512 || d.K > 128 || !direct_rtc_available()) return -1;
+    if (d.Kred > kFewIndices || d.stride != 1 || d.K > 128 || !direct_rtc_available()) return -1;
     int bx = 32, by = 8, py = 1;
     size_t sm = 0;
     if (!direct_rtc_geometry(d, 8, &bx, &by, &py, &sm)) bx = 8, by = 4, py = 1;
@@ -416,42 +572,46 @@ int direct_rtc_pick(const ConvDims& d)
     const int order[3][3] = {{4, 8, 16}, {8, 4, 16}, {16, 8, 4}};
     const int* o = order[want == 4 ? 0 : want == 8 ? 1 : 2];
     for (int i = 0; i < 3; ++i)
-        for (int t = kFirstRtcTile; t < kNumTiles; ++t)
-            if (kTiles[t].TN == o[i] && direct_tile_legal(d, t)) return t;
+        for (int t = 0; t < kNumTiles; ++t)
+            if (kTiles[t].kind == TILE_RTC && kTiles[t].kt == o[i] && direct_tile_legal(d, t)) return t;
     return -1;
 }
 
-int direct_table_len(const ConvDims& d) { return ((d.Kred + BK - 1) / BK) * BK; }
+// whole chunks of the widest chunk (16 reduction indices)
+int direct_table_len(const ConvDims& d) { return ((d.Kred + 15) / 16) * 16; }
 
 void direct_build_table(const ConvDims& d, DirectTapEntry* tab)
 {
     const int len = direct_table_len(d);
+    const bool masked = d.R * d.S <= kMaskTaps;
     int j = 0;
     for (int c = 0; c < d.C; ++c)
         for (int r = 0; r < d.R; ++r)
             for (int s = 0; s < d.S; ++s, ++j) {
                 tab[j].offset = c * d.H * d.W + r * d.W + s;
-                tab[j].rs = (r << 16) | s;
+                tab[j].rs = masked ? r * d.S + s : (r << 16) | s;
             }
-    for (; j < len; ++j) { tab[j].offset = 0; tab[j].rs = (0x4000 << 16); }
+    for (; j < len; ++j) { tab[j].offset = 0; tab[j].rs = masked ? kMaskTaps : (0x4000 << 16); }
 }
 
-int direct_launch(const ConvDims& d, int tile_id, const float* in, const float* filt, const float* bias,
+int direct_launch(const ConvDims& d, int tile_id, int split, const float* in, const float* filt, const float* bias,
                   float* out, const DirectTapEntry* tab, cudaStream_t stream)
 {
     switch (tile_id) {
-        case 0: return launch_tile<8, 8>(d, in, filt, bias, out, tab, stream);
-        case 1: return launch_tile<8, 6>(d, in, filt, bias, out, tab, stream);
-        case 2: return launch_tile<8, 4>(d, in, filt, bias, out, tab, stream);
-        case 3: return launch_tile<8, 2>(d, in, filt, bias, out, tab, stream);
-        case 4: return launch_tile<4, 4>(d, in, filt, bias, out, tab, stream);
-        case 5: return launch_tile<4, 2>(d, in, filt, bias, out, tab, stream);
-        case 6: return launch_tile<4, 1>(d, in, filt, bias, out, tab, stream);
-        case 7: return launch_tile<2, 2>(d, in, filt, bias, out, tab, stream);
-        case 8: return launch_tile<2, 1>(d, in, filt, bias, out, tab, stream);
+        case 0: return launch_tile<2, 4, 8, 8, 8>(d, in, filt, bias, out, tab, split, stream);
+        case 1: return launch_tile<2, 4, 8, 6, 16>(d, in, filt, bias, out, tab, split, stream);
+        case 2: return launch_tile<2, 2, 8, 8, 8>(d, in, filt, bias, out, tab, split, stream);
+        case 3: return launch_tile<2, 2, 8, 4, 8>(d, in, filt, bias, out, tab, split, stream);
+        case 4: return launch_tile<1, 2, 8, 8, 8>(d, in, filt, bias, out, tab, split, stream);
+        case 5: return launch_tile<1, 2, 8, 4, 8>(d, in, filt, bias, out, tab, split, stream);
+        case 6: return launch_tile<2, 1, 4, 4, 8>(d, in, filt, bias, out, tab, split, stream);
+        case 7: return launch_tile<1, 2, 4, 4, 16>(d, in, filt, bias, out, tab, split, stream);
+        case 8: return launch_tile<1, 1, 4, 4, 8>(d, in, filt, bias, out, tab, split, stream);
         case 9: return launch_pixel<8>(d, in, filt, bias, out, stream);
         case 10: return launch_pixel<16>(d, in, filt, bias, out, stream);
         case 11: return launch_pixel<32>(d, in, filt, bias, out, stream);
+        case 16: return launch_tile<1, 2, 8, 6, 8>(d, in, filt, bias, out, tab, split, stream);
+        case 17: return launch_tile<2, 2, 8, 6, 8>(d, in, filt, bias, out, tab, split, stream);
         default: return BODA_ERR_UNSUPPORTED;
     }
 }

@@ -1,0 +1,180 @@
+// Operand staging kernels.
+//
+// Bound: latency and HBM/L2 (a layer's input is read once and its staged copy written once; a few MB at the usual batch
+// sizes).  One launch handles the input and, on calls that bring their filters along, the filters too: the two re-layouts are
+// independent, so one of them runs under the other instead of behind it, and a launch less stands in front of the main kernel.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "stage.h"
+
+namespace boda {
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int kTilePx = 128;                 // points per input tile (32 channels): 16 loads in flight per thread
+constexpr int kTilePitch = kTilePx + 1;      // odd pitch: channel-quad reads hit distinct banks
+constexpr int kMaxSmemTaps = 36;             // filter taps staged through shared memory (8 warps x 32 channels x taps floats)
+
+__device__ __forceinline__ float rna(float x)
+{
+    uint32_t r;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+    return __uint_as_float(r);
+}
+
+// four consecutive channels of one staged row
+template <int MODE>
+__device__ __forceinline__ void put4(void* base, size_t row, int Cp, int c, float x0, float x1, float x2, float x3)
+{
+    if constexpr (MODE == STAGE_F16) {
+        const __half2 a = __floats2half2_rn(x0, x1), b = __floats2half2_rn(x2, x3);
+        *reinterpret_cast<uint2*>(static_cast<__half*>(base) + row * Cp + c) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    } else if constexpr (MODE == STAGE_FP32) {
+        *reinterpret_cast<float4*>(static_cast<float*>(base) + row * Cp + c) = make_float4(x0, x1, x2, x3);
+    } else {
+        float* dst = static_cast<float*>(base) + row * (MODE == STAGE_TF32_SPLIT ? 2 * Cp : Cp) + c;
+        const float4 hi = make_float4(rna(x0), rna(x1), rna(x2), rna(x3));
+        *reinterpret_cast<float4*>(dst) = hi;
+        if constexpr (MODE == STAGE_TF32_SPLIT)
+            *reinterpret_cast<float4*>(dst + Cp) = make_float4(rna(x0 - hi.x), rna(x1 - hi.y), rna(x2 - hi.z), rna(x3 - hi.w));
+    }
+}
+template <int MODE>
+__device__ __forceinline__ void put1(void* base, size_t row, int Cp, int c, float x)
+{
+    if constexpr (MODE == STAGE_F16) static_cast<__half*>(base)[row * Cp + c] = __float2half_rn(x);
+    else if constexpr (MODE == STAGE_FP32) static_cast<float*>(base)[row * Cp + c] = x;
+    else {
+        float* dst = static_cast<float*>(base) + row * (MODE == STAGE_TF32_SPLIT ? 2 * Cp : Cp) + c;
+        const float hi = rna(x);
+        dst[0] = hi;
+        if constexpr (MODE == STAGE_TF32_SPLIT) dst[Cp] = rna(x - hi);
+    }
+}
+
+// Blocks [0, filter_blocks) stage the filters, the rest the input.
+template <int MODE>
+__global__ void __launch_bounds__(kThreads)
+stage_kernel(const StageInput x, const StageFilters w, int filter_blocks, int m_tiles)
+{
+    extern __shared__ float sm[];
+    pdl_launch_dependents();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if ((int)blockIdx.x >= filter_blocks) {
+        // ---- input: 128 points (numbered through all images) x 32 channels, transposed through shared memory
+        const int b = (int)blockIdx.x - filter_blocks;
+        const int bc = b / m_tiles;
+        const int px0 = (b - bc * m_tiles) * kTilePx, c0 = 32 * bc;
+        const long long M = (long long)x.N * x.HW;
+        const int px = tid & (kTilePx - 1), ch = tid / kTilePx;          // channels ch, ch + 2, ...
+        const long long m = (long long)px0 + px;
+        const bool ok = m < M;
+        const int n = ok ? (int)(m / x.HW) : 0;
+        const float* src = x.in + ((size_t)n * x.C + c0 + ch) * x.HW + (ok ? (int)(m - (long long)n * x.HW) : 0);
+        pdl_wait();
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = (ok && c0 + ch + 2 * i < x.C) ? __ldg(src + (size_t)(2 * i) * x.HW) : 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sm[(ch + 2 * i) * kTilePitch + px] = v[i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int p = (tid >> 3) + 32 * i, c = 4 * (tid & 7);
+            if (px0 + (long long)p < M) {
+                const float* t = sm + c * kTilePitch + p;
+                put4<MODE>(x.xp, (size_t)px0 + p, x.Cp, c0 + c, t[0], t[kTilePitch], t[2 * kTilePitch], t[3 * kTilePitch]);
+            }
+        }
+        return;
+    }
+    pdl_wait();
+    if (w.RS == 1) {
+        // ---- 1x1 filters are [K][C] rows already: a copy with rounding and padding, 512 consecutive channels' worth per warp
+        const long long total = (long long)w.K * w.Cp;
+        const long long base = ((long long)blockIdx.x * 8 + warp) * 512;
+        float v[16];
+        const int k0 = (int)(base / w.Cp), r0 = (int)(base - (long long)k0 * w.Cp);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            int k = k0, c = r0 + lane + 32 * i;
+            while (c >= w.Cp) { c -= w.Cp; ++k; }
+            v[i] = (k < w.K && c < w.C) ? __ldg(w.filt + (size_t)k * w.C + c) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            int k = k0, c = r0 + lane + 32 * i;
+            while (c >= w.Cp) { c -= w.Cp; ++k; }
+            if (base + lane + 32 * i < total) put1<MODE>(w.wp, (size_t)k, w.Cp, c, v[i]);
+        }
+        return;
+    }
+    // ---- filters: a warp takes 32 channels of one output channel: 32*RS consecutive floats in, RS rows of 32 channels out
+    const int cblocks = w.Cp >> 5;
+    const long long unit = (long long)blockIdx.x * 8 + warp;
+    if (unit >= (long long)w.K * cblocks) return;
+    const int k = (int)(unit / cblocks), c0 = 32 * (int)(unit - (long long)k * cblocks);
+    const float* src = w.filt + ((size_t)k * w.C + c0) * w.RS;
+    const int live = min(32, w.C - c0);                                  // channels that exist (may be 0 or less)
+    if (w.RS <= kMaxSmemTaps) {
+        float* s = sm + warp * 32 * w.RS;
+        const int n = max(live, 0) * w.RS;
+        int i = lane;
+        for (; i + 96 < 32 * w.RS; i += 128) {
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = i + 32 * u < n ? __ldg(src + i + 32 * u) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s[i + 32 * u] = v[u];
+        }
+        for (; i < 32 * w.RS; i += 32) s[i] = i < n ? __ldg(src + i) : 0.f;
+        __syncwarp();
+        for (int t = 0; t < w.RS; ++t) put1<MODE>(w.wp, (size_t)t * w.K + k, w.Cp, c0 + lane, s[lane * w.RS + t]);
+    } else {
+#pragma unroll 4
+        for (int t = 0; t < w.RS; ++t)
+            put1<MODE>(w.wp, (size_t)t * w.K + k, w.Cp, c0 + lane, lane < live ? __ldg(src + lane * w.RS + t) : 0.f);
+    }
+}
+
+}  // namespace
+
+int stage_operands(StageMode mode, const StageInput* input, const StageFilters* filters, cudaStream_t stream)
+{
+    StageInput x = {nullptr, nullptr, 0, 0, 0, 1};
+    StageFilters w = {nullptr, nullptr, 0, 0, 0, 1};
+    long long fblocks = 0, m_tiles = 1, iblocks = 0;
+    size_t smem = 0;
+    if (filters) {
+        w = *filters;
+        if (w.RS == 1) {
+            fblocks = ((long long)w.K * w.Cp + 8 * 512 - 1) / (8 * 512);
+        } else {
+            fblocks = ((long long)w.K * (w.Cp / 32) + 7) / 8;
+            if (w.RS <= kMaxSmemTaps) smem = (size_t)8 * 32 * w.RS * sizeof(float);
+        }
+    }
+    if (input) {
+        x = *input;
+        m_tiles = ((long long)x.N * x.HW + kTilePx - 1) / kTilePx;
+        iblocks = m_tiles * (x.Cp / 32);
+        smem = std::max(smem, (size_t)32 * kTilePitch * sizeof(float));
+    }
+    if (fblocks + iblocks > 0x7fffffffLL) return BODA_ERR_TOO_LARGE;
+    const dim3 grid((unsigned)(fblocks + iblocks)), block(kThreads);
+    cudaError_t e;
+    switch (mode) {
+        case STAGE_TF32: e = launch_kernel(stage_kernel<STAGE_TF32>, grid, block, smem, stream, 1, x, w, (int)fblocks, (int)m_tiles); break;
+        case STAGE_TF32_SPLIT: e = launch_kernel(stage_kernel<STAGE_TF32_SPLIT>, grid, block, smem, stream, 1, x, w, (int)fblocks, (int)m_tiles); break;
+        case STAGE_F16: e = launch_kernel(stage_kernel<STAGE_F16>, grid, block, smem, stream, 1, x, w, (int)fblocks, (int)m_tiles); break;
+        default: e = launch_kernel(stage_kernel<STAGE_FP32>, grid, block, smem, stream, 1, x, w, (int)fblocks, (int)m_tiles); break;
+    }
+    if (e != cudaSuccess) return record_cuda_error(e, "stage_kernel");
+    count_launch();
+    return BODA_OK;
+}
+
+}  // namespace boda

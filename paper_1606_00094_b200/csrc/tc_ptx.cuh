@@ -39,7 +39,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 // Bounded wait.  Returns false if the CTA is aborting or the limit expired (then it raises the abort flag
 // and records where it gave up).  The limit is counted on the SM's own cycle counter, which is cheap to read
 // (the global nanosecond timer is not, and must stay out of the fast path): 4e9 cycles, about two seconds.
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int where)
+static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int where)
 {
     long long t0 = 0;
     for (uint32_t spin = 1;; ++spin) {
@@ -69,7 +69,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // Bounded wait for threads that are not on the critical path (the epilogue waiting for the accumulator):
 // polls rarely and sleeps in between, so that it does not compete with the producer's and the MMA issuer's
 // barrier traffic.  The limit is the same number of cycles, counted in sleep quanta.
-__device__ __noinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int where)
+static __device__ __noinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int where)
 {
     const long long t0 = clock64();
     for (;;) {

@@ -19,7 +19,6 @@
 // Every wait is bounded (4e9 SM cycles, about two seconds): on expiry the kernel records BODA_ERR_DEVICE_TIMEOUT in the
 // status word, all roles leave their loops, tensor memory is released and the CTA returns.
 #include <cuda.h>
-#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <cstdio>
@@ -29,6 +28,7 @@
 #include <vector>
 
 #include "igemm_tf32.h"
+#include "stage.h"
 #include "tc_ptx.cuh"
 #include "tconv_halo.cuh"
 #include "gconv_tf32.cuh"
@@ -487,67 +487,11 @@ igemm_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 }
 
 // ------------------------------------------------------------------------------------------------
-// Operand staging ("input transformation", Section 5): NCHW -> NHWC with channels padded to a multiple of
-// 32 and values rounded to TF32 (round to nearest, ties away), so that the tensor core's truncation of the
-// low mantissa bits is exact.
 __device__ __forceinline__ float round_tf32(float x)
 {
     uint32_t r;
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
     return __uint_as_float(r);
-}
-
-// With `split` the row holds 2*Cp values: the TF32-rounded value hi at channel c and the rounded remainder
-// lo = rna(x - hi) at channel Cp + c (error-compensated mode: x = hi + lo up to 2^-22 relative).
-__global__ void __launch_bounds__(256)
-pack_input_nhwc_kernel(const float* __restrict__ in, float* __restrict__ xp, int C, int Cp, int HW, int split)
-{
-    __shared__ float tile[32][33];
-    pdl_launch_dependents();
-    pdl_wait();
-    const int n = blockIdx.z;
-    const int hw0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;          // 32 x 8
-    const float* src = in + (size_t)n * C * HW;
-    const int Cs = split ? 2 * Cp : Cp;
-    float* dst = xp + (size_t)n * HW * Cs;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int c = c0 + ty + 8 * i, hw = hw0 + tx;
-        tile[ty + 8 * i][tx] = (c < C && hw < HW) ? __ldg(src + (size_t)c * HW + hw) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int hw = hw0 + ty + 8 * i, c = c0 + tx;
-        if (hw < HW) {
-            const float x = tile[tx][ty + 8 * i];
-            const float hi = round_tf32(x);
-            dst[(size_t)hw * Cs + c] = hi;
-            if (split) dst[(size_t)hw * Cs + Cp + c] = round_tf32(x - hi);
-        }
-    }
-}
-
-// filters KCRS -> [R*S][K][Cp], TF32-rounded, zero in the padded channels
-__global__ void __launch_bounds__(256)
-pack_filters_kernel(const float* __restrict__ filt, float* __restrict__ wp, int K, int C, int Cp, int RS, int split)
-{
-    pdl_launch_dependents();
-    pdl_wait();
-    const long long total = (long long)RS * K * Cp;
-    const int Cs = split ? 2 * Cp : Cp;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(idx % Cp);
-        const long long t = idx / Cp;
-        const int k = (int)(t % K);
-        const int tap = (int)(t / K);
-        const float x = c < C ? __ldg(filt + ((size_t)k * C + c) * RS + tap) : 0.f;
-        const float hi = round_tf32(x);
-        wp[t * Cs + c] = hi;
-        if (split) wp[t * Cs + Cp + c] = round_tf32(x - hi);         // see pack_input_nhwc_kernel
-    }
 }
 
 // Space-to-depth staging for strided layers.  A convolution with stride t on C channels equals a stride-1
@@ -1482,95 +1426,31 @@ void igemm_plan_describe(const IgemmPlan* p, char* buf, size_t n)
                   p->splits, p->tiles_m, p->tiles_n, p->splits);
 }
 
-// fp16 operand staging (reduced-precision storage, the paper's Section 2 remark on 16-bit storage): the same two
-// re-layouts with the values rounded to fp16 (nearest even) and channels padded to a multiple of 64
-__global__ void __launch_bounds__(256)
-pack_input_nhwc_half_kernel(const float* __restrict__ in, __half* __restrict__ xp, int C, int Cp, int HW)
-{
-    __shared__ float tile[32][33];
-    pdl_launch_dependents();
-    pdl_wait();
-    const int n = blockIdx.z;
-    const int hw0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const float* src = in + (size_t)n * C * HW;
-    __half* dst = xp + (size_t)n * HW * Cp;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int c = c0 + ty + 8 * i, hw = hw0 + tx;
-        tile[ty + 8 * i][tx] = (c < C && hw < HW) ? __ldg(src + (size_t)c * HW + hw) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int hw = hw0 + ty + 8 * i, c = c0 + tx;
-        if (hw < HW) dst[(size_t)hw * Cp + c] = __float2half_rn(tile[tx][ty + 8 * i]);
-    }
-}
-
-__global__ void __launch_bounds__(256)
-pack_filters_half_kernel(const float* __restrict__ filt, __half* __restrict__ wp, int K, int C, int Cp, int RS)
-{
-    pdl_launch_dependents();
-    pdl_wait();
-    const long long total = (long long)RS * K * Cp;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(idx % Cp);
-        const long long t = idx / Cp;
-        const int k = (int)(t % K);
-        const int tap = (int)(t / K);
-        wp[idx] = __float2half_rn(c < C ? __ldg(filt + ((size_t)k * C + c) * RS + tap) : 0.f);
-    }
-}
-
-// 1x1 filters with C a multiple of 4 are already [K][C] rows: the staging is a rounding copy, 16 bytes per thread
-__global__ void __launch_bounds__(256)
-pack_filters_1x1_kernel(const float4* __restrict__ filt, float* __restrict__ wp, int K, int C4, int Cp, int split)
-{
-    pdl_launch_dependents();
-    pdl_wait();
-    const int Cs = split ? 2 * Cp : Cp, Cp4 = Cp >> 2;
-    const int total = K * Cp4;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-        const int k = idx / Cp4, c4 = idx - k * Cp4;
-        const float4 x = c4 < C4 ? __ldg(filt + (size_t)k * C4 + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 hi = make_float4(round_tf32(x.x), round_tf32(x.y), round_tf32(x.z), round_tf32(x.w));
-        float* row = wp + (size_t)k * Cs;
-        reinterpret_cast<float4*>(row)[c4] = hi;
-        if (split)
-            reinterpret_cast<float4*>(row + Cp)[c4] = make_float4(round_tf32(x.x - hi.x), round_tf32(x.y - hi.y),
-                                                                  round_tf32(x.z - hi.z), round_tf32(x.w - hi.w));
-    }
-}
+static StageMode stage_mode(const IgemmPlan* p) { return p->half ? STAGE_F16 : p->terms == 3 ? STAGE_TF32_SPLIT : STAGE_TF32; }
+// Does the plan's kernel read its filters as plain [R*S][K][Cp] rows (stage_operands)?  The others have a layout of their own.
+static bool plain_filters(const IgemmPlan* p) { return p->nacc != -3 && p->nacc != -1 && !p->s2d; }
+static StageFilters stage_filters(const IgemmPlan* p, const float* filt) { return {filt, p->d_wp, p->d.K, p->d.C, p->Cp, p->d.R * p->d.S}; }
 
 static int pack_filters(IgemmPlan* p, const float* filt, cudaStream_t stream)
 {
     const ConvDims& d = p->d;
-    const long long total = (long long)d.R * d.S * d.K * p->Cp;
-    const int blocks = (int)std::min<long long>((total + 255) / 256, 148 * 8);
+    if (plain_filters(p)) {
+        const StageFilters w = stage_filters(p, filt);
+        return stage_operands(stage_mode(p), nullptr, &w, stream);
+    }
     if (p->nacc == -3) {
         const int fblocks = std::min((p->fl_Rb * p->fl_Sb * d.K * first::kViewChannels + 255) / 256, 148 * 8);
         BODA_CUDA_TRY(launch_kernel(first::pack_filters_first_layer_kernel, dim3(fblocks), dim3(256), 0, stream, 1, filt, p->d_wp,
                                     d.K, d.R, d.S, p->fl_Rb, p->fl_Sb));
-    } else if (p->half) {
-        BODA_CUDA_TRY(launch_kernel(pack_filters_half_kernel, dim3(blocks), dim3(256), 0, stream, 1, filt, reinterpret_cast<__half*>(p->d_wp),
-                                    d.K, d.C, p->Cp, d.R * d.S));
     } else if (p->nacc == -1) {
         const int Kp = p->gather_chunks * 32;
         const int gblocks = (int)std::min<long long>(((long long)d.K * Kp + 255) / 256, 148 * 8);
         BODA_CUDA_TRY(launch_kernel(pack_filters_flat_kernel, dim3(gblocks), dim3(256), 0, stream, 1, filt, p->d_wp, d.K, d.Kred, Kp));
-    } else if (p->s2d) {
+    } else {
         const ConvDims& o = p->orig;
+        const int blocks = (int)std::min<long long>(((long long)d.R * d.S * d.K * p->Cp + 255) / 256, 148 * 8);
         BODA_CUDA_TRY(launch_kernel(pack_filters_s2d_kernel, dim3(blocks), dim3(256), 0, stream, 1, filt, p->d_wp, o.K, o.C, o.R,
                                     o.S, o.stride, d.R, d.S, p->Cp));
-    } else if (d.R * d.S == 1 && d.C % 4 == 0 && ((uintptr_t)filt & 15) == 0 && (long long)d.K * p->Cp < (1LL << 31)) {
-        const int blocks4 = (int)std::min<long long>((total / 4 + 255) / 256, 148 * 8);
-        BODA_CUDA_TRY(launch_kernel(pack_filters_1x1_kernel, dim3(blocks4), dim3(256), 0, stream, 1,
-                                    reinterpret_cast<const float4*>(filt), p->d_wp, d.K, d.C / 4, p->Cp, p->terms == 3 ? 1 : 0));
-    } else {
-        BODA_CUDA_TRY(launch_kernel(pack_filters_kernel, dim3(blocks), dim3(256), 0, stream, 1, filt, p->d_wp, d.K, d.C, p->Cp,
-                                    d.R * d.S, p->terms == 3 ? 1 : 0));
     }
     count_launch();
     return BODA_OK;
@@ -1680,9 +1560,11 @@ int igemm_launch(IgemmPlan* p, const float* in, const float* filt, const float* 
     if (needs_staging && !workspace) return BODA_ERR_NOMEM;
     if (needs_staging && ((uintptr_t)workspace & 255) != 0) return BODA_ERR_INVALID_ARG;
     float* xp = p->in_packed ? const_cast<float*>(in) : (float*)workspace;
-    if (filt != p->bound_filt || !filt) {
-        if (!filt) return BODA_ERR_INVALID_ARG;
-        int rc = pack_filters(p, filt, stream);       // unbound: re-layout on every call
+    if (!filt) return BODA_ERR_INVALID_ARG;
+    const bool bound = filt == p->bound_filt;         // unbound: re-layout on every call
+    const bool stage_both = !bound && p->nacc == 0 && !p->s2d && !p->in_packed;     // in one launch with the input, below
+    if (!bound && !stage_both) {
+        const int rc = pack_filters(p, filt, stream);
         if (rc != BODA_OK) return rc;
     }
     if (p->nacc == -3) {
@@ -1797,13 +1679,10 @@ int igemm_launch(IgemmPlan* p, const float* in, const float* filt, const float* 
         }
     }
     if (!p->s2d && !p->in_packed) {
-        const int HW = d.H * d.W;
-        dim3 grid((HW + 31) / 32, p->Cp / 32, d.N);
-        if (p->half)
-            BODA_CUDA_TRY(launch_kernel(pack_input_nhwc_half_kernel, grid, dim3(256), 0, stream, 1, in, reinterpret_cast<__half*>(xp), d.C, p->Cp, HW));
-        else
-            BODA_CUDA_TRY(launch_kernel(pack_input_nhwc_kernel, grid, dim3(256), 0, stream, 1, in, xp, d.C, p->Cp, HW, p->terms == 3 ? 1 : 0));
-        count_launch();
+        const StageInput x = {in, xp, d.N, d.C, p->Cp, d.H * d.W};
+        const StageFilters w = stage_filters(p, filt);
+        const int rc = stage_operands(stage_mode(p), &x, stage_both ? &w : nullptr, stream);
+        if (rc != BODA_OK) return rc;
     }
     if (p->map_a_base != xp) {
         int rc = encode_map_a(p, xp);
@@ -1910,15 +1789,12 @@ int igemm_run_in_region(const ConvDims& d, int variant, const float* in, const f
     BODA_CUDA_TRY(cudaMemsetAsync(base, 0, head_bytes, stream));      // the status word starts at zero
     rc = encode_map_b(p);
     if (rc == BODA_OK) rc = encode_map_a(p, xp);
-    if (rc == BODA_OK) rc = pack_filters(p, filt, stream);
-    if (rc != BODA_OK) { p->d_wp = nullptr; return rc; }
-    {
-        const int HW = d.H * d.W;
-        dim3 grid((HW + 31) / 32, p->Cp / 32, d.N);
-        cudaError_t e = launch_kernel(pack_input_nhwc_kernel, grid, dim3(256), 0, stream, 1, in, xp, d.C, p->Cp, HW, 0);
-        if (e != cudaSuccess) { p->d_wp = nullptr; return record_cuda_error(e, "pack_input_nhwc_kernel"); }
-        count_launch();
+    if (rc == BODA_OK) {
+        const StageInput x = {in, xp, d.N, d.C, p->Cp, d.H * d.W};
+        const StageFilters w = stage_filters(p, filt);
+        rc = stage_operands(STAGE_TF32, &x, &w, stream);
     }
+    if (rc != BODA_OK) { p->d_wp = nullptr; return rc; }
     IgemmParams prm;
     prm.M = d.M; prm.stride = d.stride; prm.pad = d.pad; prm.S = d.S;
     prm.cchunks = p->Cp / BKC;

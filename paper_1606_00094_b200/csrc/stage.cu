@@ -69,12 +69,12 @@ stage_kernel(const StageInput x, const StageFilters w, int filter_blocks, int m_
         const int b = (int)blockIdx.x - filter_blocks;
         const int bc = b / m_tiles;
         const int px0 = (b - bc * m_tiles) * PX, c0 = 32 * bc;
-        const long long M = (long long)x.N * x.HW;
+        const unsigned M = (unsigned)x.N * (unsigned)x.HW;              // tensors hold at most 2^31 elements
         const int px = tid & (PX - 1), ch = tid / PX;          // channels ch, ch + STEP, ...
-        const long long m = (long long)px0 + px;
+        const unsigned m = (unsigned)(px0 + px);
         const bool ok = m < M;
-        const int n = ok ? (int)(m / x.HW) : 0;
-        const float* src = x.in + ((size_t)n * x.C + c0 + ch) * x.HW + (ok ? (int)(m - (long long)n * x.HW) : 0);
+        const unsigned n = ok ? m / (unsigned)x.HW : 0u;
+        const float* src = x.in + ((size_t)n * x.C + c0 + ch) * x.HW + (ok ? m - n * (unsigned)x.HW : 0u);
         pdl_wait();
         float v[LOADS];
 #pragma unroll
@@ -85,7 +85,7 @@ stage_kernel(const StageInput x, const StageFilters w, int filter_blocks, int m_
 #pragma unroll
         for (int i = 0; i < PX / 32; ++i) {
             const int p = (tid >> 3) + 32 * i, c = 4 * (tid & 7);
-            if (px0 + (long long)p < M) {
+            if ((unsigned)(px0 + p) < M) {
                 const float* t = sm + c * PITCH + p;
                 put4<MODE>(x.xp, (size_t)px0 + p, x.Cp, c0 + c, t[0], t[PITCH], t[2 * PITCH], t[3 * PITCH]);
             }
@@ -159,13 +159,14 @@ int stage_operands(StageMode mode, const StageInput* input, const StageFilters* 
         }
     }
     // Wide tiles keep more loads in flight per thread and win once they fill the SMs a few times over; below, narrow tiles
-    // spread the same loads over more blocks.  Measured, whole layer: 3x3 on 256 channels, 13x13, batch 20 (27 x 8 wide tiles)
-    // 20.8 us wide, 19.5 narrow; 93.7 us against 90.3 wide with an 11 MB input.
+    // spread the same loads over more blocks.  Measured, whole layer: 3x3 on 256 channels, 13x13, batch 20 (216 wide tiles)
+    // 20.8 us wide, 19.0 narrow; 49x51 on 97 channels (320) 12.7 wide, 13.1 narrow; 39x39 on 333, batch 8 (1140) 15.2 / 18.0.
+    // The split staging writes twice as much per load: 41x41 on 32 channels, batch 31 (408) 30.1 wide, 29.4 narrow.
     bool wide = false;
     if (input) {
         x = *input;
         const long long M = (long long)x.N * x.HW;
-        wide = (M + 127) / 128 * (x.Cp / 32) >= 148 * 8;
+        wide = (M + 127) / 128 * (x.Cp / 32) >= (mode == STAGE_TF32_SPLIT ? 148 * 8 : 148 * 2);
         const int px = wide ? 128 : 32;
         m_tiles = (M + px - 1) / px;
         iblocks = m_tiles * (x.Cp / 32);

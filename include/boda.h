@@ -101,7 +101,8 @@ typedef struct boda_plan_opts {
                                     (K1CONV by TMA straight from NCHW; split_k > 1: a cluster split over the input
                                     channels), 23..25 first_512x64/96/128 (TCONV for 3 input channels, stride 4, no
                                     padding, windows up to 11x11: the space-to-depth view built in shared memory
-                                    straight from NCHW, nothing staged).  A tile that cannot run the shape is refused
+                                    straight from NCHW, nothing staged), 26..30 pair_256x64/96/128/192/256 (the im2col
+                                    operands on pairs of SMs, no split).  A tile that cannot run the shape is refused
                                     with BODA_ERR_UNSUPPORTED. */
     int split_k;                 /* 0: automatic; otherwise the number of reduction splits (tensor-core variants and the GEMM-blocked
                                     FP32 tiles) */

@@ -47,12 +47,12 @@ int record_cuda_error(cudaError_t e, const char* what);
 // ---- kernel launch helper
 // Every kernel of the library is launched with programmatic dependent launch: it calls pdl_launch_dependents()
 // at once and pdl_wait() before it first touches global memory that an earlier kernel on the stream may have
-// written (or may still read), so its prologue overlaps the previous kernel's tail.  cluster_z > 1 groups the
-// CTAs along grid.z into a thread-block cluster.  BODA_NO_PDL=1 in the environment turns the overlap off.
+// written (or may still read), so its prologue overlaps the previous kernel's tail.  `cluster` (or cluster_z along grid.z)
+// groups the CTAs into thread-block clusters.  BODA_NO_PDL=1 in the environment turns the overlap off.
 bool pdl_enabled();
 
 template <typename Kernel, typename... Args>
-cudaError_t launch_kernel(Kernel kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster_z, Args... args)
+cudaError_t launch_clusters(Kernel kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, dim3 cluster, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -61,11 +61,11 @@ cudaError_t launch_kernel(Kernel kernel, dim3 grid, dim3 block, size_t smem, cud
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     unsigned n = 0;
-    if (cluster_z > 1) {
+    if (cluster.x * cluster.y * cluster.z > 1) {
         attr[n].id = cudaLaunchAttributeClusterDimension;
-        attr[n].val.clusterDim.x = 1;
-        attr[n].val.clusterDim.y = 1;
-        attr[n].val.clusterDim.z = (unsigned)cluster_z;
+        attr[n].val.clusterDim.x = cluster.x;
+        attr[n].val.clusterDim.y = cluster.y;
+        attr[n].val.clusterDim.z = cluster.z;
         ++n;
     }
     if (pdl_enabled()) {
@@ -76,6 +76,11 @@ cudaError_t launch_kernel(Kernel kernel, dim3 grid, dim3 block, size_t smem, cud
     cfg.attrs = attr;
     cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename Kernel, typename... Args>
+cudaError_t launch_kernel(Kernel kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster_z, Args... args)
+{
+    return launch_clusters(kernel, grid, block, smem, stream, dim3(1, 1, (unsigned)cluster_z), args...);
 }
 
 // cudaFuncSetAttribute applies to the current device only: a kernel's dynamic shared-memory limit is raised once per

@@ -34,6 +34,7 @@
 #include "gconv_tf32.cuh"
 #include "k1nchw_tf32.cuh"
 #include "tconv_first_layer.cuh"
+#include "pair_conv.cuh"
 
 namespace boda {
 namespace {
@@ -663,10 +664,11 @@ int load_driver_entry_points()
 // with NACC accumulators of 128 rows each (ids 5..8: 1, 9..12: 2, 13..15: 4).
 // accumulators per tile: 0 = im2col kernel, 1 / 2 / 4 = halo kernel, -1 = gather kernel (gconv_tf32.cuh)
 // Ids 20..22: 1x1 layers by TMA straight from NCHW (k1nchw_tf32.cuh), accumulator code -2.
+// Ids 26..30: the im2col operands on CTA pairs (pair_conv.cuh; 256 points per tile), accumulator code -4.
 // Ids 23..25: first-layer kernel (tconv_first_layer.cuh; 3 channels, stride 4, straight from NCHW), accumulator code -3.
 constexpr int kTileBN[] = {64, 96, 128, 192, 256, /*halo*/ 64, 128, 192, 256, 96, 128, 192, 256, 64, 96, 128, /*gather*/ 64, 96, 128, 192,
-                           /*1x1 from NCHW*/ 64, 128, 192, /*first layer*/ 64, 96, 128};
-constexpr int kTileNacc[] = {0, 0, 0, 0, 0, 1, 1, 1, 1, 2, 2, 2, 2, 4, 4, 4, -1, -1, -1, -1, -2, -2, -2, -3, -3, -3};
+                           /*1x1 from NCHW*/ 64, 128, 192, /*first layer*/ 64, 96, 128, /*CTA pairs*/ 64, 96, 128, 192, 256};
+constexpr int kTileNacc[] = {0, 0, 0, 0, 0, 1, 1, 1, 1, 2, 2, 2, 2, 4, 4, 4, -1, -1, -1, -1, -2, -2, -2, -3, -3, -3, -4, -4, -4, -4, -4};
 constexpr int kFirstK1nTile = 20;
 constexpr int kFirstGatherTile = 16;
 constexpr int kNumIgemmTiles = sizeof(kTileBN) / sizeof(kTileBN[0]);
@@ -684,6 +686,7 @@ struct IgemmPlan {
     int BN = 128;
     int Cp = 0;
     int terms = 1;                   // 3: error-compensated TF32, staged operands hold hi and lo parts (2*Cp channels)
+    bool pair = false;               // CTA pairs (pair_conv.cuh); otherwise a plan of the im2col kernel (nacc == 0)
     bool half = false;               // fp16 operands: staged tensors hold __half, Cp is a multiple of 64
     int Cs() const { return terms == 3 ? 2 * Cp : Cp; }
     int esize() const { return half ? 2 : 4; }            // bytes per staged operand element
@@ -808,7 +811,7 @@ namespace {
 
 // Cost model (SM clocks) used when a plan is not tuned by timing; fitted to a sweep of every tile and split over
 // fourteen layer shapes on B200 (its choice is within 3 % of the best measured one for each of them).
-//   main loop: a stage costs the MMAs' 2*BN clocks or about 380 clocks of producer / issuer hand-shakes, whichever
+//   main loop: a stage costs about 2.1*BN clocks of MMAs or 380 of producer / issuer hand-shakes, whichever
 //              is longer (halo kernel: 2.2*BN per accumulator, or 290 per accumulator + 390);
 //   fixed:     prologue, pipeline fill and tail, about 3500 clocks (halo kernel 5000);
 //   epilogue:  32 clocks per channel without a split (the SM writes about 32 bytes per clock); with a split by
@@ -845,7 +848,7 @@ double model_cost(const ConvDims& d, int Cp, int BN, int splits)
     const int ips = (iters + splits - 1) / splits;
     const int se = (iters + ips - 1) / ips;
     const long long tm = (d.M + BM - 1) / BM, tn = (d.K + BN - 1) / BN;
-    const double per_iter = std::max(2.0 * BN, 380.0);
+    const double per_iter = std::max(2.1 * BN, 380.0);
     return wave_count((double)tm * tn, se) * (ips * per_iter + 3500.0 + epilogue_cost(BN, se, split_exchange_fits(BN, se, stage_region_of(BN))));
 }
 
@@ -858,6 +861,13 @@ double model_cost_halo(const ConvDims& d, int Cp, int BN, int nacc, int splits)
     const long long tm = (mflat + 128 * nacc - 1) / (128 * nacc), tn = (d.K + BN - 1) / BN;
     const double per_iter = std::max(2.2 * BN * nacc, 290.0 * nacc + 390.0);
     return wave_count((double)tm * tn, se) * (ips * per_iter + 5000.0 + nacc * epilogue_cost(BN, se, false));
+}
+
+// The input staging kernel the im2col, halo and pair tiles need and the gather tiles do not: a launch, or the time to read
+// the input and write its staged copy (about 3000 bytes per clock measured on staging kernels).
+double staging_cost(const ConvDims& layer, const ConvDims& view, int Cp)
+{
+    return std::max(6000.0, ((double)layer.N * layer.C * layer.H * layer.W + (double)view.N * view.H * view.W * Cp) * 4.0 / 3000.0);
 }
 
 // Gather kernel: persistent over ceil(M/128) * ceil(K/BN) tiles.  Measured: a 32-index reduction step costs about
@@ -972,6 +982,26 @@ double model_cost_k1n(const ConvDims& d, int BN, int sm_count, int splits = 1)
     return per_cta * steps * std::max(2.0 * BN, 410.0) + 3500.0 + 32.0 * BN;
 }
 
+// MMA steps (8 TF32 or 16 fp16 channels) of a tap's last chunk that hold channels
+int last_ksteps(const ConvDims& d, int chunk, bool half)
+{
+    const int kstep = half ? 16 : 8, last = d.C - (d.C - 1) / chunk * chunk;
+    return (last + kstep - 1) / kstep;
+}
+
+// CTA pairs: persistent over ceil(M/256) * ceil(K/BN) tiles, one accumulator under way while the other is stored.  Clocks per
+// reduction step measured with every SM busy, `full` for a whole chunk and `quarter` where one MMA step of the chunk holds channels
+// (then the loads set the pace); `last` of the four steps hold channels in a tap's last chunk.
+double model_cost_pair(const ConvDims& d, int BN, int taps, int cchunks, int last, int sm_count)
+{
+    const long long tiles = (long long)((d.M + 255) / 256) * ((d.K + BN - 1) / BN);
+    const double rounds = (double)((tiles + sm_count / 2 - 1) / (sm_count / 2));
+    const double full = BN <= 64 ? 270.0 : BN <= 96 ? 315.0 : BN <= 128 ? 345.0 : BN <= 192 ? 405.0 : 525.0;
+    const double quarter = 220.0 + 0.77 * BN;
+    const double per_tile = taps * ((cchunks - 1) * full + std::max(quarter, full * last / 4.0));
+    return rounds * per_tile + 5000.0 + 32.0 * BN;
+}
+
 int encode_map_a_k1n(IgemmPlan* p, const void* in)
 {
     const ConvDims& d = p->d;
@@ -1016,6 +1046,23 @@ int launch_first_layer(IgemmPlan* p, const first::FirstParams& prm, cudaStream_t
     dim3 grid(p->tiles_m, p->tiles_n, 1);
     BODA_CUDA_TRY(launch_kernel(first::tconv_first_layer_kernel<BN>, grid, dim3(first::kThreads), (size_t)smem, stream, 1,
                                 p->map_b, p->map_b1, prm));
+    count_launch();
+    return BODA_OK;
+}
+
+template <int BN>
+int launch_pair(IgemmPlan* p, const pair::PairParams& prm, cudaStream_t stream)
+{
+    using C = pair::Cfg<BN>;
+    auto run = [&](auto kernel, DeviceSmemLimit& limit) -> cudaError_t {
+        const int smem = C::smem_bytes(prm.out_tma != 0);
+        const cudaError_t e = limit.ensure(kernel, (size_t)smem);
+        if (e != cudaSuccess) return e;
+        return launch_clusters(kernel, dim3(2 * std::min(prm.tiles_total, p->sm_count / 2)), dim3(pair::kThreads), (size_t)smem, stream,
+                               dim3(2, 1, 1), p->map_a, p->map_b, p->map_o, prm);
+    };
+    static DeviceSmemLimit limit_tf32, limit_f16;
+    BODA_CUDA_TRY(p->half ? run(pair::pair_conv_kernel<BN, true>, limit_f16) : run(pair::pair_conv_kernel<BN, false>, limit_tf32));
     count_launch();
     return BODA_OK;
 }
@@ -1154,7 +1201,7 @@ int encode_map_b(IgemmPlan* p)
     const cuuint64_t Cs = (cuuint64_t)p->Cs(), es = (cuuint64_t)p->esize();
     const cuuint64_t dims[3] = {Cs, (cuuint64_t)d.K, (cuuint64_t)(d.R * d.S)};
     const cuuint64_t strides[2] = {Cs * es, (cuuint64_t)d.K * Cs * es};
-    const cuuint32_t box[3] = {(cuuint32_t)p->chunk(), (cuuint32_t)p->BN, 1};
+    const cuuint32_t box[3] = {(cuuint32_t)p->chunk(), (cuuint32_t)(p->pair ? p->BN / 2 : p->BN), 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = g_encode_tiled(&p->map_b, p->half ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, p->d_wp, dims, strides, box, estr,
                                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1228,6 +1275,13 @@ int igemm_plan_create(const ConvDims& d_in, int variant, int tile_id, int split_
     for (int t = 0; t < kNumIgemmTiles; ++t) {
         if (tile_id >= 0 && t != tile_id) continue;
         const int nacc = kTileNacc[t];
+        if (nacc == -4) {
+            if (mode == 1 || split_k > 1) continue;
+            if (max_ws > 0 && (((size_t)d.N * d.H * d.W * p->Cs() * p->esize() + 1023) & ~(size_t)1023) > max_ws) continue;
+            const double c = staging_cost(d_in, d, p->Cp) + model_cost_pair(d, kTileBN[t], d.R * d.S, p->Cp / p->chunk(), last_ksteps(d, p->chunk(), p->half), p->sm_count);
+            if (c < best) { best = c; best_t = t; best_s = 1; }
+            continue;
+        }
         if (nacc == -3) {
             if (s2d == 0 || split_k > 1 || !first_layer_geometry(d_in, variant, x3, kTileBN[t], nullptr)) continue;
             const double c = model_cost_first_layer(d_in, kTileBN[t], p->sm_count);
@@ -1260,10 +1314,7 @@ int igemm_plan_create(const ConvDims& d_in, int variant, int tile_id, int split_
         for (int s : kSplitCandidates) {
             if (split_k > 0 && s != split_k) continue;
             if (s > p->iters_total) continue;
-            // the input staging kernel these tiles need and the gather tiles do not: a launch, or the time to read
-            // the input and write its staged copy (about 3000 bytes per clock measured on staging kernels)
-            const double staging = std::max(6000.0, ((double)d_in.N * d_in.C * d_in.H * d_in.W + (double)d.N * d.H * d.W * p->Cp) * 4.0 / 3000.0);
-            const double c = staging + (nacc > 0 ? model_cost_halo(d, p->Cp, kTileBN[t], nacc, s) : model_cost(d, p->Cp * p->terms / (p->half ? 2 : 1), kTileBN[t], s));
+            const double c = staging_cost(d_in, d, p->Cp) + (nacc > 0 ? model_cost_halo(d, p->Cp, kTileBN[t], nacc, s) : model_cost(d, p->Cp * p->terms / (p->half ? 2 : 1), kTileBN[t], s));
             if (c < best) { best = c; best_t = t; best_s = s; }
         }
     }
@@ -1273,6 +1324,12 @@ int igemm_plan_create(const ConvDims& d_in, int variant, int tile_id, int split_
     p->tile_id = best_t;
     p->BN = kTileBN[best_t];
     p->nacc = kTileNacc[best_t];
+    if (p->nacc == -4) {
+        if (mode == 1 || split_k > 1) { delete p; return BODA_ERR_UNSUPPORTED; }
+        p->pair = true;
+        p->nacc = 0;                 // operands, staging and layouts of the im2col kernel
+        best_s = 1;
+    }
     if (p->nacc == -3) {
         // ---- first-layer kernel: no staged input; filters [Rb*Sb][K][48]
         p->d = d_in;
@@ -1361,7 +1418,7 @@ int igemm_plan_create(const ConvDims& d_in, int variant, int tile_id, int split_
         p->xp_bytes = (((size_t)mflat * p->Cp * 4) + 1023) & ~(size_t)1023;
         p->partial_bytes = 0;   // split partial sums stay in shared memory (cluster reduction)
     } else {
-        p->tiles_m = (d.M + BM - 1) / BM;
+        p->tiles_m = p->pair ? (d.M + 255) / 256 : (d.M + BM - 1) / BM;
         p->xp_bytes = (((size_t)d.N * d.H * d.W * p->Cs() * p->esize()) + 1023) & ~(size_t)1023;
         p->partial_bytes = 0;   // split partial sums stay in shared memory (cluster reduction)
     }
@@ -1418,6 +1475,14 @@ void igemm_plan_describe(const IgemmPlan* p, char* buf, size_t n)
         if (p->pool_rows > 0) std::snprintf(pool, sizeof(pool), " +maxpool3x3s2(%d rows/tile)", p->pool_rows);
         std::snprintf(buf, n, "%stile=halo_%dx%d(id %d) slab=%d stages=%d split_k=%d grid=%dx%dx%d%s", view, 128 * p->nacc, p->BN,
                       p->tile_id, p->slab_rows, p->b_stages, p->splits, p->tiles_m, p->tiles_n, p->splits, pool);
+        return;
+    }
+    if (p->pair) {
+        const int tiles = p->tiles_m * p->tiles_n;
+        std::snprintf(buf, n, "%s%stile=pair_256x%d(id %d) stages=%d split_k=1 grid=%dx1x1 tiles=%d", view, p->half ? "f16 " : "", p->BN, p->tile_id,
+                      p->BN == 64 ? pair::Cfg<64>::STAGES : p->BN == 96 ? pair::Cfg<96>::STAGES : p->BN == 128 ? pair::Cfg<128>::STAGES
+                      : p->BN == 192 ? pair::Cfg<192>::STAGES : pair::Cfg<256>::STAGES,
+                      2 * std::min(tiles, p->sm_count / 2), tiles);
         return;
     }
     std::snprintf(buf, n, "%s%stile=igemm_128x%d(id %d) stages=%d split_k=%d grid=%dx%dx%d", view, p->half ? "f16 " : p->terms == 3 ? "x3 " : "", p->BN, p->tile_id,
@@ -1706,6 +1771,21 @@ int igemm_launch(IgemmPlan* p, const float* in, const float* filt, const float* 
     if (prm.out_tma && p->map_o_base != out) {
         int rc = encode_map_o(p, out);
         if (rc != BODA_OK) return rc;
+    }
+    if (p->pair) {
+        pair::PairParams pp;
+        pp.M = d.M; pp.stride = d.stride; pp.pad = d.pad; pp.S = d.S;
+        pp.cchunks = prm.cchunks; pp.last_ksteps = last_ksteps(d, p->chunk(), p->half); pp.iters = p->iters_total;
+        pp.tiles_n = p->tiles_n; pp.tiles_total = p->tiles_m * p->tiles_n;
+        pp.bias = bias; pp.o = prm.o; pp.status = p->d_status; pp.tx_extra = p->tx_extra; pp.b_early = prm.b_early; pp.out_tma = prm.out_tma;
+        switch (p->BN) {
+            case 64: return launch_pair<64>(p, pp, stream);
+            case 96: return launch_pair<96>(p, pp, stream);
+            case 128: return launch_pair<128>(p, pp, stream);
+            case 192: return launch_pair<192>(p, pp, stream);
+            case 256: return launch_pair<256>(p, pp, stream);
+            default: return BODA_ERR_UNSUPPORTED;
+        }
     }
     switch (p->BN) {
         case 64: return launch_bn<64>(p, prm, stream);

@@ -36,6 +36,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// the same without the hardware's suspended wait (a try_wait on a phase that stays open holds the thread for microseconds)
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+
 // Bounded wait.  Returns false if the CTA is aborting or the limit expired (then it raises the abort flag
 // and records where it gave up).  The limit is counted on the SM's own cycle counter, which is cheap to read
 // (the global nanosecond timer is not, and must stay out of the fast path): 4e9 cycles, about two seconds.

@@ -137,20 +137,44 @@ def _check(status: int, where: str) -> None:
 
 
 def _addr(t) -> Optional[int]:
-    if t is None:
-        return None
-    if isinstance(t, int):
+    if t is None or t.__class__ is int:
         return t
+    if isinstance(t, int):
+        return int(t)
     return t.data_ptr()
+
+
+_torch = None
+_raw_stream = _current_device = None
+
+
+def _load_torch():
+    """torch, imported on first use; the stream look-up bound once (`torch.cuda.current_stream()` builds a Stream object on
+    every call: 3.6 us against 0.3 us for the handle alone)."""
+    global _torch, _raw_stream, _current_device
+    if _torch is None:
+        import torch
+        _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
+        _torch = torch
+    return _torch
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
+        if _torch is None:
+            _load_torch()
+        return _raw_stream(_current_device()) or None
     if isinstance(stream, int):
         return stream or None
     return stream.cuda_stream or None
+
+
+def _empty_like_input(x, shape):
+    """Uninitialised fp32 tensor on x's device."""
+    torch = _torch or _load_torch()
+    if x.__class__ is torch.Tensor and x.dtype is torch.float32:
+        return x.new_empty(shape)                    # 1.9 us against 2.7 for torch.empty with its keywords
+    return torch.empty(shape, dtype=torch.float32, device=x.device)
 
 
 def boda_version() -> int:
@@ -376,9 +400,8 @@ class ConvPlan:
         boda_conv_plan_bind_filters(self.handle, filt, stream)
 
     def __call__(self, x, filt, bias=None, out=None, stream=None):
-        import torch
         if out is None:
-            out = torch.empty(self.out_shape, dtype=torch.float32, device=x.device)
+            out = _empty_like_input(x, self.out_shape)
         boda_conv_fwd_planned(self.handle, x, filt, bias, out, self.workspace, stream)
         return out
 
@@ -396,11 +419,9 @@ class ConvPlan:
 
 def conv_fwd(x, filt, bias=None, stride=1, pad=0, relu=True, stream=None):
     """One-call forward on CUDA tensors via ``boda_conv_fwd`` (plan cached inside the library)."""
-    import torch
     N, C, H, W = x.shape
     K, _, R, S = filt.shape
-    out = torch.empty((N, K, boda_conv_out_dim(H, R, stride, pad), boda_conv_out_dim(W, S, stride, pad)),
-                      dtype=torch.float32, device=x.device)
+    out = _empty_like_input(x, (N, K, boda_conv_out_dim(H, R, stride, pad), boda_conv_out_dim(W, S, stride, pad)))
     boda_conv_fwd(x, filt, bias, out, N, C, H, W, K, R, S, stride, pad, relu, stream)
     return out
 

@@ -71,8 +71,8 @@ enum { BODA_MATH_F16 = 4 };      /* reduced-precision STORAGE (Section 2 of the 
                                     10 mantissa bits, so the relative L2 error against the fp64 result stays <= 5e-3
                                     for operands inside fp16's range (|x| < 65504; larger values overflow to infinity,
                                     values below 6e-8 flush to zero), and <= 1e-5 against the fp64 result computed
-                                    from the fp16-rounded operands.  NCHW in and out only; K1CONV and TCONV (im2col
-                                    kernel); where no tensor-core variant is legal the FP32 kernel runs instead. */
+                                    from the fp16-rounded operands.  NCHW in and out only; K1CONV and TCONV (im2col and
+                                    CTA-pair tiles); where no tensor-core variant is legal the FP32 kernel runs instead. */
 
 typedef struct boda_conv_shape {
     int N, C, H, W;              /* input  [N][C][H][W] */
@@ -211,8 +211,8 @@ int boda_sgemm(const float* A, const float* B, float* C, int M, int N, int K, vo
 /*
  * Run-time compilation (Section 4 of the paper: kernels are generated and compiled for the exact problem once its
  * sizes are known, so that every extent is a literal).  The DIRECT tiles named direct_rtc_k4 / k8 / k16 / k32
- * (tile ids 12..15 of BODA_VARIANT_DIRECT; also what automatic selection uses for layers with C*R*S <= 512 and
- * K <= 128 that stay on the FP32 kernel) are compiled by NVRTC when their plan is created: one thread per output pixel and `kt` output channels,
+ * (tile ids 12..15 of BODA_VARIANT_DIRECT; also what automatic selection uses for layers with C*R*S <= 32,
+ * stride 1 and K <= 128 that stay on the FP32 kernel) are compiled by NVRTC when their plan is created: one thread per output pixel and `kt` output channels,
  * all of N, C, H, W, K, R, S, stride, pad, ReLU and the blocking as compile-time constants.  They need the NVRTC
  * shared library at run time (looked up with dlopen; without it - or with BODA_NO_RTC=1 in the environment - those
  * tiles return BODA_ERR_UNSUPPORTED and automatic selection keeps the precompiled kernels; the first plan for a

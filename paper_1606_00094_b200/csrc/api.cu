@@ -516,6 +516,9 @@ static int plan_time_ms(boda_conv_plan* p, bool chain_in, bool chain_out, int po
         if (pool_out) cudaFree(pool_out);
         if (in_packed || out_packed) (void)conv_plan_set_io(p, 0, 0, 0, 0, 0);
         if (fused) (void)conv_plan_set_pool(p, 0, 0);
+        // the scratch filters are gone: the plan must not take the caller's for them if they come to lie at that address
+        if (p->simt) simt_unbind_filters(p->simt);
+        if (p->ig) igemm_unbind_filters(p->ig);
     };
 #define TRY_T(x) do { cudaError_t _e = (x); if (_e != cudaSuccess) { rc = record_cuda_error(_e, #x); cleanup(); return rc; } } while (0)
     TRY_T(cudaMalloc(&in, n_in * 4)); TRY_T(cudaMalloc(&f, n_f * 4)); TRY_T(cudaMalloc(&b, d.K * 4));
@@ -568,7 +571,6 @@ static int plan_time_ms(boda_conv_plan* p, bool chain_in, bool chain_out, int po
     int st[STATUS_WORDS] = {0, 0, 0, 0};
     TRY_T(cudaMemcpy(st, p->d_status, sizeof(st), cudaMemcpyDeviceToHost));
     if (st[0] != 0) { (void)cudaMemset(p->d_status, 0, sizeof(st)); cleanup(); return st[0]; }
-    if (p->variant != BODA_VARIANT_DIRECT) igemm_unbind_filters(p->ig);
 #undef TRY_T
     cleanup();
     *ms_out = ms / iters;

@@ -1,0 +1,51 @@
+"""Which filters a plan computes with: those the call hands over, whatever the plan was tuned with or saw before; and what
+FP32 plans hold.  Integer-valued operands make every sum exact."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from helpers import oracle_out
+from paper_1606_00094_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _ints(shape, seed):
+    N, C, H, W, K, R, S, *_ = shape
+    return wl.integers(seed, (N, C, H, W)), wl.integers(seed + 1, (K, C, R, S)), wl.integers(seed + 2, (K,))
+
+
+def test_tuned_fp32_plan_does_not_keep_the_tuners_filters():
+    """The tuner's scratch buffers are freed when it is done; blocks of the same size that a program allocates next get their
+    addresses, and filters that it puts there are not the tuner's.  (Every call brings other filters than the one before it.)"""
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    shape = (20, 256, 13, 13, 384, 3, 3, 1, 1, 1)
+    x, w, b = _ints(shape, 9700)
+    dx, db = torch.from_numpy(x).cuda(), torch.from_numpy(b).cuda()
+    sides = [(torch.from_numpy(f).cuda(), torch.from_numpy(oracle_out(shape, x, f, b).astype(np.float32)).cuda()) for f in (w, wl.integers(9703, w.shape))]
+    out = torch.empty_like(sides[0][1])
+    torch.cuda.synchronize()
+    cudart = ctypes.CDLL("libcudart.so.12")
+    o = B.boda_plan_opts_default()
+    o.math, o.tune = B.BODA_MATH_FP32, 1
+    handle = B.boda_conv_plan_create(shape, o)
+    assert "direct_nhwc" in B.boda_conv_plan_describe(handle)
+    blocks = []
+    try:
+        for _ in range(32):
+            p = ctypes.c_void_p()
+            assert cudart.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(w.nbytes)) == 0
+            blocks.append(p)
+        ws = torch.empty(B.boda_conv_plan_workspace_bytes(handle), dtype=torch.uint8, device="cuda")
+        for i, p in enumerate(blocks):
+            filt, want = sides[i & 1]
+            assert cudart.cudaMemcpy(p, ctypes.c_void_p(filt.data_ptr()), ctypes.c_size_t(w.nbytes), ctypes.c_int(3)) == 0      # device to device
+            B.boda_conv_fwd_planned(handle, dx, p.value, db, out, ws)
+            assert torch.equal(out, want)
+    finally:
+        torch.cuda.synchronize()
+        B.boda_conv_plan_destroy(handle)
+        for p in blocks:
+            cudart.cudaFree(p)

@@ -165,6 +165,7 @@ int boda_conv_plan_kernels_per_call(const boda_conv_plan* plan);
  * a different pointer re-packs on that call.  Runs the re-layout on `stream` and waits for it (a set-up call,
  * not for the hot path): later launches may then fetch the packed filters without waiting for their predecessor
  * in the stream.  `filt` must stay unchanged while bound.
+ * FP32 plans (BODA_VARIANT_DIRECT) read `filt` on every call: for them binding returns at once and keeps nothing.
  */
 int boda_conv_plan_bind_filters(boda_conv_plan* plan, const float* filt, void* stream);
 

@@ -448,8 +448,7 @@ int boda_conv_plan_kernels_per_call(const boda_conv_plan* p)
 int boda_conv_plan_bind_filters(boda_conv_plan* p, const float* filt, void* stream)
 {
     if (!p || !filt) return BODA_ERR_INVALID_ARG;
-    if (p->simt) return simt_bind_filters(p->simt, filt, (cudaStream_t)stream);
-    if (p->variant == BODA_VARIANT_DIRECT) return BODA_OK;   // reads KCRS in place
+    if (p->variant == BODA_VARIANT_DIRECT) return BODA_OK;   // FP32 kernels read KCRS on every call
     return igemm_bind_filters(p->ig, filt, (cudaStream_t)stream);
 }
 
@@ -517,7 +516,6 @@ static int plan_time_ms(boda_conv_plan* p, bool chain_in, bool chain_out, int po
         if (in_packed || out_packed) (void)conv_plan_set_io(p, 0, 0, 0, 0, 0);
         if (fused) (void)conv_plan_set_pool(p, 0, 0);
         // the scratch filters are gone: the plan must not take the caller's for them if they come to lie at that address
-        if (p->simt) simt_unbind_filters(p->simt);
         if (p->ig) igemm_unbind_filters(p->ig);
     };
 #define TRY_T(x) do { cudaError_t _e = (x); if (_e != cudaSuccess) { rc = record_cuda_error(_e, #x); cleanup(); return rc; } } while (0)
@@ -530,7 +528,6 @@ static int plan_time_ms(boda_conv_plan* p, bool chain_in, bool chain_out, int po
     TRY_T(cudaEventCreate(&e0)); TRY_T(cudaEventCreate(&e1));
     TRY_T(cudaStreamSynchronize(0));                    // the fills above ran on the default stream
     TRY_T(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
-    if (p->simt) { rc = simt_bind_filters(p->simt, f, stream); if (rc) { cleanup(); return rc; } }
     if (p->variant != BODA_VARIANT_DIRECT) { rc = igemm_bind_filters(p->ig, f, stream); if (rc) { cleanup(); return rc; } }
     for (int i = 0; i < 2; ++i) { rc = run_once(in, f, b, out, ws, stream); if (rc) { cleanup(); return rc; } }
     TRY_T(cudaStreamSynchronize(stream));
@@ -674,7 +671,6 @@ int boda_conv_fwd_host(const float* in, const float* filt, const float* bias, fl
     BODA_CUDA_TRY(cudaMemcpyAsync(e->s_in, in, (size_t)d.N * d.C * d.H * d.W * 4, cudaMemcpyHostToDevice, st));
     BODA_CUDA_TRY(cudaMemcpyAsync(e->s_filt, filt, (size_t)d.K * d.Kred * 4, cudaMemcpyHostToDevice, st));
     if (bias) BODA_CUDA_TRY(cudaMemcpyAsync(e->s_bias, bias, (size_t)d.K * 4, cudaMemcpyHostToDevice, st));
-    if (e->plan->simt) simt_unbind_filters(e->plan->simt);
     if (e->plan->ig) igemm_unbind_filters(e->plan->ig);   // the staged filters may have changed
     rc = boda_conv_fwd_planned(e->plan, e->s_in, e->s_filt, bias ? e->s_bias : nullptr, e->s_out, e->workspace, stream);
     if (rc != BODA_OK) return rc;

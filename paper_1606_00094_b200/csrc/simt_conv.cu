@@ -326,7 +326,6 @@ struct SimtPlan {
     int bn = 128, Cp = 32, sms = kSms;
     Schedule s;
     float* d_wp = nullptr;
-    const float* bound = nullptr;
     size_t xp_bytes = 0;
     CUtensorMap map_a, map_b;
     const void* map_a_base = nullptr;
@@ -361,7 +360,8 @@ double simt_cost(const ConvDims& d, int bn)
     const int chunks = (d.C + BKC - 1) / BKC;
     const double steps = (double)s.whole / kSms * s.steps + (double)s.cut * s.steps / s.ctas;
     const double live = (double)((d.C + 3) / 4 * 4) / (chunks * BKC);        // part of the chunks that holds data
-    const double staging = ((double)d.N * d.C * d.H * d.W * 4 + (double)staged_bytes(d)) / 1734.0;
+    const double filters = (double)d.K * d.R * d.S * (d.C + chunks * BKC) * 4;
+    const double staging = ((double)d.N * d.C * d.H * d.W * 4 + (double)staged_bytes(d) + filters) / 1734.0;
     const double sums = s.cut == 0 ? 0.0 : 11400.0 + 518.0 * std::max(0.0, (double)s.ctas / s.cut - 1.0) + 2.0 * s.ctas * BM * bn * 4 / 3427.0;
     return staging + 9970.0 + steps * (32.0 * bn * live * 1.36 + 678.0) + sums;
 }
@@ -406,20 +406,6 @@ void simt_plan_describe(const SimtPlan* p, char* buf, size_t n)
     std::snprintf(buf, n, "grid=%d tiles=%dx%d cut=%d steps=%d", p->s.ctas, p->s.tiles_m, p->s.tiles_n, p->s.cut, p->s.steps);
 }
 
-static StageFilters stage_filters(SimtPlan* p, const float* filt) { return {filt, p->d_wp, p->d.K, p->d.C, p->Cp, p->d.R * p->d.S}; }
-
-int simt_bind_filters(SimtPlan* p, const float* filt, cudaStream_t stream)
-{
-    const StageFilters w = stage_filters(p, filt);
-    const int rc = stage_operands(STAGE_FP32, nullptr, &w, stream);
-    if (rc != BODA_OK) return rc;
-    BODA_CUDA_TRY(cudaStreamSynchronize(stream));
-    p->bound = filt;
-    return BODA_OK;
-}
-
-void simt_unbind_filters(SimtPlan* p) { p->bound = nullptr; }
-
 namespace {
 
 template <int WM, int WN, int TM, int TN>
@@ -445,11 +431,11 @@ int simt_launch(SimtPlan* p, const float* in, const float* filt, const float* bi
     const ConvDims& d = p->d;
     if (!workspace) return BODA_ERR_NOMEM;
     if (((uintptr_t)workspace & 255) != 0) return BODA_ERR_INVALID_ARG;
-    const bool bound = filt && filt == p->bound;
     if (!filt) return BODA_ERR_INVALID_ARG;
+    // Both operands on every call: FP32 plans read the caller's filters anew each time, as the kernels that use them in place do.
     const StageInput x = {in, workspace, d.N, d.C, p->Cp, d.H * d.W};
-    const StageFilters w = stage_filters(p, filt);
-    int rc = stage_operands(STAGE_FP32, &x, bound ? nullptr : &w, stream);
+    const StageFilters w = {filt, p->d_wp, d.K, d.C, p->Cp, d.R * d.S};
+    int rc = stage_operands(STAGE_FP32, &x, &w, stream);
     if (rc != BODA_OK) return rc;
     if (p->map_a_base != workspace) {
         const cuuint64_t Cp = (cuuint64_t)p->Cp;

@@ -11,14 +11,12 @@ struct SimtPlan;
 bool simt_legal(const ConvDims& d);
 int simt_num_widths();
 int simt_width(int i);
-double simt_cost(const ConvDims& d, int bn);                 // estimated SM clocks of one call with bound filters, staging included
+double simt_cost(const ConvDims& d, int bn);                 // estimated SM clocks of one call, staging included
 size_t simt_workspace_bytes(const ConvDims& d, int bn);
 int simt_plan_create(const ConvDims& d, int bn, int* d_status, SimtPlan** out);
 void simt_plan_destroy(SimtPlan* p);
 void simt_plan_describe(const SimtPlan* p, char* buf, size_t n);
-int simt_plan_kernels(const SimtPlan* p);                    // launches per call with bound filters
-int simt_bind_filters(SimtPlan* p, const float* filt, cudaStream_t stream);
-void simt_unbind_filters(SimtPlan* p);
+int simt_plan_kernels(const SimtPlan* p);                    // launches per call
 int simt_launch(SimtPlan* p, const float* in, const float* filt, const float* bias, float* out, void* workspace, cudaStream_t stream,
                 cudaEvent_t after_staging);
 

@@ -49,3 +49,22 @@ def test_tuned_fp32_plan_does_not_keep_the_tuners_filters():
         B.boda_conv_plan_destroy(handle)
         for p in blocks:
             cudart.cudaFree(p)
+
+
+@pytest.mark.parametrize("shape,tile", [((20, 256, 13, 13, 384, 3, 3, 1, 1, 1), -1), ((3, 36, 13, 13, 97, 3, 3, 1, 1, 1), 20), ((3, 36, 13, 13, 97, 3, 3, 1, 1, 1), 2)])
+def test_fp32_plans_read_their_filters_on_every_call(shape, tile):
+    """Binding an FP32 plan keeps nothing: filters written anew in place, and other filters in between, are what the next call uses."""
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    x, w, b = _ints(shape, 9710)
+    w2 = wl.integers(9713, w.shape)
+    dx, db = torch.from_numpy(x).cuda(), torch.from_numpy(b).cuda()
+    bound, other = torch.from_numpy(w).cuda(), torch.from_numpy(w2).cuda()
+    ref, ref2 = oracle_out(shape, x, w, b), oracle_out(shape, x, w2, b)
+    plan = B.ConvPlan(shape, math=B.BODA_MATH_FP32, variant=B.BODA_VARIANT_DIRECT, tile_id=tile)
+    plan.bind_filters(bound)
+    for filt, want in ((bound, ref), (other, ref2), (bound, ref)):
+        np.testing.assert_array_equal(plan(dx, filt, db).cpu().numpy().astype(np.float64), want, err_msg=plan.describe())
+    bound.copy_(other)
+    np.testing.assert_array_equal(plan(dx, bound, db).cpu().numpy().astype(np.float64), ref2, err_msg=plan.describe())
+    plan.close()

@@ -162,8 +162,9 @@ int boda_conv_plan_kernels_per_call(const boda_conv_plan* plan);
  * tensor-core plan, so that boda_conv_fwd_planned can skip the per-call filter re-layout.  Weights
  * are constants at deployment time (Section 2 speaks of deployment / inference).  After binding,
  * the `filt` argument of boda_conv_fwd_planned is ignored when it equals the bound pointer; passing
- * a different pointer re-packs on that call.  Runs the re-layout on `stream` and waits for it (a set-up call,
- * not for the hot path): later launches may then fetch the packed filters without waiting for their predecessor
+ * a different pointer re-packs on that call and ends the binding (the plan holds one packed copy: a graph captured
+ * while the plan was bound must not be replayed after that).  Runs the re-layout on `stream` and waits for it (a set-up
+ * call, not for the hot path): later launches may then fetch the packed filters without waiting for their predecessor
  * in the stream.  `filt` must stay unchanged while bound.
  * FP32 plans (BODA_VARIANT_DIRECT) read `filt` on every call: for them binding returns at once and keeps nothing.
  */

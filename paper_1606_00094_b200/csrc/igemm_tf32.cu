@@ -1627,6 +1627,7 @@ int igemm_launch(IgemmPlan* p, const float* in, const float* filt, const float* 
     float* xp = p->in_packed ? const_cast<float*>(in) : (float*)workspace;
     if (!filt) return BODA_ERR_INVALID_ARG;
     const bool bound = filt == p->bound_filt;         // unbound: re-layout on every call
+    if (!bound) p->bound_filt = nullptr;              // the packed copy is this call's from here on
     const bool stage_both = !bound && p->nacc == 0 && !p->s2d && !p->in_packed;     // in one launch with the input, below
     if (!bound && !stage_both) {
         const int rc = pack_filters(p, filt, stream);

@@ -68,3 +68,30 @@ def test_fp32_plans_read_their_filters_on_every_call(shape, tile):
     bound.copy_(other)
     np.testing.assert_array_equal(plan(dx, bound, db).cpu().numpy().astype(np.float64), ref2, err_msg=plan.describe())
     plan.close()
+
+
+@pytest.mark.parametrize("shape,variant,tile,math", [
+    ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 2, 0),           # im2col
+    ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 2, 3),
+    ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 6, 0),           # halo
+    ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 17, 0),          # gather
+    ((2, 3, 67, 67, 80, 11, 11, 4, 0, 1), 2, 24, 0),         # first layer
+    ((3, 64, 12, 12, 97, 1, 1, 1, 0, 1), 1, 20, 0),          # 1x1 from NCHW
+    ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 28, 4),          # CTA pairs, fp16
+])
+def test_other_filters_between_calls_with_the_bound_ones(shape, variant, tile, math):
+    """A tensor-core plan has room for one packed copy: a call with other filters writes over it, so the bound ones are packed again."""
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    x, w, b = _ints(shape, 9720)
+    w2 = wl.integers(9723, w.shape)
+    dx, db = torch.from_numpy(x).cuda(), torch.from_numpy(b).cuda()
+    bound, other = torch.from_numpy(w).cuda(), torch.from_numpy(w2).cuda()
+    ref, ref2 = oracle_out(shape, x, w, b), oracle_out(shape, x, w2, b)
+    plan = B.ConvPlan(shape, math=math, variant=variant, tile_id=tile)
+    plan.bind_filters(bound)
+    for filt, want in ((bound, ref), (other, ref2), (bound, ref), (other, ref2)):
+        np.testing.assert_array_equal(plan(dx, filt, db).cpu().numpy().astype(np.float64), want, err_msg=plan.describe())
+    plan.bind_filters(bound)
+    np.testing.assert_array_equal(plan(dx, bound, db).cpu().numpy().astype(np.float64), ref, err_msg=plan.describe())
+    plan.close()

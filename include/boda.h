@@ -184,6 +184,8 @@ int boda_conv_fwd_planned(boda_conv_plan* plan, const float* in, const float* fi
  * The forward pass in one call (the signature named by the build's specification).  Looks up, or
  * creates with default options, a plan for the shape on the current device and an internal
  * workspace, then launches on `stream`.  The first call for a shape allocates; later calls do not.
+ * Layers that run on the FP32 kernel hold no buffers here and may overlap on several streams; the tensor-core kernels'
+ * staged operands are shared by the calls of one shape, so order such calls on one stream or with events.
  */
 int boda_conv_fwd(const float* in, const float* filt, const float* bias, float* out,
                   int N, int C, int H, int W, int K, int R, int S, int stride, int pad, int relu,

@@ -593,6 +593,17 @@ static int cache_lookup(const boda_conv_shape& s, bool need_staging, CachedEntry
         boda_conv_plan* plan = nullptr;
         int rc = boda_conv_plan_create(&s, nullptr, &plan);
         if (rc != BODA_OK) return rc;
+        if (plan->simt) {
+            // Every caller of this shape gets this plan, from any thread and stream.  The FP32 kernels that read their operands
+            // where they lie hold nothing and may run side by side; a staged copy could not be shared like that.
+            boda_conv_plan_destroy(plan);
+            boda_plan_opts in_place;
+            boda_plan_opts_default(&in_place);
+            in_place.variant = BODA_VARIANT_DIRECT;
+            in_place.max_workspace = 1;
+            rc = boda_conv_plan_create(&s, &in_place, &plan);
+            if (rc != BODA_OK) return rc;
+        }
         CachedEntry ne;
         ne.plan = plan;
         if (plan->ws_bytes) {

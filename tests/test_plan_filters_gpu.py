@@ -95,3 +95,42 @@ def test_other_filters_between_calls_with_the_bound_ones(shape, variant, tile, m
     plan.bind_filters(bound)
     np.testing.assert_array_equal(plan(dx, bound, db).cpu().numpy().astype(np.float64), ref, err_msg=plan.describe())
     plan.close()
+
+
+# few filters, or little work: layers that the one-call entry point runs on the FP32 kernel
+ONE_CALL_FP32 = [(1, 370, 23, 23, 10, 9, 9, 1, 4, 1), (88, 651, 14, 14, 3, 7, 7, 2, 0, 1)]
+
+
+@pytest.mark.parametrize("shape", ONE_CALL_FP32)
+def test_one_call_fp32_layers_hold_no_buffers(shape):
+    """Calls of one shape share a cached plan: a kernel that stages its operands there would let two streams overwrite each other's,
+    so these layers run on the one kernel that reads them where they lie."""
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    x, w, b = _ints(shape, 9730)
+    dx, dw, db = (torch.from_numpy(t).cuda() for t in (x, w, b))
+    args = dict(stride=shape[7], pad=shape[8], relu=True)
+    B.conv_fwd(dx, dw, db, **args)
+    before = B.boda_kernel_launch_count()
+    got = B.conv_fwd(dx, dw, db, **args)
+    assert B.boda_kernel_launch_count() - before == 1
+    np.testing.assert_array_equal(got.cpu().numpy().astype(np.float64), oracle_out(shape, x, w, b))
+
+
+def test_one_call_fp32_layers_on_two_streams():
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    shape = ONE_CALL_FP32[0]
+    sides = []
+    for seed in (9731, 9741):
+        x, w, b = _ints(shape, seed)
+        sides.append((torch.cuda.Stream(), [torch.from_numpy(t).cuda() for t in (x, w, b)],
+                      torch.from_numpy(oracle_out(shape, x, w, b).astype(np.float32)).cuda(), []))
+    torch.cuda.synchronize()
+    for _ in range(50):
+        for stream, (dx, dw, db), _, outs in sides:
+            with torch.cuda.stream(stream):
+                outs.append(B.conv_fwd(dx, dw, db, stride=shape[7], pad=shape[8], relu=True))
+    torch.cuda.synchronize()
+    for _, _, want, outs in sides:
+        assert all(torch.equal(o, want) for o in outs)

@@ -149,7 +149,10 @@ int boda_conv_plan_destroy(boda_conv_plan* plan);
 int boda_conv_plan_describe(const boda_conv_plan* plan, char* buf, size_t buf_bytes);
 
 /* Bytes of caller-provided scratch that boda_conv_fwd_planned needs (0 if none).  The scratch holds
- * the re-laid-out input (the "input transformation" that the paper's k1conv and tconv apply, Section 5). */
+ * the re-laid-out input (the "input transformation" that the paper's k1conv and tconv apply, Section 5), its channels
+ * padded to a multiple of 32 (64 for fp16 storage; two such parts in the error-compensated mode), and for the FP32 tiles
+ * direct_nhwc_* the partial sums of tiles cut between CTAs (up to 19 MB).  A plan whose direct_nhwc_* tile was picked by
+ * rule also runs without (workspace NULL, or off its 256-byte alignment), on a slower kernel that stages nothing. */
 size_t boda_conv_plan_workspace_bytes(const boda_conv_plan* plan);
 
 /* Kernels one boda_conv_fwd_planned call launches when the filters are bound: 1 for the kernels that read NCHW themselves
@@ -172,7 +175,7 @@ int boda_conv_plan_bind_filters(boda_conv_plan* plan, const float* filt, void* s
 
 /*
  * The forward pass with an explicit plan.  `workspace` must point to at least
- * boda_conv_plan_workspace_bytes(plan) bytes of device memory, 256-byte aligned (NULL if 0 bytes);
+ * boda_conv_plan_workspace_bytes(plan) bytes of device memory, 256-byte aligned (NULL if 0 bytes; see there);
  * it may be shared between plans whose launches are ordered on one stream.  No allocation and no
  * synchronisation happen here.  The same plan must not be used from two streams at once.
  * Errors: INVALID_ARG (NULL tensor), CUDA (launch failure).

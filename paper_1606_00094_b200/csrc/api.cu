@@ -144,6 +144,7 @@ struct boda_conv_plan {
     DirectRtc* rtc = nullptr;            // DIRECT, tiles compiled at run time
     int split = 1;                       // DIRECT, GEMM-blocked tiles: CTAs of a cluster that share a tile's reduction
     SimtPlan* simt = nullptr;            // DIRECT, tiles over a staged input
+    int plain_tile = -1, plain_split = 1;    // DIRECT, a staged tile picked by rule: what calls without workspace run on
     IgemmPlan* ig = nullptr;             // K1CONV / TCONV
     size_t ws_bytes = 0;
     bool in_packed = false;              // chained layers: the input arrives in the staged layout
@@ -157,10 +158,11 @@ int conv_fwd_planned_ex(boda_conv_plan* p, const float* in, const float* filt, c
     if (!p || !in || !out) return BODA_ERR_INVALID_ARG;
     if (p->variant == BODA_VARIANT_DIRECT) {
         if (!filt) return BODA_ERR_INVALID_ARG;
-        if (p->simt) return simt_launch(p->simt, in, filt, bias, out, workspace, stream, after_staging);
+        const bool plain = p->plain_tile >= 0 && (!workspace || ((uintptr_t)workspace & 255) != 0);
+        if (p->simt && !plain) return simt_launch(p->simt, in, filt, bias, out, workspace, stream, after_staging);
         if (after_staging) BODA_CUDA_TRY(cudaEventRecord(after_staging, stream));
         if (p->rtc) return direct_rtc_launch(p->rtc, in, filt, bias, out, stream);
-        return direct_launch(p->d, p->tile_id, p->split, in, filt, bias, out, p->d_tab, stream);
+        return direct_launch(p->d, plain ? p->plain_tile : p->tile_id, plain ? p->plain_split : p->split, in, filt, bias, out, p->d_tab, stream);
     }
     if (p->ws_bytes && !workspace && !p->in_packed) return BODA_ERR_NOMEM;
     return igemm_launch(p->ig, in, filt, bias, out, workspace, stream, after_staging);
@@ -273,6 +275,13 @@ static int plan_build(const boda_conv_shape& shape, const boda_plan_opts& o, Dev
             const size_t ws = simt_workspace_bytes(p->d, bn);
             rc = o.max_workspace > 0 && ws > o.max_workspace ? BODA_ERR_NOMEM : simt_plan_create(p->d, bn, p->d_status, &p->simt);
             if (rc == BODA_OK) p->ws_bytes = ws;
+            if (tile_id < 0) {
+                // the caller asked for an FP32 layer, not for this tile: it also runs without workspace, or where the
+                // staged tile's own memory is not to be had
+                const int t = direct_pick_tile(p->d, 1);
+                if (rc == BODA_OK) { p->plain_tile = t; p->plain_split = direct_pick_split(p->d, t); }
+                else { p->tile_id = t; rc = BODA_OK; }
+            }
         }
         p->split = split_k > 0 ? std::min(split_k, direct_max_split(p->d, p->tile_id)) : direct_pick_split(p->d, p->tile_id);
     } else {

@@ -134,3 +134,27 @@ def test_one_call_fp32_layers_on_two_streams():
     torch.cuda.synchronize()
     for _, _, want, outs in sides:
         assert all(torch.equal(o, want) for o in outs)
+
+
+def test_fp32_plan_runs_without_workspace():
+    """FP32 plans picked by rule take workspace where they can use it and run without (or with one off its alignment) on the
+    kernel that needs none; only a forced staged tile insists."""
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    shape = (20, 256, 13, 13, 384, 3, 3, 1, 1, 1)
+    x, w, b = _ints(shape, 9740)
+    dx, dw, db = (torch.from_numpy(t).cuda() for t in (x, w, b))
+    want = oracle_out(shape, x, w, b)
+    out = torch.empty(want.shape, device="cuda")
+    plan = B.ConvPlan(shape, math=B.BODA_MATH_FP32)
+    assert "direct_nhwc" in plan.describe()
+    for ws in (None, plan.workspace, plan.workspace[4:], None):
+        out.fill_(float("nan"))
+        B.boda_conv_fwd_planned(plan.handle, dx, dw, db, out, ws)
+        np.testing.assert_array_equal(out.cpu().numpy().astype(np.float64), want)
+    plan.close()
+    forced = B.ConvPlan(shape, math=B.BODA_MATH_FP32, variant=B.BODA_VARIANT_DIRECT, tile_id=18)
+    with pytest.raises(B.BodaError) as e:
+        B.boda_conv_fwd_planned(forced.handle, dx, dw, db, out, None)
+    assert e.value.status == B.BODA_ERR_NOMEM
+    forced.close()

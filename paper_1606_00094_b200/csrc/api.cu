@@ -360,7 +360,7 @@ int boda::conv_plan_create_chained(const boda_conv_shape* shape, const boda_plan
         // view).  The fastest plan is kept and remembered in the file named by BODA_TUNE_CACHE (if set).
         char key[160];
         // the leading number names the tile tables: entries written by a build with other tables are not matched
-        constexpr int kTileTableVersion = 4;
+        constexpr int kTileTableVersion = 5;
         std::snprintf(key, sizeof(key), "t%d:%d,%d,%d,%d,%d,%d,%d,%d,%d,v%d,s%d,k%d,m%d,io%d%d", kTileTableVersion, shape->N, shape->C,
                       shape->H, shape->W, shape->K, shape->R, shape->S, shape->stride, shape->pad, o.variant, o.s2d, o.split_k, o.math,
                       chain_in ? 1 : 0, chain_out ? 1 : 0);

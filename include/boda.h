@@ -84,7 +84,8 @@ typedef struct boda_conv_shape {
 typedef struct boda_plan_opts {
     int math;                    /* BODA_MATH_* */
     int tune;                    /* 0: pick variant and tile by rule; 1: time the candidates on the device (synchronises):
-                                    every tile and split of the rule's variant and, where `variant` and `math` are
+                                    every tile of the rule's variant (tensor-core tiles: with every split; FP32 tiles:
+                                    with the split of their cost model, or `split_k`) and, where `variant` and `math` are
                                     left automatic, of the alternative variant too (FP32 kernel against tensor-core
                                     kernel, a strided TCONV layer with and without its space-to-depth view) */
     int variant;                 /* BODA_VARIANT_AUTO or a forced variant (used by tests) */

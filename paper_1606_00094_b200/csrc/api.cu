@@ -354,8 +354,8 @@ int boda::conv_plan_create_chained(const boda_conv_shape* shape, const boda_plan
             (o.math == BODA_MATH_AUTO || o.math == BODA_MATH_TF32X3 || o.math == BODA_MATH_F16))
             rc = plan_build(*shape, o, ctx, BODA_VARIANT_DIRECT, -1, 0, plan);
     } else {
-        // Automated tuning: the rule above names a variant; timing confirms or overturns it.  Every tile and split
-        // of that variant is timed and, when the caller left variant and math open, so is the alternative (the FP32
+        // Automated tuning: the rule above names a variant; timing confirms or overturns it.  Every tile
+        // of that variant is timed, a tensor-core tile with every split, and, when the caller left variant and math open, so is the alternative (the FP32
         // kernel against the tensor-core variant, and a strided tconv layer with and without its space-to-depth
         // view).  The fastest plan is kept and remembered in the file named by BODA_TUNE_CACHE (if set).
         char key[160];
@@ -397,7 +397,8 @@ int boda::conv_plan_create_chained(const boda_conv_shape* shape, const boda_plan
             for (int t = 0; t < ntiles; ++t) {
                 const int nsplit = c.variant == BODA_VARIANT_DIRECT ? 1 : igemm_num_split_candidates();
                 for (int si = 0; si < nsplit; ++si) {
-                    const int split = c.variant == BODA_VARIANT_DIRECT ? 0 : igemm_split_candidate(si);
+                    // FP32 tiles: the split that the caller forces, else the one that the tile's model picks
+                    const int split = c.variant != BODA_VARIANT_DIRECT ? igemm_split_candidate(si) : variant == BODA_VARIANT_DIRECT ? o.split_k : 0;
                     if (o.split_k > 0 && split != o.split_k) continue;
                     boda_conv_plan* cand = nullptr;
                     if (plan_build(*shape, oc, ctx, c.variant, t, split, &cand) != BODA_OK) continue;

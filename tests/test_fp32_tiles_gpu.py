@@ -82,3 +82,16 @@ def test_workspace_limit_keeps_fp32_plans_off_the_staged_tiles():
     with pytest.raises(B.BodaError) as e:
         B.ConvPlan(shape, math=1, variant=0, tile_id=18, max_workspace=4096)
     assert e.value.status == B.BODA_ERR_NOMEM
+
+
+def test_tuning_an_fp32_layer_with_a_forced_split_times_its_tiles(tmp_path, monkeypatch):
+    from paper_1606_00094_b200 import binding as B
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("BODA_TUNE_CACHE", str(cache))
+    plan = B.ConvPlan((3, 36, 13, 13, 97, 3, 3, 1, 1, 1), math=B.BODA_MATH_FP32, tune=1, split_k=3)
+    try:
+        # (nothing is written down where nothing was timed)
+        assert cache.exists() and len(cache.read_text().strip().splitlines()) == 1
+        assert "split_k=3" in plan.describe() or "split_k=1" in plan.describe()      # 1: a tile that does not split was faster
+    finally:
+        plan.close()

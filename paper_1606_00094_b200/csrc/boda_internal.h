@@ -12,7 +12,7 @@ namespace boda {
 
 // Device status word layout (int[4]): [0] status code, [1] where (kernel id), [2] block, [3] detail.
 enum { STATUS_WORDS = 4 };
-enum { KERNEL_ID_DIRECT = 1, KERNEL_ID_IGEMM = 2, KERNEL_ID_PACK = 3 };
+enum { KERNEL_ID_DIRECT = 1, KERNEL_ID_IGEMM = 2, KERNEL_ID_PACK = 3, KERNEL_ID_SIMT = 4 };
 
 struct ConvDims {
     int N, C, H, W, K, R, S, stride, pad, relu;

@@ -465,6 +465,7 @@ igemm_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         cluster_arrive();
         cluster_wait();
     }
+    if (s_abort) settle_after_abort();
     __syncthreads();
     if (p.splits > 1) {
         if (!exchange) {
@@ -1246,17 +1247,9 @@ int igemm_plan_create(const ConvDims& d_in, int variant, int tile_id, int split_
     p->d = d;
     p->orig = d_in;
     p->s2d = use_s2d;
-    {
-        // Test hooks, off unless the environment asks: a transfer-size mismatch that lets one bounded wait run out,
-        // and a shorter limit for that wait (failure detection is tested without faulting or hanging the GPU).
-        const char* mm = std::getenv("BODA_TEST_TX_MISMATCH");
-        p->tx_extra = (mm && *mm == '1') ? 16 : 0;
-        const char* lim = std::getenv("BODA_WAIT_LIMIT_CYCLES");
-        long long cycles = lim ? std::atoll(lim) : kWaitLimitCycles;
-        if (cycles < 1000000) cycles = 1000000;
-        cudaError_t ce = cudaMemcpyToSymbol(c_wait_limit_cycles, &cycles, sizeof(cycles));
-        if (ce != cudaSuccess) { delete p; return record_cuda_error(ce, "wait limit upload"); }
-    }
+    p->tx_extra = test_tx_extra();
+    rc = upload_wait_limit();
+    if (rc != BODA_OK) { delete p; return rc; }
     p->variant = variant;
     p->d_status = d_status;
     p->half = mode == 2;

@@ -23,6 +23,7 @@
 #include <cstdlib>
 #include <new>
 
+#define BODA_WAIT_KERNEL_ID KERNEL_ID_SIMT
 #include "simt_conv.h"
 #include "stage.h"
 #include "tc_ptx.cuh"
@@ -48,6 +49,7 @@ struct SimtParams {
     float* partial;                                      // two slots of [BN][128] per CTA
     int relu;
     int* status;
+    int tx_extra;                                        // test hook: bytes the first stage of CTA 0 expects and never gets
 };
 
 template <int WM, int WN, int TM, int TN>
@@ -152,6 +154,8 @@ simt_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         return true;
     };
     if (loader) {
+        if (p.tx_extra && blockIdx.x == 0)
+            asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" :: "r"(full_bar), "r"(p.tx_extra) : "memory");
         lw.start(p);
         load_piece();
         for (int i = 0; i < AHEAD; ++i) (void)load_step();
@@ -176,7 +180,10 @@ simt_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         int chunk = i0 % p.cchunks;
         for (int it = i0; it < i1; ++it) {
             if (loader) (void)load_step();
-            if (!mbar_wait(full_bar + 8 * stage, par, &s_abort, p.status, 52)) return;
+            if (!mbar_wait(full_bar + 8 * stage, par, &s_abort, p.status, 52)) {
+                if (loader) settle_after_abort();        // the loads in flight are this thread's; the block's memory stays until it leaves
+                return;
+            }
             __syncwarp();                // the loading lane rejoins its warp
             const uint8_t* a_row = smem + stage * G::STAGE_BYTES + m_local * 128;
             const uint8_t* b_row = smem + stage * G::STAGE_BYTES + A_STAGE_BYTES + n_local * 128;
@@ -330,6 +337,7 @@ struct SimtPlan {
     CUtensorMap map_a, map_b;
     const void* map_a_base = nullptr;
     int* d_status = nullptr;
+    int tx_extra = 0;
 };
 
 bool simt_legal(const ConvDims& d)
@@ -377,6 +385,8 @@ int simt_plan_create(const ConvDims& d, int bn, int* d_status, SimtPlan** out)
     p->bn = bn;
     p->Cp = ((d.C + BKC - 1) / BKC) * BKC;
     p->d_status = d_status;
+    p->tx_extra = test_tx_extra();
+    if ((rc = upload_wait_limit()) != BODA_OK) { delete p; return rc; }
     p->s = schedule(d, bn, kSms);
     p->xp_bytes = staged_bytes(d);
     cudaError_t e = cudaMalloc(&p->d_wp, (size_t)d.R * d.S * d.K * p->Cp * 4);
@@ -457,7 +467,7 @@ int simt_launch(SimtPlan* p, const float* in, const float* filt, const float* bi
     prm.last_groups = (d.C - BKC * (prm.cchunks - 1) + 3) / 4;
     prm.steps = p->s.steps;
     prm.tiles_n = p->s.tiles_n; prm.whole_tiles = p->s.whole; prm.cut_tiles = p->s.cut;
-    prm.bias = bias; prm.out = out; prm.relu = d.relu; prm.status = p->d_status;
+    prm.bias = bias; prm.out = out; prm.relu = d.relu; prm.status = p->d_status; prm.tx_extra = p->tx_extra;
     prm.partial = reinterpret_cast<float*>(static_cast<char*>(workspace) + p->xp_bytes);
     switch (p->bn) {
         case 128: return launch_width<2, 4, 8, 8>(p, prm, stream);

@@ -6,14 +6,38 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cstdlib>
+
 #include "boda_internal.h"
+
+// what a wait that ran out is recorded under: a source file whose kernels are others says so before it includes this one
+#ifndef BODA_WAIT_KERNEL_ID
+#define BODA_WAIT_KERNEL_ID KERNEL_ID_IGEMM
+#endif
 
 namespace boda {
 namespace tc {
 
 constexpr long long kWaitLimitCycles = 4000000000ll;
-// The limit actually used (SM cycles).  Tests shorten it through the environment variable BODA_WAIT_LIMIT_CYCLES.
-__constant__ long long c_wait_limit_cycles = kWaitLimitCycles;
+// The limit actually used (SM cycles).  Tests shorten it through the environment variable BODA_WAIT_LIMIT_CYCLES.  Each source
+// file that includes this one has its own copy, which its plans set (upload_wait_limit).
+static __constant__ long long c_wait_limit_cycles = kWaitLimitCycles;
+
+// Test hooks, off unless the environment asks: a transfer-size mismatch that lets one bounded wait run out, and a shorter limit
+// for that wait (failure detection is tested without faulting or hanging the GPU).
+[[maybe_unused]] static int test_tx_extra()
+{
+    const char* mm = std::getenv("BODA_TEST_TX_MISMATCH");
+    return (mm && *mm == '1') ? 16 : 0;
+}
+[[maybe_unused]] static int upload_wait_limit()
+{
+    const char* lim = std::getenv("BODA_WAIT_LIMIT_CYCLES");
+    long long cycles = lim ? std::atoll(lim) : kWaitLimitCycles;
+    if (cycles < 1000000) cycles = 1000000;
+    BODA_CUDA_TRY(cudaMemcpyToSymbol(c_wait_limit_cycles, &cycles, sizeof(cycles)));
+    return BODA_OK;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -63,7 +87,7 @@ static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity
             } else if (clock64() - t0 > c_wait_limit_cycles) {
                 *abort_flag = 1;
                 if (atomicCAS(status, 0, (int)BODA_ERR_DEVICE_TIMEOUT) == 0) {
-                    status[1] = KERNEL_ID_IGEMM;
+                    status[1] = BODA_WAIT_KERNEL_ID;
                     status[2] = (int)(blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z));
                     status[3] = where;
                 }
@@ -78,6 +102,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return mbar_wait_slow(bar, parity, abort_flag, status, where);
 }
 
+// For a CTA that is giving up, before its last barrier: copies into its shared memory and MMAs that read it may still be under way,
+// and their barriers may never complete (a byte count that was not posted), so what is waited for is time: half a millisecond, a
+// hundred times what the slowest of them takes.
+static __device__ __noinline__ void settle_after_abort()
+{
+    const long long t0 = clock64();
+    while (clock64() - t0 < 1000000) __nanosleep(1000);
+}
+
 // Bounded wait for threads that are not on the critical path (the epilogue waiting for the accumulator):
 // polls rarely and sleeps in between, so that it does not compete with the producer's and the MMA issuer's
 // barrier traffic.  The limit is the same number of cycles, counted in sleep quanta.
@@ -90,7 +123,7 @@ static __device__ __noinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t par
         if (clock64() - t0 > c_wait_limit_cycles) {
             *abort_flag = 1;
             if (atomicCAS(status, 0, (int)BODA_ERR_DEVICE_TIMEOUT) == 0) {
-                status[1] = KERNEL_ID_IGEMM;
+                status[1] = BODA_WAIT_KERNEL_ID;
                 status[2] = (int)(blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z));
                 status[3] = where;
             }

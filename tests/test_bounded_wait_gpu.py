@@ -16,7 +16,7 @@ from helpers import TF32_TOL, assert_parity, oracle_out
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("tile,split", [(2, 1), (6, 1), (3, 2), (10, 2), (17, 1)])   # im2col and halo kernels, with and without a cluster; gather kernel
+@pytest.mark.parametrize("tile,split", [(2, 1), (6, 1), (3, 2), (10, 2), (17, 1), (26, 1), (30, 1)])   # im2col and halo kernels, with and without a cluster; gather kernel; CTA pairs
 def test_expired_wait_sets_status_and_context_survives(tile, split):
     import torch
     from paper_1606_00094_b200 import binding as B
@@ -107,3 +107,36 @@ def test_expired_wait_in_the_first_layer_kernel():
     assert B.boda_query_status() == 0
     plan.close()
     assert_parity(got, oracle_out(shape, x, w, b), TF32_TOL)
+
+
+@pytest.mark.parametrize("tile", [18, 22])
+def test_expired_wait_in_the_staged_fp32_kernel(tile):
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    shape = (3, 64, 13, 13, 200, 3, 3, 1, 1, 1)
+    N, C, H, W, K, R, S, st, pad, relu = shape
+    x, w, b = wl.integers(10, (N, C, H, W)), wl.integers(11, (K, C, R, S)), wl.integers(12, (K,))
+    dx, dw, db = (torch.from_numpy(t).cuda() for t in (x, w, b))
+    assert B.boda_query_status() == 0
+    os.environ["BODA_TEST_TX_MISMATCH"] = "1"
+    os.environ["BODA_WAIT_LIMIT_CYCLES"] = "100000000"
+    try:
+        plan = B.ConvPlan(shape, math=B.BODA_MATH_FP32, variant=B.BODA_VARIANT_DIRECT, tile_id=tile)
+    finally:
+        del os.environ["BODA_TEST_TX_MISMATCH"]
+        del os.environ["BODA_WAIT_LIMIT_CYCLES"]
+    start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    start.record()
+    plan(dx, dw, db)
+    end.record()
+    torch.cuda.synchronize()
+    assert start.elapsed_time(end) < 500                        # the shortened limit counts here too (the full one is two seconds)
+    assert B.boda_query_status() == B.BODA_ERR_DEVICE_TIMEOUT
+    assert B.boda_query_status() == 0
+    plan.close()
+    plan = B.ConvPlan(shape, math=B.BODA_MATH_FP32, variant=B.BODA_VARIANT_DIRECT, tile_id=tile)
+    got = plan(dx, dw, db).cpu().numpy()
+    torch.cuda.synchronize()
+    assert B.boda_query_status() == 0
+    plan.close()
+    np.testing.assert_array_equal(got.astype(np.float64), oracle_out(shape, x, w, b))

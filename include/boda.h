@@ -71,7 +71,8 @@ enum { BODA_MATH_F16 = 4 };      /* reduced-precision STORAGE (Section 2 of the 
                                     10 mantissa bits, so the relative L2 error against the fp64 result stays <= 5e-3
                                     for operands inside fp16's range (|x| < 65504; larger values overflow to infinity,
                                     values below 6e-8 flush to zero), and <= 1e-5 against the fp64 result computed
-                                    from the fp16-rounded operands.  NCHW in and out only; K1CONV and TCONV (im2col and
+                                    from the fp16-rounded operands (reductions C*R*S up to 8192; the tensor core
+                                    truncates its sums, so beyond that the bound grows with the reduction).  NCHW in and out only; K1CONV and TCONV (im2col and
                                     CTA-pair tiles); where no tensor-core variant is legal the FP32 kernel runs instead. */
 
 typedef struct boda_conv_shape {

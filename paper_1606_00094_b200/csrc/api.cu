@@ -403,6 +403,7 @@ int boda::conv_plan_create_chained(const boda_conv_shape* shape, const boda_plan
                     boda_conv_plan* cand = nullptr;
                     if (plan_build(*shape, oc, ctx, c.variant, t, split, &cand) != BODA_OK) continue;
                     float ms = 0.f;
+                    if (cand->ig && igemm_plan_sums_too_long(cand->ig)) { boda_conv_plan_destroy(cand); continue; }
                     if (plan_time_ms(cand, chain_in, chain_out, pool_ksz, pool_stride, &ms) == BODA_OK && ms < best_ms) {
                         if (best) boda_conv_plan_destroy(best);
                         best = cand;

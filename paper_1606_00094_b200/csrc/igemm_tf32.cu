@@ -1003,6 +1003,22 @@ double model_cost_pair(const ConvDims& d, int BN, int taps, int cchunks, int las
     return rounds * per_tile + 5000.0 + 32.0 * BN;
 }
 
+// Accumulators of a pair tile, and the MMA steps that each of them takes.  At 1.6e-8 a step (pair::Cfg::ACCS) 256 steps keep a sum
+// within 4e-6 and kMaxPairSteps within 1e-5; layers with longer reductions stay on the one-CTA tiles, whose cluster split
+// shares them out.
+constexpr int kMaxPairSteps = 512;
+int pair_mma_steps(const ConvDims& d, int chunk, bool half) { return d.R * d.S * (4 * ((d.C + chunk - 1) / chunk - 1) + last_ksteps(d, chunk, half)); }
+int pair_accs(const ConvDims& d, int BN, int chunk, bool half)
+{
+    const int most = BN <= 64 ? pair::Cfg<64>::ACCS : BN <= 128 ? pair::Cfg<128>::ACCS : pair::Cfg<256>::ACCS;
+    return std::min(most, (pair_mma_steps(d, chunk, half) + 255) / 256);
+}
+int pair_steps(const ConvDims& d, int BN, int chunk, bool half)
+{
+    const int accs = pair_accs(d, BN, chunk, half);
+    return (pair_mma_steps(d, chunk, half) + accs - 1) / accs;
+}
+
 int encode_map_a_k1n(IgemmPlan* p, const void* in)
 {
     const ConvDims& d = p->d;
@@ -1269,7 +1285,7 @@ int igemm_plan_create(const ConvDims& d_in, int variant, int tile_id, int split_
         if (tile_id >= 0 && t != tile_id) continue;
         const int nacc = kTileNacc[t];
         if (nacc == -4) {
-            if (mode == 1 || split_k > 1) continue;
+            if (mode == 1 || split_k > 1 || pair_steps(d, kTileBN[t], p->chunk(), p->half) > kMaxPairSteps) continue;
             if (max_ws > 0 && (((size_t)d.N * d.H * d.W * p->Cs() * p->esize() + 1023) & ~(size_t)1023) > max_ws) continue;
             const double c = staging_cost(d_in, d, p->Cp) + model_cost_pair(d, kTileBN[t], d.R * d.S, p->Cp / p->chunk(), last_ksteps(d, p->chunk(), p->half), p->sm_count);
             if (c < best) { best = c; best_t = t; best_s = 1; }
@@ -1438,6 +1454,7 @@ int igemm_plan_tile(const IgemmPlan* p) { return p->tile_id; }
 bool igemm_plan_writes_packed(const IgemmPlan* p) { return p->nacc != -2 && p->terms != 3 && !p->half; }
 int igemm_plan_kernels_per_call(const IgemmPlan* p) { return (p->nacc < 0 || p->in_packed) ? 1 : 2; }
 int igemm_plan_splits(const IgemmPlan* p) { return p->splits; }
+bool igemm_plan_sums_too_long(const IgemmPlan* p) { return p->pair && pair_steps(p->d, p->BN, p->chunk(), p->half) > kMaxPairSteps; }
 size_t igemm_plan_workspace_bytes(const IgemmPlan* p) { return p->xp_bytes + p->partial_bytes; }
 
 void igemm_plan_describe(const IgemmPlan* p, char* buf, size_t n)
@@ -1770,6 +1787,7 @@ int igemm_launch(IgemmPlan* p, const float* in, const float* filt, const float* 
         pair::PairParams pp;
         pp.M = d.M; pp.stride = d.stride; pp.pad = d.pad; pp.S = d.S;
         pp.cchunks = prm.cchunks; pp.last_ksteps = last_ksteps(d, p->chunk(), p->half); pp.iters = p->iters_total;
+        pp.accs = pair_accs(d, p->BN, p->chunk(), p->half);
         pp.tiles_n = p->tiles_n; pp.tiles_total = p->tiles_m * p->tiles_n;
         pp.bias = bias; pp.o = prm.o; pp.status = p->d_status; pp.tx_extra = p->tx_extra; pp.b_early = prm.b_early; pp.out_tma = prm.out_tma;
         switch (p->BN) {

@@ -26,6 +26,8 @@ int igemm_plan_tile(const IgemmPlan* p);
 bool igemm_plan_writes_packed(const IgemmPlan* p);       // can the plan write a consumer's staged layout?
 int igemm_plan_kernels_per_call(const IgemmPlan* p);     // 1, or 2 where an input staging kernel runs first
 int igemm_plan_splits(const IgemmPlan* p);
+// a tile whose accumulators would take more MMA steps than the error bars allow: run when forced, never picked
+bool igemm_plan_sums_too_long(const IgemmPlan* p);
 size_t igemm_plan_workspace_bytes(const IgemmPlan* p);
 void igemm_plan_describe(const IgemmPlan* p, char* buf, size_t n);
 int igemm_bind_filters(IgemmPlan* p, const float* filt, cudaStream_t stream);

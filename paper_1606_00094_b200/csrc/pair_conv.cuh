@@ -33,6 +33,7 @@ struct PairParams {
     int cchunks;                 // reduction chunks per tap (128 bytes of channels each)
     int last_ksteps;             // 32-byte MMA steps of a tap's last chunk that hold channels (1..4): the rest are padding and skipped
     int iters;                   // taps * cchunks
+    int accs;                    // accumulators that a tile's stages take turns with (at most Cfg::ACCS, and the stages of a tile)
     int tiles_n, tiles_total;    // tiles are numbered point tile * tiles_n + channel tile
     const float* bias;
     OutSpec o;
@@ -51,7 +52,14 @@ template <int BN> struct Cfg {
     static constexpr int STAGE_BYTES = CPS * (A_CHUNK_BYTES + B_CHUNK_BYTES);
     static constexpr int STORE_BYTES = 8 * BOX_BYTES;
     static constexpr int STAGES = BN >= 256 ? 5 : (192 * 1024) / STAGE_BYTES;
-    static constexpr int TMEM_COLS = 2 * BN <= 128 ? 128 : 2 * BN <= 256 ? 256 : 512;
+    // Accumulators that a tile may have, taking the stages in turn; two tiles' worth fill tensor memory.  The tensor core truncates
+    // an accumulator at every MMA, so the error of a sum grows with the MMAs that one accumulator takes: measured 1.6e-8 of the
+    // result per MMA (1563 of them 2.5e-5).  Reading more than one back costs a short reduction up to 10 % (its epilogue does not
+    // hide under the next tile), so only the longer ones have them (PairParams::accs).
+    static constexpr int ACCS = BN <= 64 ? 4 : BN <= 128 ? 2 : 1;
+    static constexpr int TILE_COLS = ACCS * BN;
+    static constexpr int TMEM_COLS = 512;
+    static_assert(2 * TILE_COLS <= TMEM_COLS, "two tiles fit");
     // (the boxes are only there where the output leaves through tensor stores: without them a CTA can become resident beside the
     // staging kernel's and overlap its prologue)
     static constexpr int smem_bytes(bool boxes) { return STAGES * STAGE_BYTES + 256 /*barriers*/ + (boxes ? STORE_BYTES : 0) + 1024 /*alignment*/; }
@@ -217,6 +225,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             constexpr uint32_t idesc = instr_desc<BN, F16>();
             const uint64_t da0 = smem_desc_k_sw128(smem_a), db0 = smem_desc_k_sw128(smem_b);
             uint32_t stage = 0, par = 0;
+            const int accs = C::ACCS > 1 ? p.accs : 1;
             bool ok = true, landed = false;
             int local = 0;
             for (int t = pair_id; t < p.tiles_total && ok; t += pairs, ++local) {
@@ -224,7 +233,8 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 ok = __all_sync(0xffffffffu, mbar_wait(acc_empty + 8 * slot, ((uint32_t)(local >> 1) & 1u) ^ 1u, &s_abort, p.status, 64));
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t acc = tmem + slot * (uint32_t)BN;
+                const uint32_t acc0 = tmem + slot * (uint32_t)C::TILE_COLS;
+                uint32_t acc = acc0;
                 int chunk = 0;
                 for (int i = 0; i < p.iters; i += CPS) {
                     if (!landed) {
@@ -246,23 +256,25 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                         if (last1) chunk = 0;
                         ks1 = last1 ? p.last_ksteps : 4;
                     }
+                    const bool used = i >= accs * CPS;                // the accumulator holds an earlier stage's sums
                     if (elect_one()) {
                         if (CPS == 2 && ks0 + ks1 == 8) {
 #pragma unroll
                             for (int k = 0; k < 8; ++k)
                                 mma<F16>(acc, da + (k >> 2) * (A_CHUNK_BYTES >> 4) + 2 * (k & 3), db + (k >> 2) * (C::B_CHUNK_BYTES >> 4) + 2 * (k & 3),
-                                         idesc, (i | k) ? 1u : 0u);
+                                         idesc, (used || k) ? 1u : 0u);
                         } else if (CPS == 1 && ks0 == 4) {
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) mma<F16>(acc, da + 2 * k, db + 2 * k, idesc, (i | k) ? 1u : 0u);
+                            for (int k = 0; k < 4; ++k) mma<F16>(acc, da + 2 * k, db + 2 * k, idesc, (used || k) ? 1u : 0u);
                         } else {
-                            for (int k = 0; k < ks0; ++k) mma<F16>(acc, da + 2 * k, db + 2 * k, idesc, (i | k) ? 1u : 0u);
+                            for (int k = 0; k < ks0; ++k) mma<F16>(acc, da + 2 * k, db + 2 * k, idesc, (used || k) ? 1u : 0u);
                             for (int k = 0; k < ks1; ++k)
                                 mma<F16>(acc, da + (A_CHUNK_BYTES >> 4) + 2 * k, db + (C::B_CHUNK_BYTES >> 4) + 2 * k, idesc, 1u);
                         }
                         commit_both(empty_bar + 8 * stage);
                         if (i + CPS >= p.iters) commit_both(acc_full + 8 * slot);
                     }
+                    if (C::ACCS > 1) { acc += (uint32_t)BN; if (acc == acc0 + (uint32_t)(accs * BN)) acc = acc0; }
                     landed = __all_sync(0xffffffffu, peek);
                     stage = next;
                     par = next_par;
@@ -277,6 +289,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         const int c_begin = group ? HALF : 0, c_end = group ? NCH : HALF;
         const uint32_t box = store + (uint32_t)(4 * group + quarter) * BOX_BYTES;
         const uint32_t empty0 = map_to_cta(acc_empty, 0);
+        const int accs = C::ACCS > 1 ? p.accs : 1;
         int local = 0;
         for (int t = pair_id; t < p.tiles_total; t += pairs, ++local) {
             const int tm = t / p.tiles_n, k0 = (t - tm * p.tiles_n) * BN;
@@ -297,12 +310,20 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                          : "=r"(stop) : "r"((uint32_t)s_abort) : "memory");
             if (stop) break;
             tc_fence_after();
-            const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + slot * (uint32_t)BN;
+            const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + slot * (uint32_t)C::TILE_COLS;
 #pragma unroll 1
             for (int c = c_begin; c < c_end; ++c) {
                 uint32_t v[32];
                 tmem_ld_32cols(trow + 32 * c, v);
                 tmem_ld_wait();
+#pragma unroll 1
+                for (int a = 1; a < accs; ++a) {
+                    uint32_t u[32];
+                    tmem_ld_32cols(trow + (uint32_t)(a * BN + 32 * c), u);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(u[j]));
+                }
                 if (c + 1 == c_end) {                  // the accumulator has been read: hand it back to the issuer
                     tc_fence_before();
                     __syncwarp();

@@ -4,7 +4,7 @@ pairs (both accumulators in turn), staged output through tensor stores.  Integer
 import numpy as np
 import pytest
 
-from helpers import oracle_out, run_planned
+from helpers import FP32_TOL, assert_parity, oracle_out, run_planned
 from paper_1606_00094_b200 import workloads as wl
 
 pytestmark = pytest.mark.gpu
@@ -55,3 +55,33 @@ def test_pair_tiles_in_a_chain(tile, consumer):
     a = orc.conv_fwd(a.astype(np.float32), *params[1], stride=1, pad=1, relu=True).astype(np.float32)
     a = ((a.view(np.int32) + 0x1000) & ~0x1FFF).view(np.float32)
     np.testing.assert_array_equal(got.astype(np.float64), orc.maxpool_fwd(a), err_msg=str(descs))
+
+
+def _as_tf32(a):
+    """The value the staging kernel stores: nearest TF32, ties away."""
+    return ((a.view(np.int32) + 0x1000) & ~0x1FFF).view(np.float32)
+
+
+def _accumulation_error(shape, math, **plan):
+    """Real-valued operands; the oracle is fed what the staging kernel stores, which leaves fp32 accumulation as the only difference."""
+    N, C, H, W, K, R, S, *_ = shape
+    x, w, b = wl.half_normal(9700, (N, C, H, W)), wl.normal(9701, (K, C, R, S), 0.0, (2.0 / (C * R * S)) ** 0.5), wl.normal(9702, (K,), 0.0, 0.01)
+    staged = [a.astype(np.float16).astype(np.float32) if math == 4 else _as_tf32(a) for a in (x, w)]
+    got, desc = run_planned(shape, x, w, b, math=math, **plan)
+    return assert_parity(got, oracle_out(shape, *staged, b), FP32_TOL, desc), desc
+
+
+@pytest.mark.parametrize("shape", [(2, 512, 13, 13, 100, 3, 3, 1, 1, 1), (3, 1024, 14, 14, 160, 1, 1, 1, 0, 0), (2, 70, 13, 13, 70, 5, 5, 1, 2, 0)])
+@pytest.mark.parametrize("tile", [26, 28, 30])
+@pytest.mark.parametrize("math", [0, 4])
+def test_real_valued_sums(shape, tile, math):
+    _, desc = _accumulation_error(shape, math, variant=1 if shape[5] * shape[6] == 1 else 2, tile_id=tile, s2d=0)
+    assert "pair_256" in desc
+
+
+def test_longest_sums_by_rule():
+    """Layers of several rounds of tiles, which suit the pairs, with reductions of 7100 and 11650: the FP32 bar on staged operands
+    holds for what the rule picks."""
+    _accumulation_error((47, 284, 24, 24, 84, 5, 5, 1, 2, 0), 4)
+    _accumulation_error((11, 466, 28, 28, 59, 5, 5, 1, 2, 0), 4)
+    _accumulation_error((11, 466, 28, 28, 59, 5, 5, 1, 2, 0), 0)

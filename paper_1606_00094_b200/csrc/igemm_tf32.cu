@@ -999,8 +999,13 @@ double model_cost_pair(const ConvDims& d, int BN, int taps, int cchunks, int las
     const double rounds = (double)((tiles + sm_count / 2 - 1) / (sm_count / 2));
     const double full = BN <= 64 ? 270.0 : BN <= 96 ? 315.0 : BN <= 128 ? 345.0 : BN <= 192 ? 405.0 : 525.0;
     const double quarter = 220.0 + 0.77 * BN;
-    const double per_tile = taps * ((cchunks - 1) * full + std::max(quarter, full * last / 4.0));
-    return rounds * per_tile + 5000.0 + 32.0 * BN;
+    // A tile's epilogue runs under the next tile's main loop where that is the longer of the two.  Its clocks are fitted to 160 layers
+    // of 1 ... 36 steps a tile, every tile timed: the tile picked from pairs and one-CTA tiles is within 0.4 % of the best in the
+    // geometric mean, against 3.7 % with the epilogue left out (1x1 on 75 channels, 356 filters, 13x13, batch 227: 33 us on the tile picked
+    // then, 26 on the gather kernel).
+    const double epilogue = 3500.0 + 8.0 * BN;
+    const double per_tile = std::max(epilogue, taps * ((cchunks - 1) * full + std::max(quarter, full * last / 4.0)));
+    return rounds * per_tile + 5300.0 + 32.0 * BN;
 }
 
 // Accumulators of a pair tile, and the MMA steps that each of them takes.  At 1.6e-8 a step (pair::Cfg::ACCS) 256 steps keep a sum
@@ -1285,6 +1290,9 @@ int igemm_plan_create(const ConvDims& d_in, int variant, int tile_id, int split_
         if (tile_id >= 0 && t != tile_id) continue;
         const int nacc = kTileNacc[t];
         if (nacc == -4) {
+            // Not on a space-to-depth view by rule: its staging takes what the pairs save.  Of eleven first layers that this rule once
+            // moved here all were slower than before (7x7 stride 2, 48 filters, 178x178, batch 56: 130 us against 90 on the gather kernel).
+            if (use_s2d && s2d < 0) continue;
             if (mode == 1 || split_k > 1 || pair_steps(d, kTileBN[t], p->chunk(), p->half) > kMaxPairSteps) continue;
             if (max_ws > 0 && (((size_t)d.N * d.H * d.W * p->Cs() * p->esize() + 1023) & ~(size_t)1023) > max_ws) continue;
             const double c = staging_cost(d_in, d, p->Cp) + model_cost_pair(d, kTileBN[t], d.R * d.S, p->Cp / p->chunk(), last_ksteps(d, p->chunk(), p->half), p->sm_count);

@@ -85,3 +85,25 @@ def test_longest_sums_by_rule():
     _accumulation_error((47, 284, 24, 24, 84, 5, 5, 1, 2, 0), 4)
     _accumulation_error((11, 466, 28, 28, 59, 5, 5, 1, 2, 0), 4)
     _accumulation_error((11, 466, 28, 28, 59, 5, 5, 1, 2, 0), 0)
+
+
+@pytest.mark.parametrize("tile", [26, 28, 30])
+@pytest.mark.parametrize("shape", [(3, 8, 31, 29, 70, 5, 5, 2, 2, 1), (2, 3, 67, 67, 100, 11, 11, 4, 0, 1), (2, 20, 22, 23, 33, 3, 3, 3, 1, 0)])
+def test_pair_tiles_on_a_space_to_depth_view_exact(shape, tile):
+    N, C, H, W, K, R, S, *_ = shape
+    x, w, b = wl.integers(9800, (N, C, H, W)), wl.integers(9801, (K, C, R, S)), wl.integers(9802, (K,))
+    for bind in (False, True):
+        got, desc = run_planned(shape, x, w, b, variant=2, tile_id=tile, s2d=1, bind=bind)
+        assert "pair_256" in desc and "s2d" in desc
+        np.testing.assert_array_equal(got.astype(np.float64), oracle_out(shape, x, w, b), err_msg=desc)
+
+
+@pytest.mark.parametrize("shape", [(14, 3, 150, 150, 48, 7, 7, 2, 0, 1), (33, 3, 215, 215, 48, 5, 5, 2, 2, 1),       # strided first layers
+                                   (227, 75, 13, 13, 356, 1, 1, 1, 0, 1)])                                           # three steps a tile
+def test_rule_leaves_these_to_the_gather_kernel(shape):
+    from paper_1606_00094_b200 import binding as B
+    plan = B.ConvPlan(shape)
+    try:
+        assert "gconv" in plan.describe()
+    finally:
+        plan.close()

@@ -9,6 +9,7 @@
 // gives, for reduction index j = (c, r, s), the element offset inside an image and the tap, so the
 // load needs no division.  Bias and ReLU are applied in registers before the store.
 #include <algorithm>
+#include <cmath>
 
 #include "boda_internal.h"
 #include "simt_conv.h"
@@ -494,6 +495,30 @@ static double gemm_cost(const ConvDims& d, int t, int split)
            (splits > 1 ? m->cluster + 300.0 * splits : 0.0);
 }
 
+// Do the pixel-per-thread forms suit the layer, and with how many output channels per thread (0: no)?  They have no channel tile to
+// fill and no chunk hand-overs, but load more per multiply-add.
+//  * up to kFewIndices reduction indices: yes (27 indices, 16 filters, 32x32: 3.1 against 3.3 us at batch 1, 12.5 against 19.4 at 256);
+//  * up to 512: where few filters leave the narrowest GEMM-blocked tile mostly empty.  The logarithm of what the run-time compiled form
+//    gains over the best of those tiles, linear in the logarithms of the sizes, is fitted to 517 layers timed both ways (rms 0.2): 7x7
+//    on 5 channels, one filter, 56x59, batch 15: 9.6 against 28.9 us; 5x5 on 2 channels, 4 filters, 42x45, batch 9: 3.2 against 4.8; the
+//    other way 3x3 on 13 channels, 4 filters, 30x32, batch 1.  With the margin of 0.12 the choice gains 11 % over those layers in the
+//    geometric mean (the best choice 14.6 %) and is more than 3 % behind the tiles on ten of them.
+//  * never with a stride (27 indices with stride 2, 96 filters, batch 7: 17.8 against 16.0 us).
+static int pixel_channels(const ConvDims& d)
+{
+    if (d.stride != 1 || d.K > 128) return 0;
+    if (d.Kred <= kFewIndices) return 8;
+    if (d.Kred > 512 || d.K > 32) return 0;
+    const double m = std::min(std::log(d.M / 10000.0), 4.1), c = std::log((double)d.C), w = std::log((double)(d.R * d.S));
+    auto gain = [&](int kt, double k1, double km, double k, double kkm, double kc, double kw, double kmc, double kmw) {
+        const double k16 = std::log((double)((d.K + 15) / 16 * 16) / ((d.K + kt - 1) / kt * kt));       // channels paid for, tile / form
+        return k1 + km * m + k * k16 + kkm * k16 * m + kc * c + kw * w + kmc * m * c + kmw * m * w;
+    };
+    const double g4 = gain(4, -0.285, -0.339, 0.331, 0.129, -0.114, 0.078, 0.076, 0.078);
+    const double g8 = gain(8, -0.296, -0.310, 0.586, 0.167, -0.114, 0.060, 0.085, 0.079);
+    return std::max(g4, g8) < 0.12 ? 0 : g4 >= g8 ? 4 : 8;
+}
+
 int direct_pick_split(const ConvDims& d, int tile)
 {
     if (tile < 0 || tile >= kNumTiles || kTiles[tile].kind != TILE_GEMM) return 1;
@@ -517,15 +542,11 @@ int direct_tile_staged_width(int tile) { return tile >= 0 && tile < kNumTiles &&
 
 int direct_pick_tile(const ConvDims& d, size_t max_ws)
 {
-    // a handful of reduction indices and many output pixels: the pixel-per-thread form, the smallest KT that covers K in one group
-    // (or 32 channels per group).  Measured against the GEMM-blocked tiles: 18.3 against 19.4 us for 3x3 on 3 channels, 16 filters,
-    // 32x32, batch 256; from 45 indices on, or with a stride, the GEMM-blocked tiles win (75 indices, 48 filters, stride 2, batch
-    // 46: 28.8 against 56.4 us).
-    if (d.Kred <= kFewIndices && d.stride == 1 && d.K <= 128 && d.M >= 32768) {
-        const int KT = d.K <= 8 ? 8 : d.K <= 16 ? 16 : 32;
-        int ih, iw, iwp;
-        size_t smem;
-        if (pixel_geometry(d, KT, &ih, &iw, &iwp, &smem)) return kFirstPixelTile + (KT == 8 ? 0 : KT == 16 ? 1 : 2);
+    // many output pixels where the pixel-per-thread form suits: the smallest KT that covers K in one group (or 32 channels per
+    // group).  Measured against the GEMM-blocked tiles: 18.3 against 19.4 us for 3x3 on 3 channels, 16 filters, 32x32, batch 256.
+    if (d.M >= 32768 && pixel_channels(d) > 0) {
+        const int t = kFirstPixelTile + (d.K <= 8 ? 0 : d.K <= 16 ? 1 : 2);
+        if (direct_tile_legal(d, t)) return t;
     }
     int best = 8;
     double best_cost = 1e300;
@@ -558,17 +579,16 @@ int direct_tile_rtc_kt(int tile_id) { return (tile_id >= 0 && tile_id < kNumTile
 
 int direct_rtc_pick(const ConvDims& d)
 {
-    // Measured on B200: the run-time compiled kernel beats the GEMM-blocked tiles where the reduction is a handful of indices (27
-    // indices, 16 filters, 32x32: 3.1 against 3.3 us at batch 1, 12.5 against 19.4 us at batch 256) and loses beyond, or with a
-    // stride (45 indices: 4.9 against 4.2 us; 27 with stride 2, 96 filters, batch 7: 17.8 against 16.0 us; 375 indices: 9.5 against 4.6).
-    // Eight channels per thread as a rule; four where that leaves fewer than 64 blocks (more blocks hide the
-    // staging latency); sixteen where 16 covers all output channels of a large layer (the input patch is staged once).
-    if (d.Kred > kFewIndices || d.stride != 1 || d.K > 128 || !direct_rtc_available()) return -1;
+    // Where the pixel-per-thread form suits.  Eight channels per thread as a rule; four where that leaves fewer than 64 blocks (more
+    // blocks hide the staging latency); sixteen where 16 covers all output channels of a large layer (the input patch is staged
+    // once); for the longer reductions what pixel_channels() says.
+    const int suits = pixel_channels(d);
+    if (suits == 0 || !direct_rtc_available()) return -1;
     int bx = 32, by = 8, py = 1;
     size_t sm = 0;
     if (!direct_rtc_geometry(d, 8, &bx, &by, &py, &sm)) bx = 8, by = 4, py = 1;
     const long long blocks8 = (long long)((d.Q + bx - 1) / bx) * ((d.P + by * py - 1) / (by * py)) * d.N * ((d.K + 7) / 8);
-    const int want = (d.K <= 16 && d.M >= 16384) ? 16 : blocks8 < 64 ? 4 : 8;
+    const int want = d.Kred > kFewIndices ? suits : (d.K <= 16 && d.M >= 16384) ? 16 : blocks8 < 64 ? 4 : 8;
     const int order[3][3] = {{4, 8, 16}, {8, 4, 16}, {16, 8, 4}};
     const int* o = order[want == 4 ? 0 : want == 8 ? 1 : 2];
     for (int i = 0; i < 3; ++i)

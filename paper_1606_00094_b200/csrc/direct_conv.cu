@@ -503,12 +503,15 @@ static double gemm_cost(const ConvDims& d, int t, int split)
 //    on 5 channels, one filter, 56x59, batch 15: 9.6 against 28.9 us; 5x5 on 2 channels, 4 filters, 42x45, batch 9: 3.2 against 4.8; the
 //    other way 3x3 on 13 channels, 4 filters, 30x32, batch 1.  With the margin of 0.12 the choice gains 11 % over those layers in the
 //    geometric mean (the best choice 14.6 %) and is more than 3 % behind the tiles on ten of them.
+//    One channel up to 81 indices and two up to 50 gain 9 to 66 % whatever the fit says, but for
+//    narrow images and many filters on many points (5x5 on 2 channels, 15 filters, 52x52, batch 2:
+//    3.2 / 4.0 us); beyond the set's 64 channels nothing is known.
 //  * never with a stride (27 indices with stride 2, 96 filters, batch 7: 17.8 against 16.0 us).
 static int pixel_channels(const ConvDims& d)
 {
     if (d.stride != 1 || d.K > 128) return 0;
     if (d.Kred <= kFewIndices) return 8;
-    if (d.Kred > 512 || d.K > 32) return 0;
+    if (d.Kred > 512 || d.K > 32 || d.C > 64) return 0;
     const double m = std::min(std::log(d.M / 10000.0), 4.1), c = std::log((double)d.C), w = std::log((double)(d.R * d.S));
     auto gain = [&](int kt, double k1, double km, double k, double kkm, double kc, double kw, double kmc, double kmw) {
         const double k16 = std::log((double)((d.K + 15) / 16 * 16) / ((d.K + kt - 1) / kt * kt));       // channels paid for, tile / form
@@ -516,7 +519,8 @@ static int pixel_channels(const ConvDims& d)
     };
     const double g4 = gain(4, -0.285, -0.339, 0.331, 0.129, -0.114, 0.078, 0.076, 0.078);
     const double g8 = gain(8, -0.296, -0.310, 0.586, 0.167, -0.114, 0.060, 0.085, 0.079);
-    return std::max(g4, g8) < 0.12 ? 0 : g4 >= g8 ? 4 : 8;
+    const bool always = (d.C == 1 ? d.Kred <= 81 : d.C == 2 && d.Kred <= 50) && d.Q >= 12 && (d.K <= 16 || d.M <= 4096);
+    return !always && std::max(g4, g8) < 0.12 ? 0 : g4 >= g8 ? 4 : 8;
 }
 
 int direct_pick_split(const ConvDims& d, int tile)

@@ -212,7 +212,7 @@ def test_rtc_tile_with_several_rows_per_thread(rows, monkeypatch):
     np.testing.assert_array_equal(got.astype(np.float64), oracle_out(shape, x, w, b), err_msg=desc)
 
 
-@pytest.mark.parametrize("shape,rtc", [((15, 5, 56, 59, 1, 7, 7, 1, 3, 1), True), ((13, 7, 56, 58, 1, 5, 5, 1, 2, 1), True), ((9, 2, 42, 45, 4, 5, 5, 1, 2, 1), True),
+@pytest.mark.parametrize("shape,rtc", [((15, 5, 56, 59, 1, 7, 7, 1, 3, 1), True), ((13, 7, 56, 58, 1, 5, 5, 1, 2, 1), True), ((9, 2, 42, 45, 4, 5, 5, 1, 2, 1), True), ((2, 2, 52, 52, 15, 5, 5, 1, 2, 1), True), ((3, 73, 20, 22, 2, 1, 1, 1, 0, 1), False),
                                        ((1, 13, 30, 32, 4, 3, 3, 1, 1, 1), False), ((4, 13, 57, 57, 9, 3, 3, 2, 1, 1), False)])
 def test_few_filters_pick_the_run_time_compiled_form(shape, rtc):
     """Where the narrowest GEMM-blocked tile would mostly multiply channels that are not there."""

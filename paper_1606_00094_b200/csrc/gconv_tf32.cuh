@@ -287,7 +287,6 @@ gconv_tf32_kernel(const __grid_constant__ CUtensorMap map_b, const GconvParams p
         }
     }
     tc_fence_before();
-    if (s_abort) settle_after_abort();
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();

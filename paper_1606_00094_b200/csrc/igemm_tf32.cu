@@ -465,7 +465,6 @@ igemm_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         cluster_arrive();
         cluster_wait();
     }
-    if (s_abort) settle_after_abort();
     __syncthreads();
     if (p.splits > 1) {
         if (!exchange) {

@@ -236,7 +236,6 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         }
     }
     tc_fence_before();
-    if (s_abort) settle_after_abort();
     __syncthreads();
     if (p.splits > 1) {
         // step 2: every CTA of the cluster sums its share of the channels over all peers' parked accumulators in rank

@@ -358,7 +358,6 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         if (p.out_tma && lane == 0) bulk_wait_all();
     }
     tc_fence_before();
-    if (s_abort) settle_after_abort();
     __syncthreads();
     cluster_sync_all();              // nobody leaves while the peer may still signal its barriers or its MMAs read this shared memory
     if (warp == 1) {

@@ -180,10 +180,7 @@ simt_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         int chunk = i0 % p.cchunks;
         for (int it = i0; it < i1; ++it) {
             if (loader) (void)load_step();
-            if (!mbar_wait(full_bar + 8 * stage, par, &s_abort, p.status, 52)) {
-                if (loader) settle_after_abort();        // the loads in flight are this thread's; the block's memory stays until it leaves
-                return;
-            }
+            if (!mbar_wait(full_bar + 8 * stage, par, &s_abort, p.status, 52)) return;
             __syncwarp();                // the loading lane rejoins its warp
             const uint8_t* a_row = smem + stage * G::STAGE_BYTES + m_local * 128;
             const uint8_t* b_row = smem + stage * G::STAGE_BYTES + A_STAGE_BYTES + n_local * 128;

@@ -72,6 +72,15 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// The thread whose wait ran out stays for half a millisecond, a hundred times what the slowest copy takes: copies into the CTA's
+// shared memory and MMAs that read it may still be under way, and their barriers may never complete (a byte count that was not posted).
+// The others leave their loops at once and meet it at the kernel's last barrier; a CTA's memory is its own until its last thread leaves.
+static __device__ __noinline__ void settle_after_abort()
+{
+    const long long t0 = clock64();
+    while (clock64() - t0 < 1000000) __nanosleep(1000);
+}
+
 // Bounded wait.  Returns false if the CTA is aborting or the limit expired (then it raises the abort flag
 // and records where it gave up).  The limit is counted on the SM's own cycle counter, which is cheap to read
 // (the global nanosecond timer is not, and must stay out of the fast path): 4e9 cycles, about two seconds.
@@ -91,6 +100,7 @@ static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity
                     status[2] = (int)(blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z));
                     status[3] = where;
                 }
+                settle_after_abort();
                 return false;
             }
         }
@@ -100,15 +110,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 {
     if (mbar_try_wait(bar, parity)) return true;
     return mbar_wait_slow(bar, parity, abort_flag, status, where);
-}
-
-// For a CTA that is giving up, before its last barrier: copies into its shared memory and MMAs that read it may still be under way,
-// and their barriers may never complete (a byte count that was not posted), so what is waited for is time: half a millisecond, a
-// hundred times what the slowest of them takes.
-static __device__ __noinline__ void settle_after_abort()
-{
-    const long long t0 = clock64();
-    while (clock64() - t0 < 1000000) __nanosleep(1000);
 }
 
 // Bounded wait for threads that are not on the critical path (the epilogue waiting for the accumulator):
@@ -127,6 +128,7 @@ static __device__ __noinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t par
                 status[2] = (int)(blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z));
                 status[3] = where;
             }
+            settle_after_abort();
             return false;
         }
         __nanosleep(200);

@@ -307,7 +307,6 @@ tconv_first_layer_kernel(const __grid_constant__ CUtensorMap map_b0, const __gri
         if (etid == 0) FL_STAMP(7);
         tc_fence_before();
     }
-    if (s_abort) settle_after_abort();
     __syncthreads();
     if (warp == 1) {
         __syncwarp();

@@ -464,7 +464,6 @@ tconv_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                                 s_bias, &s_abort, accum_bar, f0, k0, warp, lane);
         tc_fence_before();
     }
-    if (s_abort) settle_after_abort();
     __syncthreads();
     if (p.splits > 1) {
         // Split reduction through the cluster (one CTA per split), one 128-row accumulator at a time: park the

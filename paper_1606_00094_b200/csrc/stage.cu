@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "stage.h"
 
@@ -14,6 +15,10 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kMaxSmemTaps = 36;             // filter taps staged through shared memory (8 warps x 32 channels x taps floats)
+// Larger windows are dealt out in runs of taps, 32 bytes of each channel's row: with all the taps of 32 channels on one warp the
+// filters of an 11x11 layer (150 channels, 22 filters) took 30 us, the layer 75 us instead of 45.  They have a form of the kernel
+// of their own: with both in one the other windows' filters took 0.5 to 1.2 us longer.
+constexpr int kTapRun = 8;
 
 __device__ __forceinline__ float rna(float x)
 {
@@ -54,8 +59,8 @@ __device__ __forceinline__ void put1(void* base, size_t row, int Cp, int c, floa
 }
 
 // Blocks [0, filter_blocks) stage the filters, the rest the input.
-// PX: points per input tile (32 channels each).
-template <int MODE, int PX>
+// PX: points per input tile (32 channels each).  RUNS: filters of more than kMaxSmemTaps taps.
+template <int MODE, int PX, bool RUNS>
 __global__ void __launch_bounds__(kThreads)
 stage_kernel(const StageInput x, const StageFilters w, int filter_blocks, int m_tiles)
 {
@@ -93,7 +98,7 @@ stage_kernel(const StageInput x, const StageFilters w, int filter_blocks, int m_
         return;
     }
     pdl_wait();
-    if (w.RS == 1) {
+    if (!RUNS && w.RS == 1) {
         // ---- 1x1 filters are [K][C] rows already: a copy with rounding and padding, 512 consecutive channels' worth per warp
         const long long total = (long long)w.K * w.Cp;
         const long long base = ((long long)blockIdx.x * 8 + warp) * 512;
@@ -115,12 +120,18 @@ stage_kernel(const StageInput x, const StageFilters w, int filter_blocks, int m_
     }
     // ---- filters: a warp takes 32 channels of one output channel: 32*RS consecutive floats in, RS rows of 32 channels out
     const int cblocks = w.Cp >> 5;
-    const long long unit = (long long)blockIdx.x * 8 + warp;
+    long long unit = (long long)blockIdx.x * 8 + warp;
+    int t0 = 0;
+    if constexpr (RUNS) {
+        const int runs = (w.RS + kTapRun - 1) / kTapRun;
+        t0 = kTapRun * (int)(unit % runs);
+        unit /= runs;
+    }
     if (unit >= (long long)w.K * cblocks) return;
     const int k = (int)(unit / cblocks), c0 = 32 * (int)(unit - (long long)k * cblocks);
     const float* src = w.filt + ((size_t)k * w.C + c0) * w.RS;
     const int live = min(32, w.C - c0);                                  // channels that exist (may be 0 or less)
-    if (w.RS <= kMaxSmemTaps) {
+    if constexpr (!RUNS) {
         float* s = sm + warp * 32 * w.RS;
         const int n = max(live, 0) * w.RS;
         int i = lane;
@@ -135,9 +146,12 @@ stage_kernel(const StageInput x, const StageFilters w, int filter_blocks, int m_
         __syncwarp();
         for (int t = 0; t < w.RS; ++t) put1<MODE>(w.wp, (size_t)t * w.K + k, w.Cp, c0 + lane, s[lane * w.RS + t]);
     } else {
-#pragma unroll 4
-        for (int t = 0; t < w.RS; ++t)
-            put1<MODE>(w.wp, (size_t)t * w.K + k, w.Cp, c0 + lane, lane < live ? __ldg(src + lane * w.RS + t) : 0.f);
+        float v[kTapRun];
+#pragma unroll
+        for (int u = 0; u < kTapRun; ++u) v[u] = lane < live && t0 + u < w.RS ? __ldg(src + lane * w.RS + t0 + u) : 0.f;
+#pragma unroll
+        for (int u = 0; u < kTapRun; ++u)
+            if (t0 + u < w.RS) put1<MODE>(w.wp, (size_t)(t0 + u) * w.K + k, w.Cp, c0 + lane, v[u]);
     }
 }
 
@@ -154,19 +168,21 @@ int stage_operands(StageMode mode, const StageInput* input, const StageFilters* 
         if (w.RS == 1) {
             fblocks = ((long long)w.K * w.Cp + 8 * 512 - 1) / (8 * 512);
         } else {
-            fblocks = ((long long)w.K * (w.Cp / 32) + 7) / 8;
+            const int runs = w.RS <= kMaxSmemTaps ? 1 : (w.RS + kTapRun - 1) / kTapRun;
+            fblocks = ((long long)w.K * (w.Cp / 32) * runs + 7) / 8;
             if (w.RS <= kMaxSmemTaps) smem = (size_t)8 * 32 * w.RS * sizeof(float);
         }
     }
     // Wide tiles keep more loads in flight per thread and win once they fill the SMs a few times over; below, narrow tiles
-    // spread the same loads over more blocks.  Measured, whole layer: 3x3 on 256 channels, 13x13, batch 20 (216 wide tiles)
-    // 20.8 us wide, 19.0 narrow; 49x51 on 97 channels (320) 12.7 wide, 13.1 narrow; 39x39 on 333, batch 8 (1140) 15.2 / 18.0.
+    // spread the same loads over more blocks.  Measured, whole layer, wide against 32-point tiles, over 117 layers by their number of
+    // wide tiles: 296 ... 400 0.97 x the speed, 400 ... 450 1.01, 600 ... 800 1.07, 800 ... 1200 1.1 (3x3 on 256 channels, 13x13, batch 20,
+    // 216 of them: 20.8 us wide, 19.0 narrow; 39x39 on 333 channels, batch 8, 1140: 15.2 / 18.0).
     // The split staging writes twice as much per load: 41x41 on 32 channels, batch 31 (408) 30.1 wide, 29.4 narrow.
     bool wide = false;
     if (input) {
         x = *input;
         const long long M = (long long)x.N * x.HW;
-        wide = (M + 127) / 128 * (x.Cp / 32) >= (mode == STAGE_TF32_SPLIT ? 148 * 8 : 148 * 2);
+        wide = (M + 127) / 128 * (x.Cp / 32) >= (mode == STAGE_TF32_SPLIT ? 148 * 8 : 400);
         const int px = wide ? 128 : 32;
         m_tiles = (M + px - 1) / px;
         iblocks = m_tiles * (x.Cp / 32);
@@ -174,15 +190,19 @@ int stage_operands(StageMode mode, const StageInput* input, const StageFilters* 
     }
     if (fblocks + iblocks > 0x7fffffffLL || m_tiles > 0x7fffffffLL) return BODA_ERR_TOO_LARGE;
     const dim3 grid((unsigned)(fblocks + iblocks)), block(kThreads);
-    auto run = [&](auto narrow_kernel, auto wide_kernel) {
-        return launch_kernel(wide ? wide_kernel : narrow_kernel, grid, block, smem, stream, 1, x, w, (int)fblocks, (int)m_tiles);
+    auto run = [&](auto mode) {
+        constexpr int MODE = decltype(mode)::value;
+        const bool runs = w.RS > kMaxSmemTaps;
+        return launch_kernel(wide ? (runs ? stage_kernel<MODE, 128, true> : stage_kernel<MODE, 128, false>)
+                                  : (runs ? stage_kernel<MODE, 32, true> : stage_kernel<MODE, 32, false>),
+                             grid, block, smem, stream, 1, x, w, (int)fblocks, (int)m_tiles);
     };
     cudaError_t e;
     switch (mode) {
-        case STAGE_TF32: e = run(stage_kernel<STAGE_TF32, 32>, stage_kernel<STAGE_TF32, 128>); break;
-        case STAGE_TF32_SPLIT: e = run(stage_kernel<STAGE_TF32_SPLIT, 32>, stage_kernel<STAGE_TF32_SPLIT, 128>); break;
-        case STAGE_F16: e = run(stage_kernel<STAGE_F16, 32>, stage_kernel<STAGE_F16, 128>); break;
-        default: e = run(stage_kernel<STAGE_FP32, 32>, stage_kernel<STAGE_FP32, 128>); break;
+        case STAGE_TF32: e = run(std::integral_constant<int, STAGE_TF32>()); break;
+        case STAGE_TF32_SPLIT: e = run(std::integral_constant<int, STAGE_TF32_SPLIT>()); break;
+        case STAGE_F16: e = run(std::integral_constant<int, STAGE_F16>()); break;
+        default: e = run(std::integral_constant<int, STAGE_FP32>()); break;
     }
     if (e != cudaSuccess) return record_cuda_error(e, "stage_kernel");
     count_launch();

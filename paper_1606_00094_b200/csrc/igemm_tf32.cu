@@ -1004,7 +1004,7 @@ double model_cost_pair(const ConvDims& d, int BN, int taps, int cchunks, int las
     // then, 26 on the gather kernel).
     const double epilogue = 3500.0 + 8.0 * BN;
     const double per_tile = std::max(epilogue, taps * ((cchunks - 1) * full + std::max(quarter, full * last / 4.0)));
-    return rounds * per_tile + 5300.0 + 32.0 * BN;
+    return rounds * per_tile + 5000.0 + 32.0 * BN;
 }
 
 // Accumulators of a pair tile, and the MMA steps that each of them takes.  At 1.6e-8 a step (pair::Cfg::ACCS) 256 steps keep a sum

@@ -1082,8 +1082,15 @@ int launch_pair(IgemmPlan* p, const pair::PairParams& prm, cudaStream_t stream)
         return launch_clusters(kernel, dim3(2 * std::min(prm.tiles_total, p->sm_count / 2)), dim3(pair::kThreads), (size_t)smem, stream,
                                dim3(2, 1, 1), p->map_a, p->map_b, p->map_o, prm);
     };
-    static DeviceSmemLimit limit_tf32, limit_f16;
-    BODA_CUDA_TRY(p->half ? run(pair::pair_conv_kernel<BN, true>, limit_f16) : run(pair::pair_conv_kernel<BN, false>, limit_tf32));
+    static DeviceSmemLimit limit_tf32, limit_f16, limit_tf32_multi, limit_f16_multi;
+    if constexpr (C::ACCS > 1) {
+        if (prm.accs > 1) {
+            BODA_CUDA_TRY(p->half ? run(pair::pair_conv_kernel<BN, true, true>, limit_f16_multi) : run(pair::pair_conv_kernel<BN, false, true>, limit_tf32_multi));
+            count_launch();
+            return BODA_OK;
+        }
+    }
+    BODA_CUDA_TRY(p->half ? run(pair::pair_conv_kernel<BN, true, false>, limit_f16) : run(pair::pair_conv_kernel<BN, false, false>, limit_tf32));
     count_launch();
     return BODA_OK;
 }

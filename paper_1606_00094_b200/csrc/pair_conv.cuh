@@ -55,11 +55,10 @@ template <int BN> struct Cfg {
     // Accumulators that a tile may have, taking the stages in turn; two tiles' worth fill tensor memory.  The tensor core truncates
     // an accumulator at every MMA, so the error of a sum grows with the MMAs that one accumulator takes: measured 1.6e-8 of the
     // result per MMA (1563 of them 2.5e-5).  Reading more than one back costs a short reduction up to 10 % (its epilogue does not
-    // hide under the next tile), so only the longer ones have them (PairParams::accs).
+    // hide under the next tile), and a changing accumulator address the issue loop 1 to 2 %, so only the longer reductions have
+    // them (PairParams::accs), in a form of the kernel of their own (MULTI).
     static constexpr int ACCS = BN <= 64 ? 4 : BN <= 128 ? 2 : 1;
-    static constexpr int TILE_COLS = ACCS * BN;
-    static constexpr int TMEM_COLS = 512;
-    static_assert(2 * TILE_COLS <= TMEM_COLS, "two tiles fit");
+    static_assert(2 * ACCS * BN <= 512, "two tiles fit");
     // (the boxes are only there where the output leaves through tensor stores: without them a CTA can become resident beside the
     // staging kernel's and overlap its prologue)
     static constexpr int smem_bytes(bool boxes) { return STAGES * STAGE_BYTES + 256 /*barriers*/ + (boxes ? STORE_BYTES : 0) + 1024 /*alignment*/; }
@@ -107,13 +106,15 @@ __host__ __device__ constexpr uint32_t instr_desc()
     return ((F16 ? instr_desc_f16<BN>() : instr_desc_tf32<BN>()) & ~(0x1Fu << 24)) | ((uint32_t)(256 >> 4) << 24);
 }
 
-template <int BN, bool F16>
+template <int BN, bool F16, bool MULTI>
 __global__ void __launch_bounds__(kThreads, 1)
 pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_o,
                  const PairParams p)
 {
     using C = Cfg<BN>;
     constexpr int STAGES = C::STAGES, CH = F16 ? 64 : 32;
+    constexpr int ACCS = MULTI ? C::ACCS : 1, TILE_COLS = ACCS * BN;
+    constexpr int TMEM_COLS = 2 * TILE_COLS <= 128 ? 128 : 2 * TILE_COLS <= 256 ? 256 : 512;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     constexpr int CPS = C::CPS, A_STAGE_BYTES = CPS * A_CHUNK_BYTES, B_STAGE_BYTES = CPS * C::B_CHUNK_BYTES;
@@ -141,7 +142,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         if (p.out_tma) prefetch_tensormap(&map_o);
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"((uint32_t)C::TMEM_COLS) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"((uint32_t)TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
@@ -225,7 +226,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             constexpr uint32_t idesc = instr_desc<BN, F16>();
             const uint64_t da0 = smem_desc_k_sw128(smem_a), db0 = smem_desc_k_sw128(smem_b);
             uint32_t stage = 0, par = 0;
-            const int accs = C::ACCS > 1 ? p.accs : 1;
+            const int accs = ACCS > 1 ? p.accs : 1;
             bool ok = true, landed = false;
             int local = 0;
             for (int t = pair_id; t < p.tiles_total && ok; t += pairs, ++local) {
@@ -233,7 +234,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 ok = __all_sync(0xffffffffu, mbar_wait(acc_empty + 8 * slot, ((uint32_t)(local >> 1) & 1u) ^ 1u, &s_abort, p.status, 64));
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t acc0 = tmem + slot * (uint32_t)C::TILE_COLS;
+                const uint32_t acc0 = tmem + slot * (uint32_t)TILE_COLS;
                 uint32_t acc = acc0;
                 int chunk = 0;
                 for (int i = 0; i < p.iters; i += CPS) {
@@ -274,7 +275,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                         commit_both(empty_bar + 8 * stage);
                         if (i + CPS >= p.iters) commit_both(acc_full + 8 * slot);
                     }
-                    if (C::ACCS > 1) { acc += (uint32_t)BN; if (acc == acc0 + (uint32_t)(accs * BN)) acc = acc0; }
+                    if (ACCS > 1) { acc += (uint32_t)BN; if (acc == acc0 + (uint32_t)(accs * BN)) acc = acc0; }
                     landed = __all_sync(0xffffffffu, peek);
                     stage = next;
                     par = next_par;
@@ -289,7 +290,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         const int c_begin = group ? HALF : 0, c_end = group ? NCH : HALF;
         const uint32_t box = store + (uint32_t)(4 * group + quarter) * BOX_BYTES;
         const uint32_t empty0 = map_to_cta(acc_empty, 0);
-        const int accs = C::ACCS > 1 ? p.accs : 1;
+        const int accs = ACCS > 1 ? p.accs : 1;
         int local = 0;
         for (int t = pair_id; t < p.tiles_total; t += pairs, ++local) {
             const int tm = t / p.tiles_n, k0 = (t - tm * p.tiles_n) * BN;
@@ -310,7 +311,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                          : "=r"(stop) : "r"((uint32_t)s_abort) : "memory");
             if (stop) break;
             tc_fence_after();
-            const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + slot * (uint32_t)C::TILE_COLS;
+            const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + slot * (uint32_t)TILE_COLS;
 #pragma unroll 1
             for (int c = c_begin; c < c_end; ++c) {
                 uint32_t v[32];
@@ -362,7 +363,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     cluster_sync_all();              // nobody leaves while the peer may still signal its barriers or its MMAs read this shared memory
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)C::TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS) : "memory");
     }
 }
 

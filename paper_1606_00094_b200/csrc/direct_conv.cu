@@ -416,27 +416,27 @@ int launch_pixel(const ConvDims& d, const float* in, const float* filt, const fl
     }
 }
 
-// bm x bn outputs per block of `threads` threads, reduction chunks of bk (GEMM-blocked form; 0 otherwise)
-struct TileInfo { int kind, bm, bn, kt, threads, bk; const char* name; };
+// bm x bn outputs per block, reduction chunks of bk (GEMM-blocked form; 0 otherwise)
+struct TileInfo { int kind, bm, bn, kt, bk; const char* name; };
 enum { TILE_GEMM = 0, TILE_PIXEL = 1, TILE_RTC = 2, TILE_STAGED = 3 };
 constexpr TileInfo kTiles[] = {
-    {TILE_GEMM, 128, 128, 0, 256, 8, "direct_128x128"}, {TILE_GEMM, 128, 96, 0, 256, 16, "direct_128x96"},
-    {TILE_GEMM, 128, 64, 0, 128, 8, "direct_128x64"},   {TILE_GEMM, 128, 32, 0, 128, 8, "direct_128x32"},
-    {TILE_GEMM, 64, 64, 0, 64, 8, "direct_64x64"},     {TILE_GEMM, 64, 32, 0, 64, 8, "direct_64x32"},
-    {TILE_GEMM, 64, 16, 0, 64, 8, "direct_64x16"},      {TILE_GEMM, 32, 32, 0, 64, 16, "direct_32x32"},
-    {TILE_GEMM, 32, 16, 0, 32, 8, "direct_32x16"},
+    {TILE_GEMM, 128, 128, 0, 8, "direct_128x128"}, {TILE_GEMM, 128, 96, 0, 16, "direct_128x96"},
+    {TILE_GEMM, 128, 64, 0, 8, "direct_128x64"},   {TILE_GEMM, 128, 32, 0, 8, "direct_128x32"},
+    {TILE_GEMM, 64, 64, 0, 8, "direct_64x64"},     {TILE_GEMM, 64, 32, 0, 8, "direct_64x32"},
+    {TILE_GEMM, 64, 16, 0, 8, "direct_64x16"},      {TILE_GEMM, 32, 32, 0, 16, "direct_32x32"},
+    {TILE_GEMM, 32, 16, 0, 8, "direct_32x16"},
     // pixel-per-thread form: kt output channels per thread
-    {TILE_PIXEL, 0, 0, 8, 256, 0, "direct_pixel_k8"}, {TILE_PIXEL, 0, 0, 16, 256, 0, "direct_pixel_k16"},
-    {TILE_PIXEL, 0, 0, 32, 256, 0, "direct_pixel_k32"},
+    {TILE_PIXEL, 0, 0, 8, 0, "direct_pixel_k8"}, {TILE_PIXEL, 0, 0, 16, 0, "direct_pixel_k16"},
+    {TILE_PIXEL, 0, 0, 32, 0, "direct_pixel_k32"},
     // the same form compiled at run time for the exact shape (direct_rtc.cu)
-    {TILE_RTC, 0, 0, 4, 0, 0, "direct_rtc_k4"}, {TILE_RTC, 0, 0, 8, 0, 0, "direct_rtc_k8"},
-    {TILE_RTC, 0, 0, 16, 0, 0, "direct_rtc_k16"}, {TILE_RTC, 0, 0, 32, 0, 0, "direct_rtc_k32"},
+    {TILE_RTC, 0, 0, 4, 0, "direct_rtc_k4"}, {TILE_RTC, 0, 0, 8, 0, "direct_rtc_k8"},
+    {TILE_RTC, 0, 0, 16, 0, "direct_rtc_k16"}, {TILE_RTC, 0, 0, 32, 0, "direct_rtc_k32"},
     // more GEMM-blocked tiles (the ids above are part of the interface)
-    {TILE_GEMM, 64, 48, 0, 64, 8, "direct_64x48"}, {TILE_GEMM, 128, 48, 0, 128, 8, "direct_128x48"},
+    {TILE_GEMM, 64, 48, 0, 8, "direct_64x48"}, {TILE_GEMM, 128, 48, 0, 8, "direct_128x48"},
     // over a staged NHWC copy of the input (simt_conv.cu): needs workspace
-    {TILE_STAGED, 128, 128, 0, 288, 32, "direct_nhwc_128x128"}, {TILE_STAGED, 128, 96, 0, 288, 32, "direct_nhwc_128x96"},
-    {TILE_STAGED, 128, 64, 0, 288, 32, "direct_nhwc_128x64"},   {TILE_STAGED, 128, 48, 0, 288, 32, "direct_nhwc_128x48"},
-    {TILE_STAGED, 128, 32, 0, 288, 32, "direct_nhwc_128x32"},
+    {TILE_STAGED, 128, 128, 0, 32, "direct_nhwc_128x128"}, {TILE_STAGED, 128, 96, 0, 32, "direct_nhwc_128x96"},
+    {TILE_STAGED, 128, 64, 0, 32, "direct_nhwc_128x64"},   {TILE_STAGED, 128, 48, 0, 32, "direct_nhwc_128x48"},
+    {TILE_STAGED, 128, 32, 0, 32, "direct_nhwc_128x32"},
 };
 constexpr int kFirstPixelTile = 9;
 constexpr int kFewIndices = 32;      // reductions up to here suit the pixel-per-thread forms

@@ -635,30 +635,6 @@ pack_filters_s2d_kernel(const float* __restrict__ filt, float* __restrict__ wp, 
 
 // ------------------------------------------------------------------------------------------------
 // Host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-typedef CUresult (*EncodeIm2colFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const int*, const int*, cuuint32_t, cuuint32_t, const cuuint32_t*,
-                                   CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                   CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode_tiled = nullptr;
-EncodeIm2colFn g_encode_im2col = nullptr;
-
-int load_driver_entry_points()
-{
-    if (g_encode_tiled && g_encode_im2col) return BODA_OK;
-    void* f1 = nullptr;
-    void* f2 = nullptr;
-    cudaDriverEntryPointQueryResult q1, q2;
-    BODA_CUDA_TRY(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f1, cudaEnableDefault, &q1));
-    BODA_CUDA_TRY(cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &f2, cudaEnableDefault, &q2));
-    if (!f1 || !f2 || q1 != cudaDriverEntryPointSuccess || q2 != cudaDriverEntryPointSuccess) return BODA_ERR_UNSUPPORTED;
-    g_encode_tiled = (EncodeTiledFn)f1;
-    g_encode_im2col = (EncodeIm2colFn)f2;
-    return BODA_OK;
-}
-
 // Tile table.  Ids 16..19: gather kernel (gconv_tf32.cuh; NCHW input, tconv with short reductions and k1conv).
 // Ids 0..4: im2col kernel (any stride; k1conv and tconv).  Ids 5..12: halo kernel (tconv, stride 1)
 // with NACC accumulators of 128 rows each (ids 5..8: 1, 9..12: 2, 13..15: 4).
@@ -1247,13 +1223,13 @@ int encode_map_b(IgemmPlan* p)
 int igemm_plan_create(const ConvDims& d_in, int variant, int tile_id, int split_k, int s2d, int* d_status, IgemmPlan** out, int mode,
                       size_t max_ws)
 {
-    // mode 1 (error-compensated TF32) and mode 2 (fp16 operands) run on the im2col kernel only, NCHW in and out
+    // mode 1 (error-compensated TF32) runs on the im2col kernel only, mode 2 (fp16 operands) on that and on CTA pairs; NCHW in and out
     const bool x3 = mode != 0;
     if (!igemm_variant_legal(d_in, variant)) return BODA_ERR_UNSUPPORTED;
     // strided tconv layers may run as their stride-1 space-to-depth view
     ConvDims d = d_in;
     bool use_s2d = false;
-    if (x3 && s2d > 0) return BODA_ERR_UNSUPPORTED;      // the error-compensated mode runs on the im2col kernel only
+    if (x3 && s2d > 0) return BODA_ERR_UNSUPPORTED;      // neither mode has a space-to-depth view
     const bool force_gather = tile_id >= kFirstGatherTile && tile_id < kFirstK1nTile;
     if (force_gather && (s2d > 0 || !gather_legal(d_in, variant, x3))) return BODA_ERR_UNSUPPORTED;
     if (variant == BODA_VARIANT_TCONV && s2d != 0 && !x3 && !force_gather) {

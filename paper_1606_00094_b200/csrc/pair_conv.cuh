@@ -287,6 +287,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         const int quarter = warp & 3, group = warp >= 7 ? 1 : 0;
         const int etid = threadIdx.x - (group ? 96 : 64);
         constexpr int NCH = BN / 32, HALF = (NCH + 1) / 2;
+        static_assert(NCH >= 2, "both groups have channels, and with them a last chunk that hands the accumulator back");
         const int c_begin = group ? HALF : 0, c_end = group ? NCH : HALF;
         const uint32_t box = store + (uint32_t)(4 * group + quarter) * BOX_BYTES;
         const uint32_t empty0 = map_to_cta(acc_empty, 0);
@@ -349,11 +350,6 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 } else {
                     store_row32(p.o, d, k0 + 32 * c, y);
                 }
-            }
-            if (c_begin == c_end) {                    // a group without channels still hands the accumulator back
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" :: "r"(empty0 + 8 * slot) : "memory");
             }
         }
         if (p.out_tma && lane == 0) bulk_wait_all();

@@ -40,7 +40,7 @@ constexpr int kThreads = 32 * kWarps;
 constexpr int kMinSteps = 4;                             // reduction steps a CTA is worth starting for
 
 struct SimtParams {
-    int M, C, K, P, Q, PQ, stride, pad, S;
+    int M, K, Q, PQ, stride, pad, S;
     int cchunks, last_groups;                            // 32-channel chunks; 4-channel groups of the last one that hold data
     int steps;                                           // reduction steps per tile: taps * cchunks
     int tiles_n, whole_tiles, cut_tiles;                 // tiles computed whole, then tiles cut into equal pieces
@@ -280,29 +280,6 @@ simt_sum_kernel(const SimtParams p, int ctas)
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                  CUtensorMapFloatOOBfill);
-typedef CUresult (*EncodeIm2colFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const int*,
-                                   const int*, cuuint32_t, cuuint32_t, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode_tiled = nullptr;
-EncodeIm2colFn g_encode_im2col = nullptr;
-
-int load_encoders()
-{
-    if (g_encode_tiled && g_encode_im2col) return BODA_OK;
-    void *f1 = nullptr, *f2 = nullptr;
-    cudaDriverEntryPointQueryResult q1, q2;
-    BODA_CUDA_TRY(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f1, cudaEnableDefault, &q1));
-    BODA_CUDA_TRY(cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &f2, cudaEnableDefault, &q2));
-    if (!f1 || !f2 || q1 != cudaDriverEntryPointSuccess || q2 != cudaDriverEntryPointSuccess) return BODA_ERR_UNSUPPORTED;
-    g_encode_tiled = (EncodeTiledFn)f1;
-    g_encode_im2col = (EncodeIm2colFn)f2;
-    return BODA_OK;
-}
-
-constexpr int kWidths[] = {128, 96, 64, 48, 32};
 constexpr int kSms = 148;
 
 struct Schedule { int tiles_m, tiles_n, steps, ctas, whole, cut; };
@@ -315,7 +292,8 @@ Schedule schedule(const ConvDims& d, int bn, int sms)
     s.steps = d.R * d.S * ((d.C + BKC - 1) / BKC);
     const long long tiles = (long long)s.tiles_m * s.tiles_n;
     // whole rounds stay uncut except the last full one, which is cut together with the remainder: a CTA then has between one
-    // and two tiles' worth of cut work and at most two pieces
+    // and two tiles' worth of cut work.  (With fewer CTAs than SMs, where a tile has less than kMinSteps steps, it has more.)  At
+    // most two of its pieces are partial, its first and its last; what lies between is whole tiles.
     const long long rounds = tiles / sms;
     s.whole = tiles % sms == 0 ? (int)tiles : (int)(rounds > 1 ? (rounds - 1) * sms : 0);
     s.cut = (int)(tiles - s.whole);
@@ -327,7 +305,7 @@ Schedule schedule(const ConvDims& d, int bn, int sms)
 
 struct SimtPlan {
     ConvDims d;
-    int bn = 128, Cp = 32, sms = kSms;
+    int bn = 128, Cp = 32;
     Schedule s;
     float* d_wp = nullptr;
     size_t xp_bytes = 0;
@@ -342,9 +320,6 @@ bool simt_legal(const ConvDims& d)
     // limits of the im2col loads (window offsets and pads are small signed numbers)
     return d.R <= 11 && d.S <= 11 && d.stride <= 8 && d.pad <= 100 && d.P > 0 && d.Q > 0 && (long long)d.M * ((d.K + 31) / 32) <= 0x7fffffffLL;
 }
-
-int simt_num_widths() { return (int)(sizeof(kWidths) / sizeof(kWidths[0])); }
-int simt_width(int i) { return kWidths[i]; }
 
 static size_t staged_bytes(const ConvDims& d)
 {
@@ -374,7 +349,7 @@ double simt_cost(const ConvDims& d, int bn)
 int simt_plan_create(const ConvDims& d, int bn, int* d_status, SimtPlan** out)
 {
     if (!simt_legal(d)) return BODA_ERR_UNSUPPORTED;
-    int rc = load_encoders();
+    int rc = load_driver_entry_points();
     if (rc != BODA_OK) return rc;
     SimtPlan* p = new (std::nothrow) SimtPlan();
     if (!p) return BODA_ERR_NOMEM;
@@ -458,7 +433,7 @@ int simt_launch(SimtPlan* p, const float* in, const float* filt, const float* bi
     }
     if (after_staging) BODA_CUDA_TRY(cudaEventRecord(after_staging, stream));
     SimtParams prm;
-    prm.M = d.M; prm.C = d.C; prm.K = d.K; prm.P = d.P; prm.Q = d.Q; prm.PQ = d.P * d.Q;
+    prm.M = d.M; prm.K = d.K; prm.Q = d.Q; prm.PQ = d.P * d.Q;
     prm.stride = d.stride; prm.pad = d.pad; prm.S = d.S;
     prm.cchunks = p->Cp / BKC;
     prm.last_groups = (d.C - BKC * (prm.cchunks - 1) + 3) / 4;

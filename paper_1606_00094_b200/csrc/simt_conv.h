@@ -7,10 +7,8 @@ namespace boda {
 
 struct SimtPlan;
 
-// bn: output channels per tile (one of simt_widths()); BODA_ERR_UNSUPPORTED for windows or pads the im2col loads do not take.
+// bn: output channels per tile, 128, 96, 64, 48 or 32.  simt_legal: false for windows or pads the im2col loads do not take.
 bool simt_legal(const ConvDims& d);
-int simt_num_widths();
-int simt_width(int i);
 double simt_cost(const ConvDims& d, int bn);                 // estimated SM clocks of one call, staging included
 size_t simt_workspace_bytes(const ConvDims& d, int bn);
 int simt_plan_create(const ConvDims& d, int bn, int* d_status, SimtPlan** out);

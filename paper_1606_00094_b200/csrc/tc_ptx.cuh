@@ -81,6 +81,29 @@ static __device__ __noinline__ void settle_after_abort()
     while (clock64() - t0 < 1000000) __nanosleep(1000);
 }
 
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
+                                  CUtensorMapFloatOOBfill);
+typedef CUresult (*EncodeIm2colFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const int*,
+                                   const int*, cuuint32_t, cuuint32_t, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+static EncodeTiledFn g_encode_tiled = nullptr;
+static EncodeIm2colFn g_encode_im2col = nullptr;
+
+// The driver's tensor-map encoders, looked up on first use.
+[[maybe_unused]] static int load_driver_entry_points()
+{
+    if (g_encode_tiled && g_encode_im2col) return BODA_OK;
+    void *f1 = nullptr, *f2 = nullptr;
+    cudaDriverEntryPointQueryResult q1, q2;
+    BODA_CUDA_TRY(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f1, cudaEnableDefault, &q1));
+    BODA_CUDA_TRY(cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &f2, cudaEnableDefault, &q2));
+    if (!f1 || !f2 || q1 != cudaDriverEntryPointSuccess || q2 != cudaDriverEntryPointSuccess) return BODA_ERR_UNSUPPORTED;
+    g_encode_tiled = (EncodeTiledFn)f1;
+    g_encode_im2col = (EncodeIm2colFn)f2;
+    return BODA_OK;
+}
+
 // Bounded wait.  Returns false if the CTA is aborting or the limit expired (then it raises the abort flag
 // and records where it gave up).  The limit is counted on the SM's own cycle counter, which is cheap to read
 // (the global nanosecond timer is not, and must stay out of the fast path): 4e9 cycles, about two seconds.

@@ -786,7 +786,8 @@ int igemm_split_candidate(int i) { return kSplitCandidates[i]; }
 namespace {
 
 // Cost model (SM clocks) used when a plan is not tuned by timing; fitted to a sweep of every tile and split over
-// fourteen layer shapes on B200 (its choice is within 3 % of the best measured one for each of them).
+// fourteen layer shapes on B200, within 3 % of the best measured choice for each; one floor for every width costs up to
+// 7 % elsewhere (3x3 on 384 channels, 256 filters, 13x13, batch 20).
 //   main loop: a stage costs about 2.1*BN clocks of MMAs or 380 of producer / issuer hand-shakes, whichever
 //              is longer (halo kernel: 2.2*BN per accumulator, or 290 per accumulator + 390);
 //   fixed:     prologue, pipeline fill and tail, about 3500 clocks (halo kernel 5000);

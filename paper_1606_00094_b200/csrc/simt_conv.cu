@@ -14,7 +14,7 @@
 //
 // Measured, 3x3 on 256 channels, 384 filters, 13x13, batch 20 (6.0 GFLOP, 80 us at the pipe's 74 TFLOP/s): 499 us on the
 // GEMM-blocked kernel as it was (4-byte gather, 32x32 tiles), 171 us on its packed and split successor, 136 us here (staging
-// 3, main kernel 126, sums 5); the FP32 pipe is busy 73 % of the main kernel.  16 warps of 8 x 4 pairs instead of 8 of 8 x 8
+// of both operands, the main kernel's 126, sums 5): the main kernel runs at 64 % of the pipe's peak rate.  16 warps of 8 x 4 pairs instead of 8 of 8 x 8
 // took 159 us (more operand loads per multiply-add), two CTAs per SM with plain fmaf 174 us (register-bank conflicts).
 #include <cuda.h>
 

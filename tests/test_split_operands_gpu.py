@@ -66,6 +66,32 @@ def test_no_further_off_than_fp32_arithmetic(shape, tile):
     assert orc.rel_l2(runs[0], ref) <= 1.3e-7 + 2.0 ** -24 * (1.0 + np.sqrt(C * R * S / 256.0))
 
 
+@pytest.mark.parametrize("bits", [0x3f80ffff, 0x3f807f40])
+@pytest.mark.parametrize("tile", [23, 24, 25, 26])
+def test_products_of_the_worst_operands(bits, tile):
+    """All operands the value whose parts leave most out: with parts cut off, 0x3f80ffff (ml + lm is 2^-21 of the product); with parts rounded to
+    nearest, 0x3f807f40 (2^-24).  64 equal products: sums of hh and of the mixed ones are exact, or off by 2^-24 once; one more
+    rounding where they meet."""
+    from oracle import conv_oracle as orc
+    value = np.uint32(bits).view(np.float32)
+    x, w = np.full((1, 64, 5, 5), value, np.float32), np.full((70, 64, 1, 1), value, np.float32)
+    shape = (1, 64, 5, 5, 70, 1, 1, 1, 0, 0)
+    got, desc = run_planned(shape, x, w, None, variant=0, math=1, tile_id=tile)
+    assert orc.rel_l2(got, oracle_out(shape, x, w, None)) <= 3 * 2.0 ** -24, desc
+
+
+def test_an_infinity_times_the_smallest_values_is_one():
+    for value in (1e-45, -1e-42, 9e-41, 0.0):
+        x, w = np.full((1, 1, 4, 4), np.inf, np.float32), np.full((1, 1, 1, 1), value, np.float32)
+        for args in ((x, w), (np.full_like(x, value), np.full_like(w, np.inf))):
+            import torch
+            from paper_1606_00094_b200 import binding as B
+            plan = B.ConvPlan((1, 1, 4, 4, 1, 1, 1, 1, 0, 0), math=1, variant=0, tile_id=24)
+            got = plan(*[torch.from_numpy(t).cuda() for t in args]).cpu().numpy()
+            plan.close()
+            assert np.isnan(got).all() if value == 0 else np.array_equal(got, np.full_like(got, np.copysign(np.inf, value)))
+
+
 @pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan, 3.4e38])
 def test_infinities_and_nans_come_out_as_from_fp32_arithmetic(bad):
     import torch

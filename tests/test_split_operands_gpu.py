@@ -52,6 +52,35 @@ def test_operands_keep_all_their_bits():
     np.testing.assert_array_equal(got, np.broadcast_to(x[0, :, 4, 4][None, :, None, None], got.shape))
 
 
+@pytest.mark.parametrize("tile", [24, 26])
+def test_small_and_large_operands_keep_all_their_bits(tile):
+    """The same for operands from 2^-124, whose last bit is 2^-147, to 2^127."""
+    rng = np.random.default_rng(4)
+    size = (2, 33, 9, 9)
+    x = (rng.uniform(1, 2, size) * rng.choice([-1, 1], size)).astype(np.float32)
+    x = np.ldexp(x, rng.choice([-124, -123, -120, -116, -111, -109, -80, 0, 100, 126, 127], size)).astype(np.float32)
+    w = np.zeros((33, 33, 3, 3), np.float32)
+    w[np.arange(33), np.arange(33), 1, 1] = 1.0
+    shape = (2, 33, 9, 9, 33, 3, 3, 1, 1, 0)
+    x = np.where(np.arange(33)[None, :, None, None] == 5, np.float32(np.finfo(np.float32).max), x)
+    got, desc = run_planned(shape, x, w, None, variant=0, math=1, tile_id=tile)
+    np.testing.assert_array_equal(got, x, err_msg=desc)
+    f = x[0, :, 4, 4]
+    got, desc = run_planned(shape, np.ones_like(x), w * f[:, None, None, None], None, variant=0, math=1, tile_id=tile)
+    np.testing.assert_array_equal(got, np.broadcast_to(f[None, :, None, None], got.shape), err_msg=desc)
+
+
+@pytest.mark.parametrize("kw", [dict(variant=0, math=1, tile_id=t) for t in (23, 24, 25, 26)] + [dict(variant=2, math=3, tile_id=t) for t in (32, 34)])
+@pytest.mark.parametrize("scale", [-118, 110])
+def test_layers_of_small_and_large_operands(scale, kw):
+    """No further off than with operands around one (the bound of test_no_further_off_than_fp32_arithmetic)."""
+    from oracle import conv_oracle as orc
+    shape = (2, 256, 13, 13, 96, 3, 3, 1, 1, 0)
+    x, w = np.ldexp(wl.half_normal(1, shape[:1] + shape[1:4]), scale).astype(np.float32), wl.normal(2, (96, 256, 3, 3), 0, (2.0 / 2304) ** 0.5)
+    got, desc = run_planned(shape, x, w, None, **kw)
+    assert orc.rel_l2(np.ldexp(got.astype(np.float64), -scale), np.ldexp(oracle_out(shape, x, w, None), -scale)) <= 1.3e-7 + 2.0 ** -24 * (1.0 + np.sqrt(2304 / 256.0)), desc
+
+
 @pytest.mark.parametrize("shape", [(2, 256, 13, 13, 96, 3, 3, 1, 1, 1), (1, 900, 6, 6, 64, 5, 5, 1, 2, 0)])
 @pytest.mark.parametrize("tile", [23, 24, 25, 26])
 def test_no_further_off_than_fp32_arithmetic(shape, tile):

@@ -117,8 +117,9 @@ int direct_num_tiles();
 const char* direct_tile_name(int tile_id);
 // max_ws: 0, or the largest workspace the caller accepts
 int direct_pick_tile(const ConvDims& d, size_t max_ws = 0);
-// estimated SM clocks of the best GEMM-blocked tile and split; false from direct_mask_fits for windows whose bounds tests are not a mask
-double direct_gemm_cost(const ConvDims& d);
+// the best GEMM-blocked tile (precompiled, nothing staged) and the estimated SM clocks of it with its best split; false from
+// direct_mask_fits for windows whose bounds tests are not a mask
+int direct_pick_gemm_tile(const ConvDims& d, double* clocks);
 bool direct_mask_fits(const ConvDims& d);
 // output channels per tile of the tiles that run over a staged copy of the input (simt_conv.h); 0 for the others
 int direct_tile_staged_width(int tile_id);

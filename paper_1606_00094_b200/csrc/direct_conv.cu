@@ -534,11 +534,15 @@ static int pixel_channels(const ConvDims& d)
 
 bool direct_mask_fits(const ConvDims& d) { return d.R * d.S <= kMaskTaps; }
 
-double direct_gemm_cost(const ConvDims& d)
+int direct_pick_gemm_tile(const ConvDims& d, double* clocks)
 {
-    double best = 1e300;
-    for (const GemmModel& m : kGemmModel) best = std::min(best, gemm_cost(d, m.tile, direct_pick_split(d, m.tile)));
-    return best;
+    int tile = -1;
+    *clocks = 1e300;
+    for (const GemmModel& m : kGemmModel) {
+        const double c = gemm_cost(d, m.tile, direct_pick_split(d, m.tile));
+        if (c < *clocks) { *clocks = c; tile = m.tile; }
+    }
+    return tile;
 }
 
 int direct_pick_split(const ConvDims& d, int tile)

@@ -14,7 +14,7 @@ IN_PLACE = [
     (2, 505, 15, 15, 31, 1, 1, 1, 0, 0),         # 4.8 / 9.1
     (4, 9, 15, 15, 29, 5, 5, 1, 2, 1),           # 5.0 / 10.6
     (1, 17, 19, 21, 105, 3, 3, 2, 1, 1),         # 4.4 / 7.9
-    (1, 7, 39, 42, 16, 1, 1, 1, 0, 1),           # 3.1 / 5.8, run-time compiled
+    (1, 7, 39, 42, 16, 1, 1, 1, 0, 1),           # 3.1 / 5.8
 ]
 TENSOR = [
     (5, 480, 14, 14, 192, 1, 1, 1, 0, 1),        # 11.5 / 6.5
@@ -51,6 +51,23 @@ def test_small_layers_run_in_place(shape):
         got, desc = run_planned(shape, x, w, b, **kw)
         assert "math=tf32" in desc
         assert_parity(got, ref, TF32_TOL, desc)
+
+
+# layers that the run-time compiled tiles suit
+SUIT_COMPILED = [(1, 7, 39, 42, 16, 1, 1, 1, 0, 1), (2, 8, 25, 25, 24, 1, 1, 1, 0, 1), (3, 30, 13, 13, 100, 1, 1, 1, 0, 1), (2, 20, 40, 40, 16, 3, 3, 1, 1, 1)]
+
+
+@pytest.mark.parametrize("shape", SUIT_COMPILED)
+def test_the_rule_compiles_nothing_at_run_time(shape):
+    """A compilation would sit in the first one-call of a shape, or in a plan whose tensor-core kernel needed none."""
+    from paper_1606_00094_b200 import binding as B
+    plan = B.ConvPlan(shape)
+    desc = plan.describe()
+    plan.close()
+    assert "rtc" not in desc
+    x, w, b = _tensors(shape)
+    got, desc = run_planned(shape, x, w, b)
+    assert_parity(got, oracle_out(shape, x, w, b), FP32_TOL if "variant=direct" in desc else TF32_TOL, desc)
 
 
 @pytest.mark.parametrize("shape", TENSOR)

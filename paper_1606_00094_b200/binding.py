@@ -8,13 +8,14 @@ if the library is missing, importing this module raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional
 
-from .build import CALLS_PATH, LIB_PATH
+from .build import LIB_PATH, calls_path
 
-for _path in (LIB_PATH, CALLS_PATH):
-    if not os.path.exists(_path):
+for _path in (LIB_PATH, calls_path()):
+    if _path and not os.path.exists(_path):
         raise RuntimeError(
             f"{_path} is missing: build it with `python -m paper_1606_00094_b200.build` "
             "(there is no CPU fallback)")
@@ -170,7 +171,9 @@ def _load_calls():
     global _calls
     if _calls is None:
         _load_torch()
-        from . import _torch_calls
+        spec = importlib.util.spec_from_file_location("_torch_calls", calls_path())
+        _torch_calls = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(_torch_calls)
         _torch_calls.bind(*[ctypes.cast(f, _vp).value for f in (_lib.boda_conv_fwd_planned, _lib.boda_conv_fwd, _lib.boda_sgemm,
                                                                   _lib.boda_conv_out_dim)])
         _calls = _torch_calls

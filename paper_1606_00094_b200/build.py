@@ -1,11 +1,12 @@
 """Builds the CUDA library (``libboda.so``) in-tree with nvcc for sm_100a, and with g++ the extension through which the
-binding calls it with torch tensors (``_torch_calls.so``).
+binding calls it with torch tensors (``_torch_calls-<python>-<torch>.so``).
 
     python -m paper_1606_00094_b200.build [--force] [--verbose]
 """
 from __future__ import annotations
 
 import glob
+import importlib.metadata
 import os
 import shutil
 import subprocess
@@ -17,7 +18,7 @@ _ROOT = os.path.dirname(_PKG)
 CSRC = os.path.join(_PKG, "csrc")
 LIB_PATH = os.path.join(_PKG, "libboda.so")
 CALLS_SRC = os.path.join(CSRC, "torch_calls.cpp")
-CALLS_PATH = os.path.join(_PKG, "_torch_calls.so")
+CALLS_HEADER = os.path.join(_ROOT, "include", "boda.h")
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"] + os.environ.get("BODA_NVCC_EXTRA", "").split()
 
@@ -46,23 +47,43 @@ def _headers():
         + glob.glob(os.path.join(_ROOT, "include", "*.h"))
 
 
-def build_calls(force: bool = False) -> str:
-    """Compile the extension over torch tensors; returns its path."""
-    if not force and os.path.exists(CALLS_PATH) and os.path.getmtime(CALLS_PATH) > os.path.getmtime(CALLS_SRC):
-        return CALLS_PATH
+def calls_path():
+    """Where the extension for this Python and the installed torch lies (None: no torch).  It is bound to the C++ interfaces of both, so
+    another version of either looks for another file."""
+    try:
+        version = importlib.metadata.version("torch")
+    except importlib.metadata.PackageNotFoundError:
+        return None
+    return os.path.join(_PKG, f"_torch_calls-{sys.implementation.cache_tag}-torch{version}.so")
+
+
+def calls_stale() -> bool:
+    path = calls_path()
+    return path is not None and (not os.path.exists(path) or
+                                 os.path.getmtime(path) <= max(os.path.getmtime(p) for p in (CALLS_SRC, CALLS_HEADER)))
+
+
+def build_calls(force: bool = False):
+    """Compile the extension over torch tensors; returns its path (None without torch: the library serves raw addresses)."""
+    path = calls_path()
+    if path is None or not (force or calls_stale()):
+        return path
     import torch
     from torch.utils import cpp_extension
-    tmp = CALLS_PATH + f".tmp{os.getpid()}"
+    tmp = path + f".tmp{os.getpid()}"
     cuda_home = os.path.dirname(os.path.dirname(_nvcc()))
     includes = [sysconfig.get_paths()["include"], *cpp_extension.include_paths(), os.path.join(cuda_home, "include")]
     libs = os.path.join(os.path.dirname(torch.__file__), "lib")
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
-    cmd += [a for i in includes for a in ("-isystem", i)] + ["-o", tmp, CALLS_SRC, "-L", libs]
+    cmd += [a for i in includes for a in ("-isystem", i)] + ["-I", os.path.dirname(CALLS_HEADER), "-o", tmp, CALLS_SRC, "-L", libs]
     res = subprocess.run(cmd + ["-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"], capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError("g++ failed:\n" + res.stdout + res.stderr)
-    os.replace(tmp, CALLS_PATH)
-    return CALLS_PATH
+    os.replace(tmp, path)
+    for old in glob.glob(os.path.join(_PKG, "_torch_calls*.so")):
+        if old != path:
+            os.remove(old)
+    return path
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:

@@ -15,16 +15,14 @@
 
 #include <climits>
 
+#include "boda.h"
+
 namespace {
 
-using Planned = int (*)(void*, const float*, const float*, const float*, float*, void*, void*);
-using Forward = int (*)(const float*, const float*, const float*, float*, int, int, int, int, int, int, int, int, int, int, void*);
-using Sgemm = int (*)(const float*, const float*, float*, int, int, int, void*);
-using OutDim = int (*)(int, int, int, int);
-Planned g_planned = nullptr;
-Forward g_forward = nullptr;
-Sgemm g_sgemm = nullptr;
-OutDim g_out_dim = nullptr;
+decltype(&boda_conv_fwd_planned) g_planned = nullptr;
+decltype(&boda_conv_fwd) g_forward = nullptr;
+decltype(&boda_sgemm) g_sgemm = nullptr;
+decltype(&boda_conv_out_dim) g_out_dim = nullptr;
 
 // A plain tensor (or parameter) with CUDA memory of its own.
 const at::Tensor* plain(PyObject* o)
@@ -66,7 +64,7 @@ PyObject* planned(PyObject*, PyObject* const* a, Py_ssize_t n)
     if (n != 7 || !PyLong_CheckExact(a[0]) || !optional(a[1], &ws) || !PyTuple_CheckExact(a[2]) || PyTuple_GET_SIZE(a[2]) != 4 ||
         !(x = plain(a[3])) || !(filt = plain(a[4])) || !optional(a[5], &bias) || !optional(a[6], &out) || at::impl::torch_function_mode_enabled())
         Py_RETURN_NONE;
-    void* handle = PyLong_AsVoidPtr(a[0]);
+    auto* handle = static_cast<boda_conv_plan*>(PyLong_AsVoidPtr(a[0]));
     if (PyErr_Occurred()) { PyErr_Clear(); Py_RETURN_NONE; }
     at::Tensor fresh;
     int64_t shape[4] = {0, 0, 0, 0};
@@ -145,10 +143,10 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n)
         p[i] = PyLong_AsVoidPtr(a[i]);
         if (PyErr_Occurred()) return nullptr;
     }
-    g_planned = reinterpret_cast<Planned>(p[0]);
-    g_forward = reinterpret_cast<Forward>(p[1]);
-    g_sgemm = reinterpret_cast<Sgemm>(p[2]);
-    g_out_dim = reinterpret_cast<OutDim>(p[3]);
+    g_planned = reinterpret_cast<decltype(g_planned)>(p[0]);
+    g_forward = reinterpret_cast<decltype(g_forward)>(p[1]);
+    g_sgemm = reinterpret_cast<decltype(g_sgemm)>(p[2]);
+    g_out_dim = reinterpret_cast<decltype(g_out_dim)>(p[3]);
     Py_RETURN_NONE;
 }
 

@@ -10,15 +10,15 @@ from __future__ import annotations
 import ctypes
 import importlib.util
 import os
+import warnings
 from typing import Optional
 
 from .build import LIB_PATH, calls_path
 
-for _path in (LIB_PATH, calls_path()):
-    if _path and not os.path.exists(_path):
-        raise RuntimeError(
-            f"{_path} is missing: build it with `python -m paper_1606_00094_b200.build` "
-            "(there is no CPU fallback)")
+if not os.path.exists(LIB_PATH):
+    raise RuntimeError(
+        f"{LIB_PATH} is missing: build it with `python -m paper_1606_00094_b200.build` "
+        "(there is no CPU fallback)")
 
 _lib = ctypes.CDLL(LIB_PATH)
 
@@ -161,6 +161,16 @@ def _load_torch():
     return _torch
 
 
+class _CtypesOnly:
+    """In the place of the extension where it cannot be loaded: every call is left to ctypes."""
+
+    @staticmethod
+    def _leave(*args):
+        return None
+
+    planned = conv_fwd = sgemm = _leave
+
+
 _calls = None
 
 
@@ -171,12 +181,19 @@ def _load_calls():
     global _calls
     if _calls is None:
         _load_torch()
-        spec = importlib.util.spec_from_file_location("_torch_calls", calls_path())
-        _torch_calls = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(_torch_calls)
-        _torch_calls.bind(*[ctypes.cast(f, _vp).value for f in (_lib.boda_conv_fwd_planned, _lib.boda_conv_fwd, _lib.boda_sgemm,
-                                                                  _lib.boda_conv_out_dim)])
-        _calls = _torch_calls
+        path = calls_path()
+        try:
+            spec = importlib.util.spec_from_file_location("_torch_calls", path)
+            native = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(native)
+        except (ImportError, AttributeError) as e:
+            warnings.warn(f"{path} is not there or does not load ({e}): calls take 3 us more through ctypes; build it with "
+                          "`python -m paper_1606_00094_b200.build`", RuntimeWarning, stacklevel=2)
+            native = _CtypesOnly
+        else:
+            native.bind(*[ctypes.cast(f, _vp).value for f in (_lib.boda_conv_fwd_planned, _lib.boda_conv_fwd, _lib.boda_sgemm,
+                                                              _lib.boda_conv_out_dim)])
+        _calls = native
     return _calls
 
 

@@ -446,7 +446,6 @@ constexpr TileInfo kTiles[] = {
     {TILE_SPLIT, 128, 64, 31, 64, "direct_nhwc_x3_128x64"}, {TILE_SPLIT, 128, 80, 32, 64, "direct_nhwc_x3_128x80"},
     {TILE_SPLIT, 128, 96, 33, 64, "direct_nhwc_x3_128x96"}, {TILE_SPLIT, 128, 128, 34, 64, "direct_nhwc_x3_128x128"},
 };
-constexpr size_t kMaxSplitWorkspace = (size_t)8 << 30;      // by rule: three parts of 64 channels take 96 times the input of a one-channel layer
 constexpr int kFirstPixelTile = 9;
 constexpr int kFewIndices = 32;      // reductions up to here suit the pixel-per-thread forms
 constexpr int kNumTiles = sizeof(kTiles) / sizeof(kTiles[0]);
@@ -582,7 +581,7 @@ int direct_pick_tile(const ConvDims& d, size_t max_ws)
         double c;
         if (kTiles[t].kind == TILE_GEMM) c = gemm_cost(d, t, direct_pick_split(d, t));
         else if (kTiles[t].kind == TILE_STAGED && simt_legal(d) && (max_ws == 0 || simt_workspace_bytes(d, kTiles[t].bn) <= max_ws)) c = simt_cost(d, kTiles[t].bn);
-        else if (kTiles[t].kind == TILE_SPLIT && igemm_split_legal(d) && igemm_split_workspace(d) <= (max_ws ? max_ws : kMaxSplitWorkspace)) c = igemm_split_cost(d, kTiles[t].kt);
+        else if (kTiles[t].kind == TILE_SPLIT && igemm_split_legal(d) && igemm_split_workspace(d) <= (max_ws ? max_ws : igemm_split_workspace_limit(d))) c = igemm_split_cost(d, kTiles[t].kt);
         else continue;
         if (c < best_cost) { best_cost = c; best = t; }
     }

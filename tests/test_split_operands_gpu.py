@@ -158,6 +158,24 @@ def test_rule_and_workspace():
             B.ConvPlan(shape, math=2, variant=2, tile_id=tile)
 
 
+def test_workspace_stays_in_proportion_to_the_tensors():
+    """16 channels: the parts of a chunk of 64 are six times the input.  Picked by rule or by the tuner, they may take four times input and
+    output together; a caller who names a limit or a tile has what was asked for."""
+    from paper_1606_00094_b200 import binding as B
+    shape = (64, 16, 224, 224, 96, 11, 11, 4, 2, 1)
+    points, tensors = 64 * 224 * 224, 4 * (64 * 16 * 224 * 224 + 64 * 96 * 55 * 55)
+    need = points * 384
+    assert 256 << 20 < 4 * tensors < need
+    for kw in (dict(math=1), dict(math=3), dict(math=1, tune=1)):
+        plan = B.ConvPlan(shape, **kw)
+        assert "x3_128" not in plan.describe() and "split_128" not in plan.describe(), plan.describe()
+        plan.close()
+    for kw in (dict(math=1, max_workspace=2 * need), dict(math=1, variant=0, tile_id=25), dict(math=3, variant=2, tile_id=33)):
+        plan = B.ConvPlan(shape, **kw)
+        assert B.boda_conv_plan_workspace_bytes(plan.handle) == need, plan.describe()
+        plan.close()
+
+
 @pytest.mark.parametrize("tile,split", [(31, 1), (34, 1), (33, 3)])
 def test_expired_wait(tile, split):
     import torch

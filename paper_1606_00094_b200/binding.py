@@ -432,7 +432,15 @@ class ConvPlan:
         o.max_workspace = max_workspace
         self.handle = boda_conv_plan_create(self.shape, o)
         nbytes = boda_conv_plan_workspace_bytes(self.handle)
-        self.workspace = torch.empty(max(nbytes, 1), dtype=torch.uint8, device="cuda") if nbytes else None
+        self.workspace = None
+        if nbytes:
+            try:
+                self.workspace = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+            except torch.OutOfMemoryError:
+                # FP32 plans picked by rule run without, on the kernel that stages nothing
+                if tile_id >= 0 or tune or not self.describe().startswith("variant=direct"):
+                    self.close()
+                    raise
         N, C, H, W, K, R, S, stride, pad, _ = self.shape
         self.out_shape = (N, K, boda_conv_out_dim(H, R, stride, pad), boda_conv_out_dim(W, S, stride, pad))
 

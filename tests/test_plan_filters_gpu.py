@@ -153,6 +153,20 @@ def test_fp32_plan_runs_without_workspace():
         B.boda_conv_fwd_planned(plan.handle, dx, dw, db, out, ws)
         np.testing.assert_array_equal(out.cpu().numpy().astype(np.float64), want)
     plan.close()
+    refused = []
+
+    def no_memory(*size, **kw):
+        refused.append(size)
+        raise torch.OutOfMemoryError("no memory")
+    with pytest.MonkeyPatch.context() as patch:
+        patch.setattr(torch, "empty", no_memory)
+        plan = B.ConvPlan(shape, math=B.BODA_MATH_FP32)
+        for kw in (dict(math=3), dict(math=1, variant=0, tile_id=24)):      # no other kernel to fall back to
+            with pytest.raises(torch.OutOfMemoryError):
+                B.ConvPlan(shape, **kw)
+    assert len(refused) == 3 and plan.workspace is None
+    np.testing.assert_array_equal(plan(dx, dw, db).cpu().numpy().astype(np.float64), want)
+    plan.close()
     forced = B.ConvPlan(shape, math=B.BODA_MATH_FP32, variant=B.BODA_VARIANT_DIRECT, tile_id=18)
     with pytest.raises(B.BodaError) as e:
         B.boda_conv_fwd_planned(forced.handle, dx, dw, db, out, None)

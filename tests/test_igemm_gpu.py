@@ -363,14 +363,18 @@ def test_tuned_choice_is_remembered_in_the_cache_file(tmp_path, monkeypatch):
     t0 = time.time(); second = B.ConvPlan(shape, tune=1); t_second = time.time() - t0
     try:
         lines = cache.read_text().strip().splitlines()
-        assert len(lines) == 1 and lines[0].startswith("t5:2,64,12,12,96,3,3,1,1,")       # one entry, keyed by tile-table version and shape
+        prefix = lines[0].split(":")[0]
+        assert len(lines) == 1 and lines[0].startswith(prefix + ":2,64,12,12,96,3,3,1,1,")  # one entry, keyed by kernels, tile tables and shape
+        revision, direct, tensor = (int(v) for v in prefix.removeprefix("t").split("."))
+        assert (revision, direct, tensor) == (6, 27, 35)                                   # a tile more, or a faster kernel: another key
         assert second.describe() == first.describe()
         assert t_second < t_first                                                          # no candidates were timed again
         # an entry written for other tile tables is ignored, not misread
-        cache.write_text(lines[0].replace("t5:", "t4:", 1) + "\n")
+        others = ["t5", f"t{revision - 1}.{direct}.{tensor}", f"t{revision}.{direct - 4}.{tensor}", f"t{revision}.{direct}.{tensor - 4}"]
+        cache.write_text("".join(lines[0].replace(prefix, o, 1) + "\n" for o in others))
         third = B.ConvPlan(shape, tune=1)
         third.close()
-        assert len(cache.read_text().strip().splitlines()) == 2
+        assert len(cache.read_text().strip().splitlines()) == len(others) + 1
     finally:
         first.close(); second.close()
 

@@ -73,10 +73,10 @@ def test_every_run_gives_the_same_bits(tile, split):
     assert np.array_equal(runs[0], runs[1])
 
 
-def test_workspace_limit_keeps_fp32_plans_off_the_staged_tiles():
+@pytest.mark.parametrize("shape,name", [((20, 256, 13, 13, 384, 3, 3, 1, 1, 1), "direct_nhwc_x3_128x"), ((3, 328, 11, 13, 9, 11, 11, 4, 0, 1), "direct_nhwc_128x")])
+def test_workspace_limit_keeps_fp32_plans_off_the_staged_tiles(shape, name):
     from paper_1606_00094_b200 import binding as B
-    shape = (20, 256, 13, 13, 384, 3, 3, 1, 1, 1)
-    assert "direct_nhwc" in B.ConvPlan(shape, math=1).describe()
+    assert name in B.ConvPlan(shape, math=1).describe()
     plan = B.ConvPlan(shape, math=1, max_workspace=4096)
     assert "workspace=0" in plan.describe() and "direct_nhwc" not in plan.describe()
     with pytest.raises(B.BodaError) as e:

@@ -51,7 +51,11 @@ def test_tuned_fp32_plan_does_not_keep_the_tuners_filters():
             cudart.cudaFree(p)
 
 
-@pytest.mark.parametrize("shape,tile", [((20, 256, 13, 13, 384, 3, 3, 1, 1, 1), -1), ((3, 36, 13, 13, 97, 3, 3, 1, 1, 1), 20), ((3, 36, 13, 13, 97, 3, 3, 1, 1, 1), 2)])
+# what the rule picks with workspace: split operands on the tensor cores, and FP32 arithmetic over a staged input
+BY_RULE = [((20, 256, 13, 13, 384, 3, 3, 1, 1, 1), "direct_nhwc_x3_128x"), ((3, 328, 11, 13, 9, 11, 11, 4, 0, 1), "direct_nhwc_128x")]
+
+
+@pytest.mark.parametrize("shape,tile", [(BY_RULE[0][0], -1), (BY_RULE[1][0], -1), ((3, 36, 13, 13, 97, 3, 3, 1, 1, 1), 20), ((3, 36, 13, 13, 97, 3, 3, 1, 1, 1), 2)])
 def test_fp32_plans_read_their_filters_on_every_call(shape, tile):
     """Binding an FP32 plan keeps nothing: filters written anew in place, and other filters in between, are what the next call uses."""
     import torch
@@ -62,6 +66,7 @@ def test_fp32_plans_read_their_filters_on_every_call(shape, tile):
     bound, other = torch.from_numpy(w).cuda(), torch.from_numpy(w2).cuda()
     ref, ref2 = oracle_out(shape, x, w, b), oracle_out(shape, x, w2, b)
     plan = B.ConvPlan(shape, math=B.BODA_MATH_FP32, variant=B.BODA_VARIANT_DIRECT, tile_id=tile)
+    assert tile >= 0 or dict(BY_RULE)[shape] in plan.describe()
     plan.bind_filters(bound)
     for filt, want in ((bound, ref), (other, ref2), (bound, ref)):
         np.testing.assert_array_equal(plan(dx, filt, db).cpu().numpy().astype(np.float64), want, err_msg=plan.describe())
@@ -73,6 +78,8 @@ def test_fp32_plans_read_their_filters_on_every_call(shape, tile):
 @pytest.mark.parametrize("shape,variant,tile,math", [
     ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 2, 0),           # im2col
     ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 2, 3),
+    ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 31, 3),          # split operands
+    ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 34, 3),
     ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 6, 0),           # halo
     ((3, 64, 13, 13, 97, 3, 3, 1, 1, 1), 2, 17, 0),          # gather
     ((2, 3, 67, 67, 80, 11, 11, 4, 0, 1), 2, 24, 0),         # first layer
@@ -136,18 +143,18 @@ def test_one_call_fp32_layers_on_two_streams():
         assert all(torch.equal(o, want) for o in outs)
 
 
-def test_fp32_plan_runs_without_workspace():
+@pytest.mark.parametrize("shape,name", BY_RULE)
+def test_fp32_plan_runs_without_workspace(shape, name):
     """FP32 plans picked by rule take workspace where they can use it and run without (or with one off its alignment) on the
     kernel that needs none; only a forced staged tile insists."""
     import torch
     from paper_1606_00094_b200 import binding as B
-    shape = (20, 256, 13, 13, 384, 3, 3, 1, 1, 1)
     x, w, b = _ints(shape, 9740)
     dx, dw, db = (torch.from_numpy(t).cuda() for t in (x, w, b))
     want = oracle_out(shape, x, w, b)
     out = torch.empty(want.shape, device="cuda")
     plan = B.ConvPlan(shape, math=B.BODA_MATH_FP32)
-    assert "direct_nhwc" in plan.describe()
+    assert name in plan.describe()
     for ws in (None, plan.workspace, plan.workspace[4:], None):
         out.fill_(float("nan"))
         B.boda_conv_fwd_planned(plan.handle, dx, dw, db, out, ws)
@@ -161,10 +168,12 @@ def test_fp32_plan_runs_without_workspace():
     with pytest.MonkeyPatch.context() as patch:
         patch.setattr(torch, "empty", no_memory)
         plan = B.ConvPlan(shape, math=B.BODA_MATH_FP32)
-        for kw in (dict(math=3), dict(math=1, variant=0, tile_id=24)):      # no other kernel to fall back to
+        with pytest.raises(torch.OutOfMemoryError):                          # a forced tile: no other kernel to fall back to
+            B.ConvPlan(shape, math=1, variant=0, tile_id=24)
+        if shape[4] >= 16:
             with pytest.raises(torch.OutOfMemoryError):
-                B.ConvPlan(shape, **kw)
-    assert len(refused) == 3 and plan.workspace is None
+                B.ConvPlan(shape, math=3)
+    assert len(refused) >= 2 and plan.workspace is None
     np.testing.assert_array_equal(plan(dx, dw, db).cpu().numpy().astype(np.float64), want)
     plan.close()
     forced = B.ConvPlan(shape, math=B.BODA_MATH_FP32, variant=B.BODA_VARIANT_DIRECT, tile_id=18)

@@ -4,7 +4,7 @@ import pytest
 
 from oracle import conv_oracle as orc
 from paper_1606_00094_b200 import workloads as wl
-from helpers import GUARD, TF32_TOL, assert_parity
+from helpers import FP32_TOL, GUARD, TF32_TOL, assert_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -59,6 +59,35 @@ def test_integer_operands_are_exact():
     A = wl.integers(0x5621, (M, K))
     Bm = wl.integers(0x5622, (K, N))
     np.testing.assert_array_equal(_run(A, Bm).astype(np.float64), orc.sgemm(A, Bm))
+
+
+# products that run on the tensor cores, staged (rows of B not a multiple of 16 bytes) or straight from B, and small ones on the FP32 kernel in place
+TENSOR_SIZES = [(1000, 1301, 770), (515, 1033, 900), (1100, 700, 333), (640, 1028, 515)]
+SMALL_SIZES = [(100, 77, 50), (130, 257, 33), (129, 129, 129)]
+
+
+def _plan(M, N, K):
+    from paper_1606_00094_b200 import binding as B
+    plan = B.ConvPlan((1, K, 1, N, M, 1, 1, 1, 0, 0))
+    desc = plan.describe()
+    plan.close()
+    return desc
+
+
+@pytest.mark.parametrize("M,N,K", TENSOR_SIZES)
+def test_ragged_sizes_on_the_tensor_cores(M, N, K):
+    assert "math=tf32" in _plan(M, N, K)
+    A, Bm = wl.integers(0x5631 + M, (M, K)), wl.integers(0x5632 + N, (K, N))
+    np.testing.assert_array_equal(_run(A, Bm).astype(np.float64), orc.sgemm(A, Bm))
+    A, Bm = wl.normal(0x5633 + M, (M, K)), wl.normal(0x5634 + N, (K, N))
+    assert_parity(_run(A, Bm), orc.sgemm(A, Bm), TF32_TOL, f"sgemm {M}x{N}x{K}")
+
+
+@pytest.mark.parametrize("M,N,K", SMALL_SIZES)
+def test_small_products_have_fp32_accuracy(M, N, K):
+    assert "variant=direct" in _plan(M, N, K)
+    A, Bm = wl.normal(0x5635 + M, (M, K)), wl.normal(0x5636 + N, (K, N))
+    assert_parity(_run(A, Bm), orc.sgemm(A, Bm), FP32_TOL, f"sgemm {M}x{N}x{K}")
 
 
 def test_rejects_bad_arguments():

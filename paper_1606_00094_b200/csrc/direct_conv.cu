@@ -575,17 +575,23 @@ int direct_pick_tile(const ConvDims& d, size_t max_ws)
         const int t = kFirstPixelTile + (d.K <= 8 ? 0 : d.K <= 16 ? 1 : 2);
         if (direct_tile_legal(d, t)) return t;
     }
-    int best = 8;
-    double best_cost = 1e300;
+    int best = 8, split = -1;
+    double best_cost = 1e300, split_rank = 1e300, split_cost = 0.0;
     for (int t = 0; t < kNumTiles; ++t) {
         double c;
+        if (kTiles[t].kind == TILE_SPLIT) {
+            if (!igemm_split_legal(d) || igemm_split_workspace(d) > (max_ws ? max_ws : igemm_split_workspace_limit(d))) continue;
+            double clocks = 0.0;
+            const double rank = igemm_split_cost(d, kTiles[t].kt, &clocks);
+            if (rank < split_rank) { split_rank = rank; split_cost = clocks; split = t; }
+            continue;
+        }
         if (kTiles[t].kind == TILE_GEMM) c = gemm_cost(d, t, direct_pick_split(d, t));
         else if (kTiles[t].kind == TILE_STAGED && simt_legal(d) && (max_ws == 0 || simt_workspace_bytes(d, kTiles[t].bn) <= max_ws)) c = simt_cost(d, kTiles[t].bn);
-        else if (kTiles[t].kind == TILE_SPLIT && igemm_split_legal(d) && igemm_split_workspace(d) <= (max_ws ? max_ws : igemm_split_workspace_limit(d))) c = igemm_split_cost(d, kTiles[t].kt);
         else continue;
         if (c < best_cost) { best_cost = c; best = t; }
     }
-    return best;
+    return split >= 0 && split_cost < best_cost ? split : best;
 }
 
 bool direct_tile_legal(const ConvDims& d, int tile_id)

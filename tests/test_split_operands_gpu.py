@@ -197,3 +197,22 @@ def test_expired_wait(tile, split):
     plan.close()
     got, desc = run_planned(shape, x, w, b, variant=2, math=3, tile_id=tile, split_k=split)
     assert_parity(got, oracle_out(shape, x, w, b), 0.0, desc)
+
+
+# layers around the line between the tiles of split operands and the others, measured times (us) split operands / the other kernel
+KEEP_OTHER = [
+    ((31, 79, 113, 116, 1, 3, 3, 1, 1, 0), 1),        # 562 / 363: one filter, a staged copy that L2 does not hold
+    ((22, 16, 82, 83, 17, 3, 3, 1, 1, 0), 1),         # 70 / 47: three quarters of a chunk are padding
+    ((36, 2, 105, 107, 119, 2, 2, 4, 0, 0), 3),       # 53 / 34
+    ((48, 5, 113, 116, 130, 1, 1, 2, 0, 0), 3),       # 123 / 87
+]
+TAKE_SPLIT = [((20, 256, 13, 13, 384, 3, 3, 1, 1, 1), 1), ((20, 64, 56, 56, 128, 3, 3, 1, 1, 1), 1), ((5, 256, 13, 13, 384, 3, 3, 1, 1, 1), 3)]
+
+
+@pytest.mark.parametrize("shape,math", KEEP_OTHER + TAKE_SPLIT)
+def test_line_between_split_operands_and_the_other_kernels(shape, math):
+    from paper_1606_00094_b200 import binding as B
+    plan = B.ConvPlan(shape, math=math)
+    desc = plan.describe()
+    plan.close()
+    assert ("direct_nhwc_x3_128x" in desc or "split_128x" in desc) == ((shape, math) in TAKE_SPLIT), desc

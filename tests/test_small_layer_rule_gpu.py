@@ -15,6 +15,8 @@ IN_PLACE = [
     (4, 9, 15, 15, 29, 5, 5, 1, 2, 1),           # 5.0 / 10.6
     (1, 17, 19, 21, 105, 3, 3, 2, 1, 1),         # 4.4 / 7.9
     (1, 7, 39, 42, 16, 1, 1, 1, 0, 1),           # 3.1 / 5.8
+    (38, 10, 35, 35, 28, 1, 1, 1, 0, 1),         # 5.7 / 11.4: one chunk, many points
+    (40, 16, 41, 43, 29, 1, 1, 1, 0, 1),         # 7.3 / 13.9
 ]
 TENSOR = [
     (5, 480, 14, 14, 192, 1, 1, 1, 0, 1),        # 11.5 / 6.5

@@ -177,7 +177,7 @@ _calls = None
 def _load_calls():
     """The native form of the forward calls (csrc/torch_calls.cpp), loaded on first use: it needs torch.  Its functions take plain
     CUDA tensors on the current stream and return None, having done nothing, for what they leave to ctypes.  A 3x3 layer on
-    one 32x32 image (kernel 2.5 us), call after call: 6.7 us through ctypes, 3.8 here, 2.3 of them the launch."""
+    one 32x32 image (kernel 2.5 us), call after call: 6.7 us through ctypes, 3.8 to 4.2 here, 2.3 of them the launch."""
     global _calls
     if _calls is None:
         _load_torch()

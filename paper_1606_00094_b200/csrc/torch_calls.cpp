@@ -1,7 +1,7 @@
 // The forward entry points as a CPython extension over torch tensors: what binding.py does for a call - output allocation, data
 // pointers, current stream, the call into libboda.so without the GIL - in native code.
 //
-// Bound: the host.  A small layer's kernel takes 2 to 7 us, and the interpreter with ctypes took 6.7 us a call; this takes 3.8, of which
+// Bound: the host.  A small layer's kernel takes 2 to 7 us, and the interpreter with ctypes took 6.7 us a call; this takes 3.8 to 4.2, of which
 // 2.3 are the launch itself.
 // Only the ordinary call is taken here (plain CUDA tensors, current stream); every function returns None for anything else, before it
 // has done anything, and the caller goes on through ctypes.  A status other than 0 is returned as an int.

@@ -42,8 +42,8 @@ void igemm_unbind_filters(IgemmPlan* p);
 int igemm_launch(IgemmPlan* p, const float* in, const float* filt, const float* bias, float* out, void* workspace,
                  cudaStream_t stream, cudaEvent_t after_staging = nullptr);
 
-// The split-operand tiles (error-compensated mode, FP32 accuracy): may they run the shape, what ranks a tile with its best split among them, the
-// estimated SM clocks of a call on it (staging of both operands included), and the workspace they need.
+// The split-operand tiles (error-compensated mode, FP32 accuracy): may they run the shape, the estimated SM clocks of one call with its
+// best split, staging of both operands included (`clocks`: by a second model), and the workspace they need.
 bool igemm_split_legal(const ConvDims& d);
 double igemm_split_cost(const ConvDims& d, int tile, double* clocks);
 size_t igemm_split_workspace(const ConvDims& d);

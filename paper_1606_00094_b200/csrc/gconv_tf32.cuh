@@ -79,7 +79,7 @@ gconv_tf32_kernel(const __grid_constant__ CUtensorMap map_b, const GconvParams p
     __shared__ __align__(16) int s_off[kMaxKred];           // element offset of every reduction index
     __shared__ int s_rs[kMaxKred];                          // its tap (r << 16) | s
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform_warp_index();
     const int lane = threadIdx.x & 31;
     const int my_tiles = ((int)blockIdx.x < p.tiles_total) ? (p.tiles_total - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int nchunks = p.nchunks;
@@ -105,11 +105,11 @@ gconv_tf32_kernel(const __grid_constant__ CUtensorMap map_b, const GconvParams p
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_acc = s_tmem_base;
+    const uint32_t tmem_acc = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     if (!(p.b_early && warp == 0)) pdl_wait();
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             // ---------------- filter tiles by TMA, one per stage; this arrival also carries the byte count
             uint32_t stage = 0, par = 1;
             bool first = true;
@@ -118,18 +118,20 @@ gconv_tf32_kernel(const __grid_constant__ CUtensorMap map_b, const GconvParams p
                 const int k0 = (tile % p.tiles_n) * BN;
                 bool ok = true;
                 for (int j = 0; j < nchunks; ++j) {
-                    ok = mbar_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 21);
+                    ok = warp_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 21);
                     if (!ok) break;
-                    mbar_expect_tx(full_bar + 8 * stage, (uint32_t)C::B_STAGE_BYTES + ((first && blockIdx.x == 0) ? (uint32_t)p.tx_extra : 0u));
+                    if (elect_one()) {
+                        mbar_expect_tx(full_bar + 8 * stage, (uint32_t)C::B_STAGE_BYTES + ((first && blockIdx.x == 0) ? (uint32_t)p.tx_extra : 0u));
+                        tma_load_2d(smem_b + stage * C::B_STAGE_BYTES, &map_b, full_bar + 8 * stage, 32 * j, k0);
+                    }
                     first = false;
-                    tma_load_2d(smem_b + stage * C::B_STAGE_BYTES, &map_b, full_bar + 8 * stage, 32 * j, k0);
                     if (++stage == (uint32_t)kStages) { stage = 0; par ^= 1u; }
                 }
                 if (!ok) break;
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             // ---------------- MMA issuer
             constexpr uint32_t idesc = instr_desc_tf32<BN>();
             const uint64_t da0 = smem_desc_k_sw128(smem_a), db0 = smem_desc_k_sw128(smem_b);
@@ -138,22 +140,26 @@ gconv_tf32_kernel(const __grid_constant__ CUtensorMap map_b, const GconvParams p
             for (int t = 0; t < my_tiles && ok; ++t) {
                 const uint32_t slot = (uint32_t)t & 1u;
                 // the accumulator slot is free once the epilogue of the tile two back has read it
-                ok = mbar_wait(acc_empty + 8 * slot, ((uint32_t)(t >> 1) & 1u) ^ 1u, &s_abort, p.status, 22);
+                ok = warp_wait(acc_empty + 8 * slot, ((uint32_t)(t >> 1) & 1u) ^ 1u, &s_abort, p.status, 22);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t acc = tmem_acc + slot * (uint32_t)BN;
                 for (int j = 0; j < nchunks; ++j) {
-                    ok = mbar_wait(full_bar + 8 * stage, par, &s_abort, p.status, 23);
+                    ok = warp_wait(full_bar + 8 * stage, par, &s_abort, p.status, 23);
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t da = da0 + (uint64_t)stage * (A_STAGE_BYTES >> 4);
                     const uint64_t db = db0 + (uint64_t)stage * (C::B_STAGE_BYTES >> 4);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) umma_tf32(acc, da + 2 * k, db + 2 * k, idesc, (j | k) ? 1u : 0u);
-                    tc_commit(empty_bar + 8 * stage);
+                        for (int k = 0; k < 4; ++k) umma_tf32(acc, da + 2 * k, db + 2 * k, idesc, (j | k) ? 1u : 0u);
+                        tc_commit(empty_bar + 8 * stage);
+                    }
+                    __syncwarp();
                     if (++stage == (uint32_t)kStages) { stage = 0; par ^= 1u; }
                 }
-                if (ok) tc_commit(acc_full + 8 * slot);
+                if (ok && elect_one()) tc_commit(acc_full + 8 * slot);
+                __syncwarp();
             }
         }
     } else if (warp < kFirstProducerWarp) {

@@ -86,7 +86,7 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     __shared__ volatile int s_abort;
     __shared__ __align__(16) float s_bias[BN];
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform_warp_index();
     const int lane = threadIdx.x & 31;
     // persistent: this CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...; tile = (image, point tile) * tiles_n + channel tile
     const int my_tiles = ((int)blockIdx.x < p.tiles_total) ? (p.tiles_total - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
@@ -111,7 +111,7 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_acc = s_tmem_base;
+    const uint32_t tmem_acc = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     // tile t of this CTA -> image, first output point, first output channel (the first tile's before the dependency wait)
     auto decode = [&](int t, int& n, int& hw0, int& k0) {
         const int tile = (int)blockIdx.x + t * (int)gridDim.x;
@@ -125,7 +125,7 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     if (!(p.b_early && warp == 3)) pdl_wait();
 
     if (warp == 0 || warp == 2) {
-        if (lane == 0) {
+        {
             // ---------------- input tiles: boxes of 32 output points x 32 channels; warp 0 loads points 0..63, warp 2 points 64..127
             const int half = warp == 0 ? 0 : 2;
             uint32_t stage = 0, par = 1;
@@ -133,17 +133,19 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             for (int t = 0; t < my_tiles && ok; ++t) {
                 if (t > 0) decode(t, n, hw0, k0);
                 for (int i = 0; i < steps; ++i) {
-                    ok = mbar_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 41);
+                    ok = warp_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 41);
                     if (!ok) break;
                     const uint32_t dst = smem_a + stage * A_STAGE_BYTES + (uint32_t)half * A_BOX_BYTES;
-                    tma_load_3d(dst, &map_a, full_bar + 8 * stage, hw0 + 32 * half, 32 * (i_begin + i), n);
-                    tma_load_3d(dst + A_BOX_BYTES, &map_a, full_bar + 8 * stage, hw0 + 32 * half + 32, 32 * (i_begin + i), n);
+                    if (elect_one()) {
+                        tma_load_3d(dst, &map_a, full_bar + 8 * stage, hw0 + 32 * half, 32 * (i_begin + i), n);
+                        tma_load_3d(dst + A_BOX_BYTES, &map_a, full_bar + 8 * stage, hw0 + 32 * half + 32, 32 * (i_begin + i), n);
+                    }
                     if (++stage == (uint32_t)kStages) { stage = 0; par ^= 1u; }
                 }
             }
         }
     } else if (warp == 3) {
-        if (lane == 0) {
+        {
             // ---------------- filter tiles and the stage's byte count
             uint32_t stage = 0, par = 1;
             uint32_t bytes = C::STAGE_BYTES + (blockIdx.x == 0 ? (uint32_t)p.tx_extra : 0u);
@@ -151,19 +153,20 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             for (int t = 0; t < my_tiles && ok; ++t) {
                 if (t > 0) decode(t, n, hw0, k0);
                 for (int i = 0; i < steps; ++i) {
-                    ok = mbar_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 42);
+                    ok = warp_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 42);
                     if (!ok) break;
-                    mbar_expect_tx(full_bar + 8 * stage, bytes);
+                    if (elect_one()) {
+                        mbar_expect_tx(full_bar + 8 * stage, bytes);
+                        tma_load_3d(smem_b + stage * C::B_STAGE_BYTES, &map_b, full_bar + 8 * stage, 32 * (i_begin + i), k0, 0);
+                    }
                     bytes = C::STAGE_BYTES;
-                    tma_load_3d(smem_b + stage * C::B_STAGE_BYTES, &map_b, full_bar + 8 * stage, 32 * (i_begin + i), k0, 0);
                     if (++stage == (uint32_t)kStages) { stage = 0; par ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer: A is MN-major (bit 15 of the instruction descriptor), B K-major; tile t accumulates in slot t & 1, so
-        // that its epilogue runs under the next tile's main loop.  The whole warp walks the loop and one elected lane issues: 25
-        // clocks an MMA instead of 70, which is what a step of a narrow tile takes.  480 channels, 14x14, 192 filters: batch 5
+        // that its epilogue runs under the next tile's main loop.  The whole warp walks the loop and one elected lane issues.  480 channels, 14x14, 192 filters: batch 5
         // 7.3 -> 6.5 us, batch 256 with 64-channel tiles 52.9 -> 45.8 (192-channel tiles, which fetch more per step: 34.7 both ways).
         constexpr uint32_t idesc = instr_desc_tf32<BN>() | (1u << 15);
         const uint64_t da0 = smem_desc_mn_sw128(smem_a), db0 = smem_desc_k_sw128(smem_b);
@@ -186,7 +189,7 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 const bool peek = mbar_test_wait(full_bar + 8 * next, next_par);
                 const uint64_t da = da0 + (uint64_t)stage * (A_STAGE_BYTES >> 4);
                 const uint64_t db = db0 + (uint64_t)stage * (C::B_STAGE_BYTES >> 4);
-                if (pair::elect_one()) {
+                if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k)       // 8 channels per MMA: 8 rows of 128 bytes further in A, 32 bytes further in B's rows
                         umma_tf32(acc, da + (uint64_t)k * (1024 >> 4), db + 2 * k, idesc, (i | k) ? 1u : 0u);

@@ -3,14 +3,12 @@
 // Two CTAs of a cluster share one output tile of 256 points x BN channels: each stages its own 128 points and HALF of the tile's
 // filter rows, and one thread of the first CTA issues MMAs that read both CTAs' shared memory and write 128 rows into each
 // CTA's tensor memory.  A CTA therefore fetches 128 + BN/2 rows per reduction step instead of 128 + BN for the same MMA time.
-// That is what bounds the one-CTA kernel below BN = 256 (shared memory fills at about 1.35 clocks per 128-byte row, so its
-// 128x128 tile waits 354 clocks a step for 256 clocks of MMAs), and why it needs wide tiles, i.e. few of them.
+// That is what bounds the one-CTA kernel below BN = 256 (L2 feeds the SMs some 10 KB a clock in all), and why it needs wide tiles, i.e. few of them.
 // The pairs are persistent (at most one CTA per SM walks the tiles) with two accumulators in tensor memory: a tile's epilogue
 // and the pipeline's fill run under the next tile's main loop.
-// Measured, clocks per 32-channel step with every SM busy (one-CTA kernel / pairs): BN 64 375 / 290, 96 380 / 334, 128 390 / 356, 192 473
-// / 434, 256 574 / 560 (512 of MMAs); whole layers: 5x5 on 96 channels, 27x27, batch 128 (115 GFLOP) 169 / 150 us, the same with
-// fp16 operands 130 / 105; 3x3 on 256 channels, 13x13, batch 128 76.5 / 69.3; 5x5 on 87 channels, 42 filters, batch 28 61 / 47.
-// One round of few tiles stays with the one-CTA kernel and its cluster split (3x3, 13x13, batch 20: 19.5 / 21.3 us).
+// Measured, one-CTA kernel / pairs of the same width: 5x5 on 96 channels, 256 filters, 27x27, fp16, batch 128 (115 GFLOP) 130 / 105 us (BN = 256), 153 / 123
+// (128); 3x3 on 256 channels, 384 filters, 13x13, batch 128 73.3 / 63.1 (128), 70.9 / 65.6 (192).
+// One round of few tiles stays with the one-CTA kernel (3x3, 13x13, batch 20: 16.8 / 17.6 us, BN = 96).
 //
 // Roles per CTA (416 threads): warp 0 = input tiles, warp 11 = filter tiles, warp 12 (first CTA) = byte counts of both CTAs, warp
 // 1 = MMA issue (first CTA) and the tensor-memory allocation, warps 2..5 and 7..10 = epilogue.  Loads signal the first CTA's full
@@ -46,8 +44,8 @@ struct PairParams {
 template <int BN> struct Cfg {
     static constexpr int B_ROWS = BN / 2;
     static constexpr int B_CHUNK_BYTES = B_ROWS * 128;
-    // Reduction chunks per stage.  The issuing warp spends about 260 clocks of barrier test and commit on a stage besides 25 per
-    // MMA: more than the MMAs of one chunk take (2*BN clocks) below BN = 256, so the narrower tiles put two chunks in a stage.
+    // Reduction chunks per stage: a stage costs the issuing warp a wait, a vote and a commit besides its MMAs, so the narrower tiles put two
+    // chunks in one.
     static constexpr int CPS = BN >= 256 ? 1 : 2;
     static constexpr int STAGE_BYTES = CPS * (A_CHUNK_BYTES + B_CHUNK_BYTES);
     static constexpr int STORE_BYTES = 8 * BOX_BYTES;
@@ -93,12 +91,6 @@ __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t
         asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
                      :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-    return p != 0;
-}
 // the same operand formats as the one-CTA kernels, M = 256
 template <int BN, bool F16>
 __host__ __device__ constexpr uint32_t instr_desc()
@@ -127,7 +119,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     __shared__ volatile int s_abort;
     __shared__ __align__(16) float s_bias[2][BN];
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_cta_rank();
     const int pair_id = (int)blockIdx.x >> 1, pairs = (int)gridDim.x >> 1;
 
@@ -149,11 +141,11 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     __syncthreads();
     cluster_sync_all();              // the peer's barriers exist from here on
     tc_fence_after();
-    const uint32_t tmem = s_tmem_base;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     if (!(p.b_early && warp >= 11)) pdl_wait();
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             // ---------------- this CTA's 128 input rows
             uint32_t stage = 0, par = 1;
             const uint32_t full0 = map_to_cta(full_bar, 0);
@@ -165,12 +157,12 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 const int cend = p.cchunks * CH;
                 int cx = 0, r = 0, s = 0;
                 for (int i = 0; i < p.iters; i += CPS) {
-                    ok = mbar_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 61);
+                    ok = warp_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 61);
                     if (!ok) break;
 #pragma unroll
                     for (int c = 0; c < CPS; ++c) {
                         if (c > 0 && i + c >= p.iters) break;
-                        load_im2col(smem_a + stage * A_STAGE_BYTES + c * A_CHUNK_BYTES, &map_a, full0 + 8 * stage, cx, w0, h0, n0, (uint16_t)s, (uint16_t)r);
+                        if (elect_one()) load_im2col(smem_a + stage * A_STAGE_BYTES + c * A_CHUNK_BYTES, &map_a, full0 + 8 * stage, cx, w0, h0, n0, (uint16_t)s, (uint16_t)r);
                         cx += CH;
                         if (cx == cend) { cx = 0; if (++s == p.S) { s = 0; ++r; } }
                     }
@@ -179,7 +171,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             }
         }
     } else if (warp == 11) {
-        if (lane == 0) {
+        {
             // ---------------- this CTA's half of the filter rows
             uint32_t stage = 0, par = 1;
             const uint32_t full0 = map_to_cta(full_bar, 0);
@@ -189,12 +181,12 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 const int cend = p.cchunks * CH;
                 int cx = 0, tap = 0;
                 for (int i = 0; i < p.iters; i += CPS) {
-                    ok = mbar_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 62);
+                    ok = warp_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 62);
                     if (!ok) break;
 #pragma unroll
                     for (int c = 0; c < CPS; ++c) {
                         if (c > 0 && i + c >= p.iters) break;
-                        load_3d(smem_b + stage * B_STAGE_BYTES + c * C::B_CHUNK_BYTES, &map_b, full0 + 8 * stage, cx, k0, tap);
+                        if (elect_one()) load_3d(smem_b + stage * B_STAGE_BYTES + c * C::B_CHUNK_BYTES, &map_b, full0 + 8 * stage, cx, k0, tap);
                         cx += CH;
                         if (cx == cend) { cx = 0; ++tap; }
                     }
@@ -203,7 +195,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             }
         }
     } else if (warp == 12) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             // ---------------- byte counts of both CTAs' loads
             uint32_t stage = 0, par = 1;
             constexpr uint32_t CHUNK = 2u * (A_CHUNK_BYTES + C::B_CHUNK_BYTES);
@@ -211,9 +203,9 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             bool ok = true;
             for (int t = pair_id; t < p.tiles_total && ok; t += pairs) {
                 for (int i = 0; i < p.iters; i += CPS) {
-                    ok = mbar_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 63);
+                    ok = warp_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 63);
                     if (!ok) break;
-                    mbar_expect_tx(full_bar + 8 * stage, (i + CPS <= p.iters ? CPS * CHUNK : CHUNK) + extra);
+                    if (elect_one()) mbar_expect_tx(full_bar + 8 * stage, (i + CPS <= p.iters ? CPS * CHUNK : CHUNK) + extra);
                     extra = 0;
                     if (++stage == (uint32_t)STAGES) { stage = 0; par ^= 1u; }
                 }
@@ -231,7 +223,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             int local = 0;
             for (int t = pair_id; t < p.tiles_total && ok; t += pairs, ++local) {
                 const uint32_t slot = (uint32_t)local & 1u;
-                ok = __all_sync(0xffffffffu, mbar_wait(acc_empty + 8 * slot, ((uint32_t)(local >> 1) & 1u) ^ 1u, &s_abort, p.status, 64));
+                ok = warp_wait(acc_empty + 8 * slot, ((uint32_t)(local >> 1) & 1u) ^ 1u, &s_abort, p.status, 64);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t acc0 = tmem + slot * (uint32_t)TILE_COLS;
@@ -239,7 +231,7 @@ pair_conv_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 int chunk = 0;
                 for (int i = 0; i < p.iters; i += CPS) {
                     if (!landed) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(full_bar + 8 * stage, par, &s_abort, p.status, 65));
+                        ok = warp_wait(full_bar + 8 * stage, par, &s_abort, p.status, 65);
                         if (!ok) break;
                     }
                     tc_fence_after();

@@ -135,6 +135,23 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return mbar_wait_slow(bar, parity, abort_flag, status, where);
 }
 
+// What single threads used to do - fill stages, issue MMAs - whole warps do here: the warp walks the loop, an elected lane issues.  Addresses and
+// descriptors then stay in uniform registers, as the instructions want them; in a branch of one lane (or with a warp index that the compiler
+// cannot know to be uniform) a load, a byte count, a commit or an MMA takes its thread 100 to 150 clocks instead of 10 to 40.  Measured by itself: four
+// 128x96 MMAs and a commit 390 clocks from one lane, 225 (the tensor pipe's time) from a warp.
+__device__ __forceinline__ int uniform_warp_index() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// the wait of such a warp, and its common decision: no lane is left alone at the next election
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int where)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, where));
+}
+
 // Bounded wait for threads that are not on the critical path (the epilogue waiting for the accumulator):
 // polls rarely and sleeps in between, so that it does not compete with the producer's and the MMA issuer's
 // barrier traffic.  The limit is the same number of cycles, counted in sleep quanta.
@@ -142,7 +159,7 @@ static __device__ __noinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t par
 {
     const long long t0 = clock64();
     for (;;) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (mbar_test_wait(bar, parity)) return true;
         if (*abort_flag) return false;
         if (clock64() - t0 > c_wait_limit_cycles) {
             *abort_flag = 1;

@@ -88,7 +88,7 @@ tconv_first_layer_kernel(const __grid_constant__ CUtensorMap map_b0, const __gri
     __shared__ volatile int s_abort;
     __shared__ __align__(16) float s_bias[BN];
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform_warp_index();
     const int lane = threadIdx.x & 31;
     const int n = (int)blockIdx.x / p.h.tiles_per_image;
     const int j = (int)blockIdx.x - n * p.h.tiles_per_image;
@@ -117,27 +117,30 @@ tconv_first_layer_kernel(const __grid_constant__ CUtensorMap map_b0, const __gri
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_acc = s_tmem_base;
+    const uint32_t tmem_acc = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     pdl_wait();
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             // ---------------- filter tiles: taps of chunk 0 (32 channels, 128-byte rows), then of chunk 1 (16 channels,
             // 64-byte rows); one ring of b_stages slots of BN*128 bytes for both
             uint32_t stage = 0, par = 1;
             for (int i = 0; i < 2 * taps; ++i) {
-                if (!mbar_wait(b_empty + 8 * stage, par, &s_abort, p.h.status, 52)) break;
+                if (!warp_wait(b_empty + 8 * stage, par, &s_abort, p.h.status, 52)) break;
                 const bool second = i >= taps;
                 const uint32_t bytes = second ? (uint32_t)(BN * 64) : (uint32_t)B_STAGE_BYTES;
-                mbar_expect_tx(b_full + 8 * stage, bytes + ((i == 0 && (blockIdx.x | blockIdx.y) == 0) ? (uint32_t)p.h.tx_extra : 0u));
-                if (second) tma_load_3d(smem_b + stage * B_STAGE_BYTES, &map_b1, b_full + 8 * stage, 32, k0, i - taps);
-                else tma_load_3d(smem_b + stage * B_STAGE_BYTES, &map_b0, b_full + 8 * stage, 0, k0, i);
+                if (elect_one()) {
+                    mbar_expect_tx(b_full + 8 * stage, bytes + ((i == 0 && (blockIdx.x | blockIdx.y) == 0) ? (uint32_t)p.h.tx_extra : 0u));
+                    if (second) tma_load_3d(smem_b + stage * B_STAGE_BYTES, &map_b1, b_full + 8 * stage, 32, k0, i - taps);
+                    else tma_load_3d(smem_b + stage * B_STAGE_BYTES, &map_b0, b_full + 8 * stage, 0, k0, i);
+                }
+                __syncwarp();
                 if (++stage == (uint32_t)p.b_stages) { stage = 0; par ^= 1u; }
             }
         }
     } else if (warp == 1 || warp == 6 || warp >= 11) {
         const int acc = warp == 1 ? 0 : warp == 6 ? 1 : warp - 9;             // warps 1, 6, 11, 12: one accumulator each
-        if (lane == 0) {
+        {
             // ---------------- MMA issuers
             constexpr uint32_t idesc = instr_desc_tf32<BN>();
             const uint32_t my_acc = tmem_acc + (uint32_t)(acc * BN);
@@ -145,7 +148,7 @@ tconv_first_layer_kernel(const __grid_constant__ CUtensorMap map_b0, const __gri
             // Between a stage's barrier and its MMAs the four issuers are all busy with bookkeeping and the tensor pipe
             // idles, so the loops hold as little of it as possible: one loop per chunk, descriptors advanced by
             // additions (a descriptor's address field counts 16-byte units: 8 per slab row of chunk 0, 4 of chunk 1).
-            bool ok = mbar_wait(slab_full, 0, &s_abort, p.h.status, 53);
+            bool ok = warp_wait(slab_full, 0, &s_abort, p.h.status, 53);
             const uint32_t S = (uint32_t)p.h.S, row_step = (uint32_t)(p.h.Wp - p.h.S + 1);   // slab rows from a tap row's last tap to the next row's first
             const uint32_t nstages = (uint32_t)p.b_stages;
             uint32_t b_addr = smem_b;
@@ -153,37 +156,44 @@ tconv_first_layer_kernel(const __grid_constant__ CUtensorMap map_b0, const __gri
                 uint64_t da = smem_desc_k_sw128(slab0 + (uint32_t)(acc * 128) * 128u);
                 uint32_t s = 0;
                 for (int i = 0; ok && i < taps; ++i) {
-                    ok = mbar_wait(b_full + 8 * stage, par, &s_abort, p.h.status, 55);
+                    ok = warp_wait(b_full + 8 * stage, par, &s_abort, p.h.status, 55);
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t db = smem_desc_k_sw128(b_addr);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) umma_tf32(my_acc, da + 2 * k, db + 2 * k, idesc, (i | k) ? 1u : 0u);
-                    tc_commit(b_empty + 8 * stage);
+                        for (int k = 0; k < 4; ++k) umma_tf32(my_acc, da + 2 * k, db + 2 * k, idesc, (i | k) ? 1u : 0u);
+                        tc_commit(b_empty + 8 * stage);
+                    }
+                    __syncwarp();
                     b_addr += B_STAGE_BYTES;
                     if (++stage == nstages) { stage = 0; par ^= 1u; b_addr = smem_b; }
                     if (++s == S) { s = 0; da += 8 * row_step; } else da += 8;
                 }
             }
             if (acc == 0) FL_STAMP(1);
-            if (ok) ok = mbar_wait(slab_full + 8, 0, &s_abort, p.h.status, 54);
+            if (ok) ok = warp_wait(slab_full + 8, 0, &s_abort, p.h.status, 54);
             {
                 uint64_t da = smem_desc_k_sw64(slab1 + (uint32_t)(acc * 128) * 64u);
                 uint32_t s = 0;
                 for (int i = 0; ok && i < taps; ++i) {
-                    ok = mbar_wait(b_full + 8 * stage, par, &s_abort, p.h.status, 55);
+                    ok = warp_wait(b_full + 8 * stage, par, &s_abort, p.h.status, 55);
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t db = smem_desc_k_sw64(b_addr);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) umma_tf32(my_acc, da + 2 * k, db + 2 * k, idesc, 1u);
-                    tc_commit(b_empty + 8 * stage);
+                        for (int k = 0; k < 2; ++k) umma_tf32(my_acc, da + 2 * k, db + 2 * k, idesc, 1u);
+                        tc_commit(b_empty + 8 * stage);
+                    }
+                    __syncwarp();
                     b_addr += B_STAGE_BYTES;
                     if (++stage == nstages) { stage = 0; par ^= 1u; b_addr = smem_b; }
                     if (++s == S) { s = 0; da += 4 * row_step; } else da += 4;
                 }
             }
-            tc_commit(accum_bar);
+            if (elect_one()) tc_commit(accum_bar);
+            __syncwarp();
             if (acc == 0) FL_STAMP(6);
             if (!ok) (void)mbar_wait(accum_bar, 0, &s_abort, p.h.status, 56);
         }

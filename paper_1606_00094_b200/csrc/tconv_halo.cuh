@@ -76,9 +76,8 @@ struct HaloCfg {
     static constexpr int ACC_COLS = BN * NACC;
     static constexpr int TMEM_COLS = ACC_COLS <= 32 ? 32 : ACC_COLS <= 64 ? 64 : ACC_COLS <= 128 ? 128 : ACC_COLS <= 256 ? 256 : 512;
     static_assert(ACC_COLS <= 512, "accumulators exceed tensor memory");
-    // One thread can issue an MMA about every 70 clocks; threads in different warps, each feeding its own
-    // accumulators, reach about 50 each (measured).  A reduction step of this kernel is 4 MMAs per accumulator, which
-    // the tensor pipe finishes in 8*BN/4 clocks: with one issuer per accumulator the pipe, not the issue, is the limit.
+    // A reduction step is 4 MMAs per accumulator, which the tensor pipe finishes in 2*BN clocks: with one issuer per accumulator the pipe, not
+    // the issue, is the limit.
     static constexpr int ISSUERS = NACC >= 4 ? 4 : NACC >= 2 ? 2 : 1;
 };
 
@@ -334,7 +333,7 @@ tconv_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     __shared__ volatile int s_abort;
     __shared__ __align__(16) float s_bias[BN];
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform_warp_index();
     const int lane = threadIdx.x & 31;
     int f0 = blockIdx.x * (128 * NACC);
     if (p.pool_rows > 0) {          // tiles of whole output rows of one image (fused pooling)
@@ -363,12 +362,12 @@ tconv_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_acc = s_tmem_base;
+    const uint32_t tmem_acc = __shfl_sync(0xffffffffu, s_tmem_base, 0);
     pdl_wait();          // everything above overlapped the previous kernel; its results are needed from here on
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------- TMA producer.  One thread; ring positions, phases and addresses are advanced
+        {
+            // ---------------- TMA producer.  Ring positions, phases and addresses are advanced
             // incrementally (no division in the loop): the loop's own latency bounds the iteration rate.
             const int row0 = f0 - p.lead;                 // may be negative: those rows read as zeros
             const int chunk0 = it_begin / p.taps;
@@ -380,20 +379,26 @@ tconv_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             bool need_slab = true;
             for (int i = 0; i < my_iters; ++i) {
                 if (need_slab) {
-                    if (!mbar_wait(a_empty + 8 * a_slot, a_par, &s_abort, p.status, 11)) break;
+                    if (!warp_wait(a_empty + 8 * a_slot, a_par, &s_abort, p.status, 11)) break;
                     const uint32_t fb = a_full + 8 * a_slot;
-                    mbar_expect_tx(fb, (uint32_t)p.a_slot_bytes);
                     const uint32_t dst = smem_a + a_slot * p.a_slot_bytes;
-                    tma_load_2d(dst, &map_a, fb, cx, row0);
-                    if (p.nbox > 1) tma_load_2d(dst + p.box_rows * 128, &map_a, fb, cx, row0 + p.box_rows);
-                    if (p.nbox > 2) tma_load_2d(dst + 2 * p.box_rows * 128, &map_a, fb, cx, row0 + 2 * p.box_rows);
+                    if (elect_one()) {
+                        mbar_expect_tx(fb, (uint32_t)p.a_slot_bytes);
+                        tma_load_2d(dst, &map_a, fb, cx, row0);
+                        if (p.nbox > 1) tma_load_2d(dst + p.box_rows * 128, &map_a, fb, cx, row0 + p.box_rows);
+                        if (p.nbox > 2) tma_load_2d(dst + 2 * p.box_rows * 128, &map_a, fb, cx, row0 + 2 * p.box_rows);
+                    }
+                    __syncwarp();
                     a_slot ^= 1u;
                     if (a_slot == 0) a_par ^= 1u;
                     need_slab = false;
                 }
-                if (!mbar_wait(be, b_par, &s_abort, p.status, 12)) break;
-                mbar_expect_tx(bf, Cfg::B_STAGE_BYTES + ((i == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) ? (uint32_t)p.tx_extra : 0u));
-                tma_load_3d(bdst, &map_b, bf, cx, k0, tap);
+                if (!warp_wait(be, b_par, &s_abort, p.status, 12)) break;
+                if (elect_one()) {
+                    mbar_expect_tx(bf, Cfg::B_STAGE_BYTES + ((i == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) ? (uint32_t)p.tx_extra : 0u));
+                    tma_load_3d(bdst, &map_b, bf, cx, k0, tap);
+                }
+                __syncwarp();
                 if (++b_stage == (uint32_t)p.b_stages) { b_stage = 0; b_par ^= 1u; bf = b_full; be = b_empty; bdst = smem_b; }
                 else { bf += 8; be += 8; bdst += Cfg::B_STAGE_BYTES; }
                 if (++tap == p.taps) { tap = 0; cx += 32; need_slab = true; }
@@ -401,7 +406,7 @@ tconv_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         }
     } else if (warp == 1 || warp == 6 || warp >= 11) {
         const int issuer = warp == 1 ? 0 : warp == 6 ? 1 : warp - 9;          // warps 1, 6, 11, 12
-        if (lane == 0 && issuer < Cfg::ISSUERS) {
+        if (issuer < Cfg::ISSUERS) {
             // ---------------- MMA issuers: each feeds its own share of the accumulators
             constexpr int ACC_PER = NACC / Cfg::ISSUERS;
             const int acc0 = issuer * ACC_PER;
@@ -421,7 +426,7 @@ tconv_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             uint32_t accumulate = 0;
             for (int i = 0; i < my_iters; ++i) {
                 if (new_slab) {
-                    ok = mbar_wait(a_full + 8 * a_slot, a_par, &s_abort, p.status, 13);
+                    ok = warp_wait(a_full + 8 * a_slot, a_par, &s_abort, p.status, 13);
                     if (!ok) break;
                     slab_addr = smem_a + a_slot * p.a_slot_bytes;
                     cur_slot = a_slot;
@@ -429,25 +434,28 @@ tconv_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     if (a_slot == 0) a_par ^= 1u;
                     new_slab = false;
                 }
-                ok = mbar_wait(bf, b_par, &s_abort, p.status, 14);
+                ok = warp_wait(bf, b_par, &s_abort, p.status, 14);
                 if (!ok) break;
                 tc_fence_after();
                 // The A tile of tap (r, s) starts (r*Wp + s) rows into the slab.  The start address may sit on any
                 // 128-byte row: the hardware derives every row's swizzle phase from its shared-memory address bits,
                 // exactly as the TMA write did (measured: the descriptor's base-offset field must stay zero).
                 const uint64_t da = smem_desc_k_sw128(slab_addr + a_off);
-#pragma unroll
-                for (int a = 0; a < ACC_PER; ++a) {
-                    const int acc = acc0 + a;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        umma_tf32(tmem_acc + acc * BN, da + (uint64_t)(acc * (128 * 128 / 16) + 2 * k), db + 2 * k, idesc,
-                                  (k == 0) ? accumulate : 1u);
-                }
-                accumulate = 1u;
-                tc_commit(be);
                 const bool chunk_done = (tap + 1 == p.taps);
-                if (chunk_done || i + 1 == my_iters) tc_commit(a_empty + 8 * cur_slot);
+                if (elect_one()) {
+#pragma unroll
+                    for (int a = 0; a < ACC_PER; ++a) {
+                        const int acc = acc0 + a;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            umma_tf32(tmem_acc + acc * BN, da + (uint64_t)(acc * (128 * 128 / 16) + 2 * k), db + 2 * k, idesc,
+                                      (k == 0) ? accumulate : 1u);
+                    }
+                    tc_commit(be);
+                    if (chunk_done || i + 1 == my_iters) tc_commit(a_empty + 8 * cur_slot);
+                }
+                __syncwarp();
+                accumulate = 1u;
                 if (++b_stage == (uint32_t)p.b_stages) { b_stage = 0; b_par ^= 1u; bf = b_full; be = b_empty; db = db0; }
                 else { bf += 8; be += 8; db += (uint64_t)(Cfg::B_STAGE_BYTES >> 4); }
                 if (chunk_done) { tap = 0; s = 0; a_row_off = 0; a_off = 0; new_slab = true; }
@@ -456,7 +464,8 @@ tconv_halo_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                     if (++s == p.S) { s = 0; a_row_off += wp_bytes; a_off = a_row_off; } else a_off += 128u;
                 }
             }
-            tc_commit(accum_bar);
+            if (elect_one()) tc_commit(accum_bar);
+            __syncwarp();
             if (!ok) (void)mbar_wait(accum_bar, 0, &s_abort, p.status, 15);
         }
     } else {

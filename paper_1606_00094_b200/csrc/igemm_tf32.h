@@ -10,8 +10,8 @@ struct IgemmPlan;
 bool igemm_variant_legal(const ConvDims& d, int variant);
 // Rule used by automatic selection: is the tensor-core path expected to beat DIRECT for this shape?
 bool igemm_variant_profitable(const ConvDims& d);
-// What the rule's tile costs in the TF32 mode (estimated SM clocks, staging of the input included) and what its kernel reads: a staged copy,
-// NCHW gathered by warps, or NCHW by TMA.  Allocates nothing.
+// What the tensor-core kernels cost in the TF32 mode as the line between FP32 and TF32 layers counts (estimated SM clocks, staging of the input
+// included), and what the kernel meant reads: a staged copy, NCHW gathered by warps, or NCHW by TMA.  Allocates nothing.
 enum IgemmKind { IGEMM_STAGES = 0, IGEMM_GATHERS = 1, IGEMM_READS_NCHW = 2 };
 double igemm_rule_cost(const ConvDims& d, int variant, size_t max_ws, IgemmKind* kind);
 int igemm_num_tiles();
@@ -21,9 +21,10 @@ int igemm_split_candidate(int i);
 // s2d: -1 automatic, 0 never, 1 force the space-to-depth view of a strided tconv layer.
 // mode: 0 TF32; 1 error-compensated TF32 (three tensor-core products per FP32 product); 2 fp16 operands (fp32
 // accumulate).  Modes 1 and 2: im2col kernel only, NCHW in and out.
-// max_ws: 0, or the largest workspace (staged input) the caller accepts; BODA_ERR_NOMEM if no tile fits it.
+// max_ws: 0, or the largest workspace (staged input) the caller accepts; BODA_ERR_NOMEM if no tile fits it.  in_chain: kernels that read NCHW only
+// are not chosen by rule where they would part the layer from its neighbours' staged layouts.
 int igemm_plan_create(const ConvDims& d, int variant, int tile_id, int split_k, int s2d, int* d_status, IgemmPlan** out,
-                      int mode = 0, size_t max_ws = 0);
+                      int mode = 0, size_t max_ws = 0, bool in_chain = false);
 bool igemm_s2d_applicable(const ConvDims& d);
 void igemm_plan_destroy(IgemmPlan* p);
 int igemm_plan_tile(const IgemmPlan* p);
@@ -46,6 +47,8 @@ int igemm_launch(IgemmPlan* p, const float* in, const float* filt, const float* 
 // best split, staging of both operands included (`clocks`: by a second model), and the workspace they need.
 bool igemm_split_legal(const ConvDims& d);
 double igemm_split_cost(const ConvDims& d, int tile, double* clocks);
+// the fastest of them for FP32 layers, wherever those run on split operands at all
+int igemm_split_tile(const ConvDims& d);
 size_t igemm_split_workspace(const ConvDims& d);
 // the most that automatic selection and the tuner let these tiles take where the caller sets no limit
 size_t igemm_split_workspace_limit(const ConvDims& d);

@@ -1,0 +1,86 @@
+"""Stride-1 windows straight from NCHW (tiles 35..46) at the edges where they can go wrong: one chunk of channels and a last one that is mostly padding,
+slabs of one row group and of the most rows that fit, windows without padding and wider than they are high, one and two issuing warps, tiles in several
+rounds, splits, tiles that end in the padding between images.  Integer operands: exact in any order, TF32 and fp16 alike."""
+import os
+
+import numpy as np
+import pytest
+
+from helpers import TF32_TOL, assert_parity, oracle_out, run_planned
+from paper_1606_00094_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+F16 = 4
+# (N,C,H,W,K,R,S,stride,pad,relu)
+SHAPES = [
+    (1, 3, 9, 11, 17, 3, 3, 1, 0, 1),            # one chunk of one MMA step, no padding
+    (2, 70, 13, 13, 130, 3, 3, 1, 1, 0),         # a last chunk of six channels, images that end inside a tile
+    (3, 33, 7, 9, 40, 2, 3, 1, 1, 1),            # R != S, one channel past a chunk
+    (1, 40, 20, 60, 33, 7, 7, 1, 3, 1),          # slabs of 512 rows, one tap a stage
+    (2, 96, 27, 27, 256, 5, 5, 1, 2, 1),         # three chunks: the sets of builders change places from tile to tile
+    (31, 64, 24, 25, 90, 3, 3, 1, 1, 1),         # 159 tiles of positions: the second round of a persistent CTA
+]
+
+
+def _ints(shape, seed):
+    N, C, H, W, K, R, S, *_ = shape
+    return wl.integers(seed, (N, C, H, W)), wl.integers(seed + 1, (K, C, R, S)), wl.integers(seed + 2, (K,))
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("tile", [35, 38, 41, 44, 46])           # 32, 80, 128, 192 and 256 channels
+@pytest.mark.parametrize("math", [0, F16])
+@pytest.mark.parametrize("split", [1, 3])
+def test_slab_tiles_exact(shape, tile, math, split):
+    x, w, b = _ints(shape, 7100)
+    ref = oracle_out(shape, x, w, b)
+    for bind in (False, True):
+        got, desc = run_planned(shape, x, w, b, variant=2, math=math, tile_id=tile, split_k=split, bind=bind)
+        assert "slab_128x" in desc and "workspace=0" in desc
+        np.testing.assert_array_equal(got.astype(np.float64), ref, err_msg=desc)
+
+
+@pytest.mark.parametrize("shape", [(2, 8, 12, 12, 16, 3, 3, 2, 1, 1), (2, 8, 12, 12, 16, 3, 3, 1, 3, 1), (1, 8, 8, 140, 16, 7, 7, 1, 3, 1)])
+def test_what_the_slab_tiles_refuse(shape):
+    """Strides, padding that is no part of the window, slabs of more than 512 rows."""
+    from paper_1606_00094_b200 import binding as B
+    with pytest.raises(B.BodaError) as e:
+        B.ConvPlan(shape, variant=2, tile_id=38)
+    assert e.value.status == B.BODA_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("shape,slab", [((20, 256, 13, 13, 384, 3, 3, 1, 1, 1), True), ((128, 256, 13, 13, 384, 3, 3, 1, 1, 1), False),
+                                        ((20, 256, 13, 13, 384, 3, 3, 2, 1, 1), False)])
+def test_rule_takes_one_round_of_slabs(shape, slab):
+    from paper_1606_00094_b200 import binding as B
+    plan = B.ConvPlan(shape)
+    try:
+        assert ("slab_128x" in plan.describe()) == slab, plan.describe()
+    finally:
+        plan.close()
+
+
+@pytest.mark.parametrize("tile,split", [(36, 1), (39, 2), (46, 1)])
+def test_expired_wait_in_the_slab_kernel(tile, split):
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    shape = (3, 64, 13, 13, 200, 3, 3, 1, 1, 1)
+    N, C, H, W, K, R, S, *_ = shape
+    x, w, b = wl.half_normal(1, (N, C, H, W)), wl.normal(2, (K, C, R, S), 0, (2.0 / (C * R * S)) ** 0.5), wl.normal(3, (K,), 0, 0.01)
+    dx, dw, db = (torch.from_numpy(t).cuda() for t in (x, w, b))
+    assert B.boda_query_status() == 0
+    os.environ["BODA_TEST_TX_MISMATCH"] = "1"
+    os.environ["BODA_WAIT_LIMIT_CYCLES"] = "100000000"
+    try:
+        plan = B.ConvPlan(shape, variant=2, tile_id=tile, split_k=split)
+    finally:
+        del os.environ["BODA_TEST_TX_MISMATCH"]
+        del os.environ["BODA_WAIT_LIMIT_CYCLES"]
+    plan(dx, dw, db)
+    torch.cuda.synchronize()
+    assert B.boda_query_status() == B.BODA_ERR_DEVICE_TIMEOUT
+    assert B.boda_query_status() == 0
+    plan.close()
+    got, desc = run_planned(shape, x, w, b, variant=2, tile_id=tile, split_k=split)
+    assert_parity(got, oracle_out(shape, x, w, b), TF32_TOL, desc)

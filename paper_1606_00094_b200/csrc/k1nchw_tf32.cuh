@@ -16,8 +16,8 @@
 // past HW are zero-filled by TMA and never stored.  Needs HW % 4 == 0 (TMA strides are multiples of 16 bytes).
 // The kernel is persistent (at most one CTA per SM walks the tiles) with two accumulators in tensor memory, so that a
 // tile's epilogue runs under the next tile's main loop.
-// Roles (256 threads): warps 0 and 2 = input-tile producers (two boxes each), warp 3 = filter tile and byte count,
-// warp 1 = TMEM owner and MMA issue (warp-uniform), warps 4..7 = epilogue.  Waits are bounded as in the other kernels.
+// Roles (384 threads): warps 0 and 2 = input-tile producers (half of the boxes each), warp 3 = filter tile and byte count,
+// warp 1 = TMEM owner and MMA issue (warp-uniform), warps 4..11 = epilogue.  Waits are bounded as in the other kernels.
 #pragma once
 
 #include "tc_ptx.cuh"
@@ -28,12 +28,12 @@ namespace k1n {
 
 using namespace tc;
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 384;
 constexpr int A_STAGE_BYTES = 128 * 128;
 constexpr int A_BOX_BYTES = 32 * 128;
 
 struct K1nParams {
-    int HW, tiles_per_image;
+    int HW, points, tiles_per_image;      // output points per tile: 128, or 64 where that still is one round of tiles
     int tiles_n, tiles_total;    // tiles are numbered (image, point tile) * tiles_n + channel tile
     int cchunks;                 // ceil(C / 32)
     const float* bias;
@@ -97,7 +97,7 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     if (threadIdx.x == 0) {
         s_abort = 0;
         for (int s = 0; s < kStages; ++s) { mbar_init(full_bar + 8 * s, 1); mbar_init(empty_bar + 8 * s, 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(acc_full + 8 * s, 1); mbar_init(acc_empty + 8 * s, 4); }
+        for (int s = 0; s < 2; ++s) { mbar_init(acc_full + 8 * s, 1); mbar_init(acc_empty + 8 * s, 8); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_b);
@@ -118,7 +118,7 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         const int mt = tile / p.tiles_n;
         k0 = (tile - mt * p.tiles_n) * BN;
         n = mt / p.tiles_per_image;
-        hw0 = (mt - n * p.tiles_per_image) * 128;
+        hw0 = (mt - n * p.tiles_per_image) * p.points;
     };
     int n, hw0, k0;
     decode(0, n, hw0, k0);
@@ -126,20 +126,21 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 
     if (warp == 0 || warp == 2) {
         {
-            // ---------------- input tiles: boxes of 32 output points x 32 channels; warp 0 loads points 0..63, warp 2 points 64..127
-            const int half = warp == 0 ? 0 : 2;
+            // ---------------- input tiles: boxes of 32 output points x 32 channels, the first half of them by warp 0, the second by warp 2.  Boxes
+            // that lie past the image are not loaded: a row of the accumulator depends on its own point only, and theirs are not stored.
+            const int half = p.points >> 6, first = warp == 0 ? 0 : half, end = first + half;
             uint32_t stage = 0, par = 1;
             bool ok = true;
             for (int t = 0; t < my_tiles && ok; ++t) {
                 if (t > 0) decode(t, n, hw0, k0);
+                const int live = min(end, (p.HW - hw0 + 31) >> 5);
                 for (int i = 0; i < steps; ++i) {
                     ok = warp_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 41);
                     if (!ok) break;
-                    const uint32_t dst = smem_a + stage * A_STAGE_BYTES + (uint32_t)half * A_BOX_BYTES;
-                    if (elect_one()) {
-                        tma_load_3d(dst, &map_a, full_bar + 8 * stage, hw0 + 32 * half, 32 * (i_begin + i), n);
-                        tma_load_3d(dst + A_BOX_BYTES, &map_a, full_bar + 8 * stage, hw0 + 32 * half + 32, 32 * (i_begin + i), n);
-                    }
+                    const uint32_t dst = smem_a + stage * A_STAGE_BYTES;
+                    if (elect_one())
+                        for (int b = first; b < live; ++b) tma_load_3d(dst + (uint32_t)b * A_BOX_BYTES, &map_a, full_bar + 8 * stage, hw0 + 32 * b, 32 * (i_begin + i), n);
+                    __syncwarp();
                     if (++stage == (uint32_t)kStages) { stage = 0; par ^= 1u; }
                 }
             }
@@ -148,18 +149,19 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         {
             // ---------------- filter tiles and the stage's byte count
             uint32_t stage = 0, par = 1;
-            uint32_t bytes = C::STAGE_BYTES + (blockIdx.x == 0 ? (uint32_t)p.tx_extra : 0u);
+            uint32_t extra = blockIdx.x == 0 ? (uint32_t)p.tx_extra : 0u;
             bool ok = true;
             for (int t = 0; t < my_tiles && ok; ++t) {
                 if (t > 0) decode(t, n, hw0, k0);
+                const uint32_t bytes = C::B_STAGE_BYTES + A_BOX_BYTES * (uint32_t)min(p.points >> 5, (p.HW - hw0 + 31) >> 5);
                 for (int i = 0; i < steps; ++i) {
                     ok = warp_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 42);
                     if (!ok) break;
                     if (elect_one()) {
-                        mbar_expect_tx(full_bar + 8 * stage, bytes);
+                        mbar_expect_tx(full_bar + 8 * stage, bytes + extra);
                         tma_load_3d(smem_b + stage * C::B_STAGE_BYTES, &map_b, full_bar + 8 * stage, 32 * (i_begin + i), k0, 0);
                     }
-                    bytes = C::STAGE_BYTES;
+                    extra = 0;
                     if (++stage == (uint32_t)kStages) { stage = 0; par ^= 1u; }
                 }
             }
@@ -203,30 +205,31 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             }
         }
     } else {
-        // ---------------- epilogue: warps 4..7, warp w reads TMEM lanes 32*(w%4) .. +31 = output points hw0 + that
-        const int quarter = warp & 3;
+        // ---------------- epilogue: warps 4..7 take the even 32-channel pieces of the accumulator, warps 8..11 the odd ones; warp w reads TMEM lanes
+        // 32*(w%4) .. +31 = output points hw0 + that
+        const int quarter = warp & 3, group = warp >= 8 ? 1 : 0;
         const int row = quarter * 32 + lane;
         for (int t = 0; t < my_tiles; ++t) {
             if (t > 0) decode(t, n, hw0, k0);
             const uint32_t slot = (uint32_t)t & 1u;
-            if (t > 0) asm volatile("bar.sync 1, 128;" ::: "memory");          // the previous tile's bias reads are over
-            for (int j = (int)threadIdx.x - 128; j < BN; j += 128)
+            if (t > 0) asm volatile("bar.sync 1, 256;" ::: "memory");          // the previous tile's bias reads are over
+            for (int j = (int)threadIdx.x - 128; j < BN; j += 256)
                 s_bias[j] = (p.bias && k0 + j < p.o.K) ? __ldg(p.bias + k0 + j) : 0.f;
             if (lane == 0) (void)mbar_wait_relaxed(acc_full + 8 * slot, (uint32_t)(t >> 1) & 1u, &s_abort, p.status, 45);
             __syncwarp();
             uint32_t stop;
-            asm volatile("{\n\t.reg .pred q, r;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.or.pred r, 1, 128, q;\n\tselp.u32 %0, 1, 0, r;\n\t}"
+            asm volatile("{\n\t.reg .pred q, r;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.or.pred r, 1, 256, q;\n\tselp.u32 %0, 1, 0, r;\n\t}"
                          : "=r"(stop) : "r"((uint32_t)s_abort) : "memory");
             if (stop) break;
             tc_fence_after();
             const uint32_t trow = tmem_acc + ((uint32_t)(quarter * 32) << 16) + slot * (uint32_t)BN;
             const int hw = hw0 + row;
-            const RowDst d = row_dst(p.o, hw < p.HW, n, 0, hw);
+            const RowDst d = row_dst(p.o, hw < p.HW && row < p.points, n, 0, hw);
             if (p.splits > 1) {
                 // split reduction, step 1: park the partial accumulator in this CTA's shared memory (the stages are idle:
                 // a split CTA has one tile); the cluster-wide sum follows after the role branches
 #pragma unroll 1
-                for (int c = 0; c < BN / 32; ++c) {
+                for (int c = group; c < BN / 32; c += 2) {
                     uint32_t v[32];
                     tmem_ld_32cols(trow + 32 * c, v);
                     tmem_ld_wait();
@@ -234,14 +237,16 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 }
                 break;
             }
+            if (quarter * 32 < p.points) {
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
-                uint32_t v[32];
-                tmem_ld_32cols(trow + 32 * c, v);
-                tmem_ld_wait();
-                float y[32];
-                bias_relu32(v, s_bias + 32 * c, p.o.relu != 0, y);
-                store_row32(p.o, d, k0 + 32 * c, y);
+                for (int c = group; c < BN / 32; c += 2) {
+                    uint32_t v[32];
+                    tmem_ld_32cols(trow + 32 * c, v);
+                    tmem_ld_wait();
+                    float y[32];
+                    bias_relu32(v, s_bias + 32 * c, p.o.relu != 0, y);
+                    store_row32(p.o, d, k0 + 32 * c, y);
+                }
             }
             // the accumulator has been read: hand the slot back to the issuer
             tc_fence_before();
@@ -255,10 +260,10 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         // step 2: every CTA of the cluster sums its share of the channels over all peers' parked accumulators in rank
         // order (the result does not depend on which CTA sums), adds the bias, applies ReLU and stores
         cluster_sync_all();
-        if (warp >= 4 && s_abort == 0) {
+        if (warp >= 4 && warp < 8 && s_abort == 0) {
             const int row = (warp & 3) * 32 + lane;
             const int hw = hw0 + row;
-            cluster_reduce_store<BN>(smem_base, row, cluster_cta_rank(), p.splits, row_dst(p.o, hw < p.HW, n, 0, hw), p.o, k0, s_bias);
+            cluster_reduce_store<BN>(smem_base, row, cluster_cta_rank(), p.splits, row_dst(p.o, hw < p.HW && row < p.points, n, 0, hw), p.o, k0, s_bias);
         }
         cluster_sync_all();          // nobody leaves while a peer may still read its shared memory
     }

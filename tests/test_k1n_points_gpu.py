@@ -1,0 +1,23 @@
+"""1x1 layers from NCHW in tiles of 64 and of 128 output points: images that end in any of a tile's boxes (those past the image are not loaded), one
+round of tiles and several."""
+import numpy as np
+import pytest
+
+from helpers import oracle_out, run_planned
+from paper_1606_00094_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("points,shape", [
+    (64, (2, 40, 2, 2, 50, 1, 1, 1, 0, 1)), (64, (2, 40, 6, 6, 50, 1, 1, 1, 0, 0)), (64, (1, 70, 10, 10, 130, 1, 1, 1, 0, 1)),
+    (128, (160, 40, 2, 2, 50, 1, 1, 1, 0, 1)), (128, (150, 40, 6, 6, 50, 1, 1, 1, 0, 0)), (128, (90, 70, 10, 10, 60, 1, 1, 1, 0, 1)),
+    (128, (150, 33, 14, 14, 70, 1, 1, 1, 0, 1)),
+])
+@pytest.mark.parametrize("tile", [20, 21])
+def test_tiles_of_64_and_128_points_exact(points, shape, tile):
+    N, C, H, W, K, *_ = shape
+    x, w, b = wl.integers(5, (N, C, H, W)), wl.integers(6, (K, C, 1, 1)), wl.integers(7, (K,))
+    got, desc = run_planned(shape, x, w, b, variant=1, tile_id=tile, split_k=1)
+    assert f"points={points}" in desc, desc
+    np.testing.assert_array_equal(got.astype(np.float64), oracle_out(shape, x, w, b), err_msg=desc)

@@ -116,7 +116,7 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     auto decode = [&](int t, int& n, int& hw0, int& k0) {
         const int tile = (int)blockIdx.x + t * (int)gridDim.x;
         const int mt = tile / p.tiles_n;
-        k0 = (tile - mt * p.tiles_n) * BN;
+        k0 = channel_tile(tile, t, p.tiles_n) * BN;
         n = mt / p.tiles_per_image;
         hw0 = (mt - n * p.tiles_per_image) * p.points;
     };

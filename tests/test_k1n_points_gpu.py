@@ -21,3 +21,15 @@ def test_tiles_of_64_and_128_points_exact(points, shape, tile):
     got, desc = run_planned(shape, x, w, b, variant=1, tile_id=tile, split_k=1)
     assert f"points={points}" in desc, desc
     np.testing.assert_array_equal(got.astype(np.float64), oracle_out(shape, x, w, b), err_msg=desc)
+
+
+# channel tiles that take turns with the CTAs (the grid of 148 is a multiple of 2 and 4, not of 3), the last of them ragged
+@pytest.mark.parametrize("tile,shape", [
+    (21, (160, 32, 6, 6, 139, 1, 1, 1, 0, 1)), (20, (90, 32, 6, 6, 196, 1, 1, 1, 0, 1)), (20, (160, 32, 6, 6, 139, 1, 1, 1, 0, 0)),
+    (18, (240, 33, 7, 7, 139, 1, 1, 1, 0, 1)), (16, (160, 33, 7, 7, 230, 1, 1, 1, 0, 1)), (16, (160, 33, 7, 7, 139, 1, 1, 1, 0, 0)),
+])
+def test_channel_tiles_in_turn_exact(tile, shape):
+    N, C, H, W, K, *_ = shape
+    x, w, b = wl.integers(5, (N, C, H, W)), wl.integers(6, (K, C, 1, 1)), wl.integers(7, (K,))
+    got, desc = run_planned(shape, x, w, b, variant=1, tile_id=tile, split_k=1)
+    np.testing.assert_array_equal(got.astype(np.float64), oracle_out(shape, x, w, b), err_msg=desc)

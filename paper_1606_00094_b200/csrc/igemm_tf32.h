@@ -20,11 +20,11 @@ int igemm_split_candidate(int i);
 
 // s2d: -1 automatic, 0 never, 1 force the space-to-depth view of a strided tconv layer.
 // mode: 0 TF32; 1 error-compensated TF32 (three tensor-core products per FP32 product); 2 fp16 operands (fp32
-// accumulate).  Modes 1 and 2: im2col kernel only, NCHW in and out.
-// max_ws: 0, or the largest workspace (staged input) the caller accepts; BODA_ERR_NOMEM if no tile fits it.  in_chain: kernels that read NCHW only
+// accumulate).  Mode 1: split operands or the im2col kernel, mode 2: im2col, pair and slab kernels; NCHW in and out.
+// max_ws: 0, or the largest workspace (staged input) the caller accepts; BODA_ERR_NOMEM if no tile fits it.  use: in a chain, kernels that read NCHW only
 // are not chosen by rule where they would part the layer from its neighbours' staged layouts.
 int igemm_plan_create(const ConvDims& d, int variant, int tile_id, int split_k, int s2d, int* d_status, IgemmPlan** out,
-                      int mode = 0, size_t max_ws = 0, bool in_chain = false);
+                      int mode = 0, size_t max_ws = 0, PlanUse use = PLAN_ALONE);
 bool igemm_s2d_applicable(const ConvDims& d);
 void igemm_plan_destroy(IgemmPlan* p);
 int igemm_plan_tile(const IgemmPlan* p);

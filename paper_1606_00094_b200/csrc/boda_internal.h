@@ -1,5 +1,6 @@
 // Internal declarations shared by the translation units of the library (not part of the ABI).
 #pragma once
+#include <mutex>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -84,22 +85,29 @@ cudaError_t launch_kernel(Kernel kernel, dim3 grid, dim3 block, size_t smem, cud
 }
 
 // cudaFuncSetAttribute applies to the current device only: a kernel's dynamic shared-memory limit is raised once per
-// device and kernel (one static DeviceSmemLimit per kernel instantiation), not once per process.
-struct DeviceSmemLimit {
-    int granted[64];
-    explicit DeviceSmemLimit(int initial = 0) { for (int& v : granted) v = initial; }
+// device and kernel (one static DeviceSmemLimit per kernel instantiation), not once per process.  Plans of one instantiation may need different
+// sizes and be called from several threads: test, call and note are one step under a lock, so that the limit only ever rises.
+class DeviceSmemLimit {
+public:
+    explicit DeviceSmemLimit(int initial = 0) : initial_(initial) {}
     template <typename Kernel>
     cudaError_t ensure(Kernel kernel, size_t bytes)
     {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
-        const bool tracked = dev >= 0 && dev < 64;
-        if (tracked && (int)bytes <= granted[dev]) return cudaSuccess;
+        std::lock_guard<std::mutex> lock(mutex_);
+        if (granted_.size() <= (size_t)dev) granted_.resize((size_t)dev + 1, initial_);
+        if ((int)bytes <= granted_[dev]) return cudaSuccess;
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e == cudaSuccess && tracked) granted[dev] = (int)bytes;
+        if (e == cudaSuccess) granted_[dev] = (int)bytes;
         return e;
     }
+
+private:
+    const int initial_;
+    std::mutex mutex_;
+    std::vector<int> granted_;
 };
 
 #ifdef __CUDACC__

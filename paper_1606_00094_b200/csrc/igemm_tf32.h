@@ -53,6 +53,7 @@ size_t igemm_split_workspace(const ConvDims& d);
 // the most that automatic selection and the tuner let these tiles take where the caller sets no limit
 size_t igemm_split_workspace_limit(const ConvDims& d);
 bool igemm_tile_is_split(int tile);
+bool igemm_tile_is_slab(int tile);
 
 // Activation layouts for chained layers.  igemm_plan_input_geometry: the staged input layout this plan reads,
 // rows [(n*Hp + y)*Wp + x][Cp] (false if the plan cannot take a staged input).  igemm_plan_set_io: in_packed =

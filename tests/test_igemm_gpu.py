@@ -366,11 +366,11 @@ def test_tuned_choice_is_remembered_in_the_cache_file(tmp_path, monkeypatch):
         prefix = lines[0].split(":")[0]
         assert len(lines) == 1 and lines[0].startswith(prefix + ":2,64,12,12,96,3,3,1,1,")  # one entry, keyed by kernels, tile tables and shape
         revision, direct, tensor = (int(v) for v in prefix.removeprefix("t").split("."))
-        assert (revision, direct, tensor) == (6, 27, 35)                                   # a tile more, or a faster kernel: another key
+        assert (revision, direct, tensor) == (7, 27, 47)                                   # a tile more, or a faster kernel: another key
         assert second.describe() == first.describe()
         assert t_second < t_first                                                          # no candidates were timed again
         # an entry written for other tile tables is ignored, not misread
-        others = ["t5", f"t{revision - 1}.{direct}.{tensor}", f"t{revision}.{direct - 4}.{tensor}", f"t{revision}.{direct}.{tensor - 4}"]
+        others = ["t5", "t6.27.35", f"t{revision - 1}.{direct}.{tensor}", f"t{revision}.{direct - 4}.{tensor}", f"t{revision}.{direct}.{tensor - 12}"]
         cache.write_text("".join(lines[0].replace(prefix, o, 1) + "\n" for o in others))
         third = B.ConvPlan(shape, tune=1)
         third.close()

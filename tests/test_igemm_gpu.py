@@ -383,7 +383,7 @@ def test_workspace_limit_steers_the_plan():
     """opts.max_workspace: tiles whose staged input does not fit are not considered; automatic selection then lands on
     a kernel that stages nothing (or the FP32 kernel), a forced tile that needs more is refused with BODA_ERR_NOMEM."""
     from paper_1606_00094_b200 import binding as B
-    shape = (4, 64, 13, 13, 96, 3, 3, 1, 1, 1)
+    shape = (4, 256, 13, 13, 96, 3, 3, 2, 1, 1)               # stride 2, 2304 indices: neither slabs nor the gather kernel
     x, w, b = _real_tensors(shape, 3100)
     ref = oracle_out(shape, x, w, b)
     free = B.ConvPlan(shape)

@@ -61,17 +61,18 @@ def test_rule_takes_one_round_of_slabs(shape, slab):
         plan.close()
 
 
-# few tiles and several chunks: by rule with fp16 storage, and in one call (the float32 plan of such a layer takes workspace)
+# few tiles and several chunks: by rule with either storage, and in one call
 @pytest.mark.parametrize("shape", [(1, 70, 5, 6, 33, 3, 3, 1, 1, 1), (1, 118, 16, 17, 86, 3, 3, 1, 1, 0)])
-def test_few_tiles_with_fp16_storage_and_in_one_call(shape):
+def test_few_tiles_by_rule_and_in_one_call(shape):
     import torch
     from paper_1606_00094_b200 import binding as B
     N, C, H, W, K, R, S, stride, pad, relu = shape
     x, w, b = wl.integers(15, (N, C, H, W)), wl.integers(16, (K, C, R, S)), wl.integers(17, (K,))
     ref = oracle_out(shape, x, w, b)
-    got, desc = run_planned(shape, x, w, b, math=F16)
-    assert "slab_128x" in desc, desc
-    np.testing.assert_array_equal(got.astype(np.float64), ref, err_msg=desc)
+    for kw in (dict(math=F16), dict(variant=2)):
+        got, desc = run_planned(shape, x, w, b, **kw)
+        assert "slab_128x" in desc, desc
+        np.testing.assert_array_equal(got.astype(np.float64), ref, err_msg=desc)
     y = B.conv_fwd(*(torch.from_numpy(a).cuda() for a in (x, w, b)), stride=stride, pad=pad, relu=bool(relu))
     np.testing.assert_array_equal(y.cpu().numpy().astype(np.float64), ref)
 

@@ -81,6 +81,7 @@ gconv_tf32_kernel(const __grid_constant__ CUtensorMap map_b, const GconvParams p
 
     const int warp = uniform_warp_index();
     const int lane = threadIdx.x & 31;
+    const bool turns = channel_tiles_in_turn(p.tiles_n);
     const int my_tiles = ((int)blockIdx.x < p.tiles_total) ? (p.tiles_total - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int nchunks = p.nchunks;
 
@@ -115,7 +116,7 @@ gconv_tf32_kernel(const __grid_constant__ CUtensorMap map_b, const GconvParams p
             bool first = true;
             for (int t = 0; t < my_tiles; ++t) {
                 const int tile = (int)blockIdx.x + t * (int)gridDim.x;
-                const int k0 = channel_tile(tile, t, p.tiles_n) * BN;
+                const int k0 = channel_tile(tile, t, p.tiles_n, turns) * BN;
                 bool ok = true;
                 for (int j = 0; j < nchunks; ++j) {
                     ok = warp_wait(empty_bar + 8 * stage, par, &s_abort, p.status, 21);
@@ -169,7 +170,7 @@ gconv_tf32_kernel(const __grid_constant__ CUtensorMap map_b, const GconvParams p
         const uint32_t row_addr = smem_out + (uint32_t)row * out_tile_row_bytes<BN>();
         for (int t = 0; t < my_tiles; ++t) {
             const int tile = (int)blockIdx.x + t * (int)gridDim.x;
-            const int m0 = (tile / p.tiles_n) * 128, k0 = channel_tile(tile, t, p.tiles_n) * BN;
+            const int m0 = (tile / p.tiles_n) * 128, k0 = channel_tile(tile, t, p.tiles_n, turns) * BN;
             const uint32_t slot = (uint32_t)t & 1u;
             // bias of this tile's channels (the four warps share it; the named barrier below orders it)
             asm volatile("bar.sync 1, 128;" ::: "memory");          // the previous tile's bias reads are over

@@ -89,6 +89,7 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     const int warp = uniform_warp_index();
     const int lane = threadIdx.x & 31;
     // persistent: this CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...; tile = (image, point tile) * tiles_n + channel tile
+    const bool turns = channel_tiles_in_turn(p.tiles_n);
     const int my_tiles = ((int)blockIdx.x < p.tiles_total) ? (p.tiles_total - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     const int i_begin = p.splits > 1 ? (int)blockIdx.z * p.chunks_per_split : 0;
     const int steps = p.splits > 1 ? min(p.cchunks, i_begin + p.chunks_per_split) - i_begin : p.cchunks;
@@ -116,7 +117,7 @@ k1nchw_tf32_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     auto decode = [&](int t, int& n, int& hw0, int& k0) {
         const int tile = (int)blockIdx.x + t * (int)gridDim.x;
         const int mt = tile / p.tiles_n;
-        k0 = channel_tile(tile, t, p.tiles_n) * BN;
+        k0 = channel_tile(tile, t, p.tiles_n, turns) * BN;
         n = mt / p.tiles_per_image;
         hw0 = (mt - n * p.tiles_per_image) * p.points;
     };

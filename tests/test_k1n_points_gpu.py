@@ -33,3 +33,14 @@ def test_channel_tiles_in_turn_exact(tile, shape):
     x, w, b = wl.integers(5, (N, C, H, W)), wl.integers(6, (K, C, 1, 1)), wl.integers(7, (K,))
     got, desc = run_planned(shape, x, w, b, variant=1, tile_id=tile, split_k=1)
     np.testing.assert_array_equal(got.astype(np.float64), oracle_out(shape, x, w, b), err_msg=desc)
+
+
+@pytest.mark.parametrize("shape", [(6, 336, 56, 56, 22, 1, 1, 1, 0, 1), (23, 362, 28, 28, 20, 1, 1, 1, 0, 1)])
+def test_a_few_tiles_of_a_second_round_do_not_change_the_kernel(shape):
+    """150 and 161 tiles on 148 SMs."""
+    from paper_1606_00094_b200 import binding as B
+    plan = B.ConvPlan(shape)
+    try:
+        assert "k1nchw_128x64" in plan.describe(), plan.describe()
+    finally:
+        plan.close()

@@ -179,6 +179,7 @@ FIRST_SHAPES = [
     (2, 3, 61, 50, 24, 7, 5, 4, 0, 1),           # 2 x 2 block taps
     (5, 3, 35, 35, 16, 8, 8, 4, 0, 1),           # window a multiple of the stride; tiny output (7 x 7)
     (1, 3, 131, 259, 32, 11, 11, 4, 0, 1),       # wide rows
+    (2, 3, 110, 110, 32, 11, 11, 4, 0, 1),       # 128 channels: within 16 bytes of an SM's shared memory
 ]
 
 

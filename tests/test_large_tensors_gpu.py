@@ -72,6 +72,8 @@ CASES = [
     ((4096, 64, 64, 64, 64, 1, 1, 1, 0, 1), 1, 2, 0),         # the same through the staged path (4.3 GB workspace)
     ((4096, 64, 64, 64, 64, 1, 1, 1, 0, 1), 1, 19, 0),        # the gather kernel
     ((2048, 32, 128, 128, 32, 3, 3, 1, 1, 1), 2, -1, 0),      # 3x3 with padding, 1.07 G elements in and out
+    ((8191, 64, 64, 64, 16, 3, 3, 1, 1, 1), 2, 35, 0),        # slabs from 2^31 - 262144 input elements (8.6 GB): offsets are 32-bit numbers there
+    ((8191, 64, 64, 64, 16, 3, 3, 1, 1, 1), 2, 37, 4),        # the same with fp16 storage
     ((1024, 3, 256, 256, 16, 3, 3, 1, 1, 1), 0, -1, 1),       # FP32 kernel (run-time compiled where NVRTC is there): 1.07 G outputs
 ]
 

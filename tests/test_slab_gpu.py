@@ -41,6 +41,62 @@ def test_slab_tiles_exact(shape, tile, math, split):
         np.testing.assert_array_equal(got.astype(np.float64), ref, err_msg=desc)
 
 
+# Windows by how their taps come to lie in stages (one, two, three or five taps of a row each) and how many stages a chunk and a row have: one stage a
+# chunk is one issuing warp's, rows of one stage and of several wrap differently.  Several chunks, more tiles than SMs for the narrow tiles.
+WINDOWS = [(2, 2, 1), (4, 4, 2), (1, 3, 0), (1, 2, 0), (1, 4, 0), (2, 1, 0), (3, 1, 0), (6, 6, 2), (9, 9, 4), (2, 10, 1)]
+
+
+@pytest.mark.parametrize("R,S,pad", WINDOWS)
+@pytest.mark.parametrize("math", [0, F16])
+def test_windows_exact(R, S, pad, math):
+    shape = (20, 70 if math == 0 else 130, 12, 11, 200, R, S, 1, pad, 1)
+    x, w, b = _ints(shape, 7300)
+    ref = oracle_out(shape, x, w, b)
+    for tile in (35, 36, 37, 39, 40, 42, 43, 45):             # the widths that the shapes above leave out, and 32
+        for split in (1, 2):
+            got, desc = run_planned(shape, x, w, b, variant=2, math=math, tile_id=tile, split_k=split, bind=split == 1)
+            assert "slab_128x" in desc
+            np.testing.assert_array_equal(got.astype(np.float64), ref, err_msg=desc)
+
+
+@pytest.mark.parametrize("tile,split", [(36, 1), (39, 2), (46, 1)])
+@pytest.mark.parametrize("math", [0, F16])
+def test_infinities_and_nan_stay_where_they_are(tile, split, math):
+    """Positions that are computed and dropped, padding and the channels past the last one read as zeros beside them."""
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    shape = (3, 70, 9, 11, 50, 3, 3, 1, 1, 0)
+    x, w, _ = _ints(shape, 7400)
+    w[w == 0] = 1.0
+    for value, at in ((np.inf, (0, 69, 0, 0)), (-np.inf, (1, 0, 8, 10)), (np.nan, (2, 33, 4, 0))):
+        x[at] = value
+    dx, dw = torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda()
+    want = torch.nn.functional.conv2d(dx.double(), dw.double(), padding=1).float()
+    plan = B.ConvPlan(shape, variant=2, math=math, tile_id=tile, split_k=split)
+    got = plan(dx, dw, None)
+    plan.close()
+    assert 0 < int((~torch.isfinite(want)).sum()) < want.numel() // 10
+    assert torch.equal(torch.nan_to_num(got, nan=1e30), torch.nan_to_num(want, nan=1e30))
+
+
+def test_filters_bound_again_between_calls():
+    import torch
+    from paper_1606_00094_b200 import binding as B
+    shape = (20, 70, 13, 13, 130, 3, 3, 1, 1, 0)
+    x, w, b = (torch.from_numpy(t).cuda() for t in _ints(shape, 7500))
+    v = w.flip(0).contiguous()
+    plan = B.ConvPlan(shape, variant=2, tile_id=39)
+    refs = [torch.nn.functional.conv2d(x.double(), f.double(), b.double(), padding=1).float() for f in (w, v)]
+    for bound, given, ref in ((w, w, 0), (v, v, 1), (None, w, 0), (None, v, 1), (w, w, 0)):
+        if bound is not None:
+            plan.bind_filters(bound)
+        assert torch.equal(plan(x, given, b), refs[ref])
+    w.copy_(v)                                                # the bound filters' values, bound again
+    plan.bind_filters(w)
+    assert torch.equal(plan(x, w, b), refs[1])
+    plan.close()
+
+
 @pytest.mark.parametrize("shape", [(2, 8, 12, 12, 16, 3, 3, 2, 1, 1), (2, 8, 12, 12, 16, 3, 3, 1, 3, 1), (1, 8, 8, 140, 16, 7, 7, 1, 3, 1)])
 def test_what_the_slab_tiles_refuse(shape):
     """Strides, padding that is no part of the window, slabs of more than 512 rows."""

@@ -117,6 +117,17 @@ def test_rule_takes_one_round_of_slabs(shape, slab):
         plan.close()
 
 
+@pytest.mark.parametrize("shape", [(43, 191, 55, 57, 43, 3, 3, 1, 1, 1), (40, 163, 51, 52, 49, 3, 3, 1, 1, 1)])
+def test_rule_leaves_many_chunks_of_fp16_to_the_pairs(shape):
+    """Several rounds of narrow tiles: the slabs, twice the channels of a TF32 chunk each, take their builders longer than the tensor cores."""
+    from paper_1606_00094_b200 import binding as B
+    plan = B.ConvPlan(shape, math=F16)
+    try:
+        assert "pair_256x64" in plan.describe(), plan.describe()
+    finally:
+        plan.close()
+
+
 # few tiles and several chunks: by rule with either storage, and in one call
 @pytest.mark.parametrize("shape", [(1, 70, 5, 6, 33, 3, 3, 1, 1, 1), (1, 118, 16, 17, 86, 3, 3, 1, 1, 0)])
 def test_few_tiles_by_rule_and_in_one_call(shape):

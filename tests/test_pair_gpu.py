@@ -107,3 +107,13 @@ def test_rule_leaves_these_to_the_gather_kernel(shape):
         assert "gconv" in plan.describe()
     finally:
         plan.close()
+
+
+def test_rule_leaves_one_round_of_halo_tiles_alone():
+    """11x11 with stride 4: 139 halo tiles of 512 positions, where pairs would begin a fourth round."""
+    from paper_1606_00094_b200 import binding as B
+    plan = B.ConvPlan((35, 3, 171, 171, 32, 11, 11, 4, 5, 1))
+    try:
+        assert "halo_512x64" in plan.describe(), plan.describe()
+    finally:
+        plan.close()

@@ -595,11 +595,7 @@ int direct_pick_tile(const ConvDims& d, size_t max_ws)
     // batch 31 takes 363 us in place and 562 there, on 16 channels, 17 filters, 82x83, batch 22 47 and 70.  Of 774 layers 4 are then 16 to 60 % faster and
     // two slower (6 and 11 %).  Elsewhere the second model would be right no more often than the first.
     const bool padding = d.C <= 16 || d.K < 16;
-    if (split_cost >= best_cost || (padding && split_second > 1.05 * best_cost)) return best;
-    const int tile = igemm_split_tile(d);
-    for (int t = 0; t < kNumTiles; ++t)
-        if (kTiles[t].kind == TILE_SPLIT && kTiles[t].kt == tile) split = t;
-    return split;
+    return split_cost < best_cost && (!padding || split_second <= 1.05 * best_cost) ? split : best;
 }
 
 bool direct_tile_legal(const ConvDims& d, int tile_id)

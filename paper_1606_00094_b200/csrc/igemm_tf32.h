@@ -47,8 +47,6 @@ int igemm_launch(IgemmPlan* p, const float* in, const float* filt, const float* 
 // best split, staging of both operands included (`clocks`: by a second model), and the workspace they need.
 bool igemm_split_legal(const ConvDims& d);
 double igemm_split_cost(const ConvDims& d, int tile, double* clocks);
-// the fastest of them for FP32 layers, wherever those run on split operands at all
-int igemm_split_tile(const ConvDims& d);
 size_t igemm_split_workspace(const ConvDims& d);
 // the most that automatic selection and the tuner let these tiles take where the caller sets no limit
 size_t igemm_split_workspace_limit(const ConvDims& d);

@@ -74,3 +74,14 @@ def test_halo_and_space_to_depth_are_refused():
         B.ConvPlan((2, 64, 13, 13, 64, 3, 3, 1, 1, 1), math=X3, variant=TC, tile_id=5)      # a halo tile
     with pytest.raises(Exception):
         B.ConvPlan((1, 3, 227, 227, 96, 11, 11, 4, 0, 1), math=X3, variant=TC, s2d=1)
+
+
+@pytest.mark.parametrize("shape", [(3, 187, 34, 34, 140, 3, 3, 1, 1, 0), (6, 134, 48, 49, 162, 3, 3, 2, 1, 0)])
+def test_rule_does_not_lengthen_sums_for_speed(shape):
+    """Four-way splits: 1.6e-8 of the sum at each of the 84 and 60 MMAs that an accumulator takes there, and 22 bits of every operand (under 5e-7 over such
+    reductions) bound the error to 1.9e-6; two-way splits of narrower tiles, which are faster, are at 2.2e-6 and above."""
+    x, w, b = _real_tensors(shape, 1700)
+    from oracle import conv_oracle as orc
+    got, desc = run_planned(shape, x, w, b, variant=TC, math=X3)
+    err = orc.rel_l2(got, oracle_out(shape, x, w, b))
+    assert err < 1.9e-6, f"{desc}: {err:.2e}"

@@ -52,6 +52,9 @@ size_t igemm_split_workspace(const ConvDims& d);
 size_t igemm_split_workspace_limit(const ConvDims& d);
 bool igemm_tile_is_split(int tile);
 bool igemm_tile_is_slab(int tile);
+// Does a kernel other than the slab kernel (mode 0 or 2) run the layer under these options?  Slabs, which take no workspace, are no reason to run one that a limit
+// on it rules out.
+bool igemm_runs_without_slabs(const ConvDims& d, int variant, int split_k, int s2d, int mode, size_t max_ws);
 
 // Activation layouts for chained layers.  igemm_plan_input_geometry: the staged input layout this plan reads,
 // rows [(n*Hp + y)*Wp + x][Cp] (false if the plan cannot take a staged input).  igemm_plan_set_io: in_packed =

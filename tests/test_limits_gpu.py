@@ -32,6 +32,18 @@ def test_a_window_layer_under_a_tight_limit(shape, tune):
     assert e.value.status == B.BODA_ERR_NOMEM
 
 
+def test_a_remembered_choice_under_a_tight_limit(tmp_path, monkeypatch):
+    """A slab tile that tuning found without a limit is not taken from the file where the limit rules the others out."""
+    from paper_1606_00094_b200 import binding as B
+    monkeypatch.setenv("BODA_TUNE_CACHE", str(tmp_path / "tune.txt"))
+    shape = (1, 200, 16, 17, 86, 3, 3, 1, 1, 1)               # 1800 indices: no gather kernel
+    assert "slab_128x" in _plan(shape, variant=TC, tune=1)
+    assert "slab_128x" in _plan(shape, variant=TC, tune=1, max_workspace=1 << 20)
+    with pytest.raises(B.BodaError) as e:
+        B.ConvPlan(shape, variant=TC, max_workspace=1024, tune=1)
+    assert e.value.status == B.BODA_ERR_NOMEM
+
+
 @pytest.mark.parametrize("shape", WINDOWS)
 def test_the_same_with_fp16_storage(shape):
     from paper_1606_00094_b200 import binding as B

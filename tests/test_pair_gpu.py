@@ -99,6 +99,7 @@ def test_pair_tiles_on_a_space_to_depth_view_exact(shape, tile):
 
 
 @pytest.mark.parametrize("shape", [(14, 3, 150, 150, 48, 7, 7, 2, 0, 1), (33, 3, 215, 215, 48, 5, 5, 2, 2, 1),       # strided first layers
+                                   (18, 16, 34, 34, 106, 3, 3, 2, 1, 1),                                             # 16 channels, stride 2
                                    (227, 75, 13, 13, 356, 1, 1, 1, 0, 1)])                                           # three steps a tile
 def test_rule_leaves_these_to_the_gather_kernel(shape):
     from paper_1606_00094_b200 import binding as B

@@ -9,7 +9,7 @@ from paper_1606_00094_b200 import workloads as wl
 pytestmark = pytest.mark.gpu
 
 # (N,C,H,W,K,R,S,stride,pad,relu): points 127 / 128 / 129 per call, channels around 32 and 64, windows on both sides of the
-# largest that is staged through shared memory (36 taps; beyond, runs of 8 taps with and without a remainder), filter counts that leave a last block nearly empty
+# largest that is staged through shared memory (36 taps; beyond and at multiples of 8, runs of 8 taps with and without a remainder), filter counts that leave a last block nearly empty
 SHAPES = [
     (1, 31, 1, 127, 17, 1, 1, 1, 0, 0),
     (1, 33, 8, 16, 9, 1, 1, 1, 0, 1),
@@ -21,6 +21,8 @@ SHAPES = [
     (1, 35, 11, 11, 8, 11, 11, 1, 5, 0),
     (2, 33, 10, 12, 9, 4, 10, 1, 2, 0),
     (1, 40, 9, 12, 19, 9, 11, 1, 4, 1),
+    (2, 33, 10, 12, 9, 4, 4, 1, 1, 0),           # 16 and 32 taps: runs too
+    (1, 70, 9, 12, 19, 8, 4, 1, 2, 1),
 ]
 
 

@@ -3,7 +3,8 @@
 // Two CTAs of a cluster share one output tile of 256 points x BN channels: each stages its own 128 points and HALF of the tile's
 // filter rows, and one thread of the first CTA issues MMAs that read both CTAs' shared memory and write 128 rows into each
 // CTA's tensor memory.  A CTA therefore fetches 128 + BN/2 rows per reduction step instead of 128 + BN for the same MMA time.
-// That is what bounds the one-CTA kernel below BN = 256 (L2 feeds the SMs some 10 KB a clock in all), and why it needs wide tiles, i.e. few of them.
+// The fetch is what bounds the one-CTA kernel below BN = 192: with every SM busy a step of 128 channels takes it 297 clocks for 256 of MMAs (L2 gives it 16.3 KB a
+// clock in all, fitted; the pairs 13.7), a pair 265.
 // The pairs are persistent (at most one CTA per SM walks the tiles) with two accumulators in tensor memory: a tile's epilogue
 // and the pipeline's fill run under the next tile's main loop.
 // Measured, one-CTA kernel / pairs of the same width: 5x5 on 96 channels, 256 filters, 27x27, fp16, batch 128 (115 GFLOP) 130 / 105 us (BN = 256), 153 / 123

@@ -7,12 +7,12 @@
 // rows, the swizzled 16-byte stores meet no bank twice, and rounding costs nothing extra.
 // What that is for:
 //  * The staging launch in front of the im2col, halo and pair kernels, with its pass over the input, was 4 to 6 us of a layer.
-//  * The im2col kernels fetch every input row once per tap, and L2 feeds the SMs some 10 KB a clock in all.  A slab is filled once per chunk
-//    of channels, and what is left are the filters: BN rows a tap where they fetch 128 + BN.  Narrow tiles then cost little, so that a
+//  * The im2col kernels fetch every input row once per tap, and L2 gives them some 16 KB a clock in all (fitted, see model_cost).  A slab is filled once per
+//    chunk of channels, and what is left are the filters: BN rows a tap where they fetch 128 + BN.  Narrow tiles then cost little, so that a
 //    round of 148 CTAs fills without a split of the reduction over a cluster and its exchange.
 // The price: positions right of and below the image are computed and dropped (7 to 16 % of the rows for 13x13 and 27x27).
-// Measured: 3x3 on 256 channels, 384 filters, 13x13, batch 20 18.9 us (im2col 128x192, split) -> 15.9 (128x96); 5x5 on 96 channels, 256 filters, 27x27, batch 20 with fp16
-// operands 24.8 (pairs) -> 20.9 (128x256); 3x3 on 64 channels, 64 filters, 56x56, one image 6.4.
+// Measured, a call of a plan with its output allocated: 3x3 on 256 channels, 384 filters, 13x13, batch 20 19.1 us (im2col 128x192, split) -> 15.7 (128x96); 5x5 on
+// 96 channels, 256 filters, 27x27, batch 20 with fp16 operands 25.1 (pairs) -> 23.0 (128x256).
 //
 // The tile's width BN is a run-time value (a multiple of 16), chosen so that the tiles fill whole rounds of the SMs.  MMAs of 128 x BN x 32
 // bytes take max(BN/2, 32 + BN/4) clocks: below 128 channels the tensor core waits for its operands from shared memory.  A stage of
@@ -48,7 +48,8 @@ constexpr int kMaxBN = 256;
 constexpr int kBarrierBytes = 512;
 constexpr int kSmemBudget = 222 * 1024;
 
-// Division of numbers below 2^31: multiply by ceil(2^(31 + l) / d), l = ceil(log2 d), and shift.
+// Division of numbers below 2^31 (Granlund and Montgomery, Division by Invariant Integers using Multiplication, 1994): multiply by ceil(2^(31 + l) / d),
+// l = ceil(log2 d), and shift.
 struct FastDiv {
     unsigned mul, shift;
     static FastDiv of(unsigned d)
